@@ -11,11 +11,12 @@
 //   layer:    one thread per site, the nine offsets unrolled; weights staged in shared memory.
 //             The adjoint layer L^dag = sum_d A_d^dag T_{-d} is the same kernel with the offsets
 //             reversed and the weights conjugate-transposed.
-//   gradient: dloss/dA_{l,d} = 2 sum_{x, colour} g_l(x) (T_d psi_{l-1})(x)^dag, per-thread sums
-//             over a grid-stride range of sites, a fixed-order block tree in FP64 and a one-block
-//             final sum over the blocks (deterministic).
+//   gradient: dloss/dA_{l,d} = 2 sum_{x, colour} g_l(x) (T_d psi_{l-1})(x)^dag: one warp per offset,
+//             FP32 sums over a few sites, FP64 sums over lanes, blocks and pairs in a fixed order
+//             (deterministic).
 //   loss:     |P b - x|^2 / |x|^2 per pair with the seed g_K = (P b - x) / |x|^2.
-//   Adam:     on the real and imaginary parts of every A entry.
+//   Adam:     on the real and imaginary parts of every A entry, in the gradient's final sum.
+// A training step runs every kernel once for a group of its pairs, not once per pair.
 #include "ok_net.cuh"
 #include "ok_pair.cuh"
 
@@ -29,15 +30,17 @@ struct ok_net {
   float* m = nullptr;       // Adam moments, [layers * 288]
   float* v = nullptr;
   double* gacc = nullptr;   // gradient accumulator [layers * 288]
-  double* scal = nullptr;   // [0..1] loss sums of the current pair, [2] loss accumulator
-  unsigned* ticket = nullptr;
+  double* scal = nullptr;   // [0] loss accumulator, [2 + 2 q, 3 + 2 q] |x|^2 and |P b - x|^2 of pair q of a group
+  unsigned* ticket = nullptr;  // [MAX_GROUP]
   long long adam_t = 0;
   int V = 0;                // volume the workspace is sized for
   int device = 0;
-  okgb::cx<float>* acts = nullptr;  // [layers][V * 12], training only
-  okgb::cx<float>* g[2] = {nullptr, nullptr};
-  double* part = nullptr;     // [blocks][9][32]
-  int part_blocks = 0;
+  okgb::cx<float>* g[2] = {nullptr, nullptr};  // layer ping-pong of an application, [V * 12]
+  int group = 0;            // pairs the training workspace holds (0: none yet)
+  okgb::cx<float>* acts = nullptr;  // [layers][group][V * 12]
+  okgb::cx<float>* tg[2] = {nullptr, nullptr};  // backward gradients, [group][V * 12]
+  double* part = nullptr;   // gradient partials [layers][blocks][9][32]
+  double* lpart = nullptr;  // loss partials [group][2 * loss blocks]
 };
 
 namespace okgb {
@@ -47,6 +50,7 @@ namespace {
 constexpr int NET_THREADS = 128;
 constexpr int NOFF = 9;
 constexpr int NPAR = NOFF * 32;  // real parameters per layer
+constexpr int MAX_GROUP = 64;    // pairs of a batch that go through the kernels together
 
 // (direction, step) of offset d; direction -1 is the on-site term.
 __host__ __device__ constexpr int off_mu(int d) { return d == 0 ? -1 : (d - 1) / 2; }
@@ -180,124 +184,259 @@ __global__ void __launch_bounds__(NET_THREADS) net_layer_kernel(const cx<float>*
   }
 }
 
-// Per block: for every offset d, sum over this block's sites of g(x)_s,c conj((T_d in)(x)_t,c)
-// (16 complex = 32 values) -> part[block][d][32] in FP64.
-__global__ void __launch_bounds__(NET_THREADS) net_grad_kernel(const cx<float>* __restrict__ L, const cx<float>* __restrict__ gr,
-                                                               const cx<float>* __restrict__ in, Geom g,
-                                                               double* __restrict__ part) {
-  __shared__ double sh[NET_THREADS / 32][32];
-  for (int d = 0; d < NOFF; ++d) {
+// Gradient partials: part[block][d][32] = sum over the block's (pair, 32-site tile)s of
+// g(x)_s,c conj((T_d in)(x)_t,c) (16 complex = 32 values).  A block has one warp per offset d, so a
+// warp keeps one offset's 32 sums over all its sites and needs one lane reduction for every
+// GRAD_CHUNK sites of a thread.  (One warp walking all nine offsets took nine five-step FP64 trees
+// of 32 values for one or two sites a thread: the FP64 pipe, 1/58 of the FP32 rate, was 76 % busy
+// and the kernel took 289 us at 16^3 x 32; this form takes 45 us.)  The lane reduction
+// transposes as it sums: each step adds the half of the values that a lane keeps to the same half of
+// its partner's, 31 FP64 additions for the 32 values instead of 160, and leaves value k in lane k.
+// The nine warps read the same tile's g and neighbours back to back, so L1 shares them.
+constexpr int GRAD_WARPS = NOFF;
+constexpr int GRAD_THREADS = 32 * GRAD_WARPS;
+constexpr int GRAD_CHUNK = 8;
+__global__ void __launch_bounds__(GRAD_THREADS, 2) net_grad_kernel(const cx<float>* __restrict__ L, const cx<float>* __restrict__ gr,
+                                                                   const cx<float>* __restrict__ in, Geom g, int pairs,
+                                                                   double* __restrict__ part, bool accumulate) {
+  const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
+  const int ntiles = (g.V + 31) / 32;
+  const long long work = (long long)ntiles * pairs;
+  double tot = 0.0;
+  for (long long w0 = blockIdx.x; w0 < work; w0 += (long long)gridDim.x * GRAD_CHUNK) {
     float C[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) C[k] = 0.f;
-    for (int x = blockIdx.x * NET_THREADS + threadIdx.x; x < g.V; x += gridDim.x * NET_THREADS) {
+#pragma unroll 1
+    for (int u = 0; u < GRAD_CHUNK; ++u) {
+      const long long w = w0 + (long long)u * gridDim.x;
+      if (w >= work) break;
+      const int q = (int)(w / ntiles), x = (int)(w % ntiles) * 32 + lane;
+      if (x >= g.V) continue;
+      const size_t off = (size_t)q * 12 * g.V;
       int c[4];
       site_coords(x, g, c);
-      cx<float> gv[4][3], w[4][3];
-      load_sp(gr, x, gv);
-      transported<false>(L, in, x, c, g, d, w);
+      cx<float> gv[4][3], wv[4][3];
+      load_sp(gr + off, x, gv);
+      transported<false>(L, in + off, x, c, g, d, wv);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           cx<float> z = mk<float>(C[2 * (4 * s + t)], C[2 * (4 * s + t) + 1]);
 #pragma unroll
-          for (int a = 0; a < 3; ++a) z = fma_cj(w[t][a], gv[s][a], z);  // g conj(w)
+          for (int a = 0; a < 3; ++a) z = fma_cj(wv[t][a], gv[s][a], z);  // g conj(w)
           C[2 * (4 * s + t)] = z.re;
           C[2 * (4 * s + t) + 1] = z.im;
         }
     }
-    // fixed-order block tree: warp shuffles, then the warps in order
+    // transposing lane reduction: after the step of width o, value index bits >= o are the lane's
+    double v[16];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      double v = C[k];
+    for (int k = 0; k < 16; ++k) {
+      const bool up = lane & 16;
+      const float keep = up ? C[k + 16] : C[k], send = up ? C[k] : C[k + 16];
+      v[k] = (double)keep + (double)__shfl_xor_sync(0xffffffffu, send, 16);
+    }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      double v = 0.0;
-      for (int w = 0; w < NET_THREADS / 32; ++w) v += sh[w][threadIdx.x];
-      part[((size_t)blockIdx.x * NOFF + d) * 32 + threadIdx.x] = v;
-    }
-    __syncthreads();
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const bool up = lane & o;
+        const double keep = up ? v[k + o] : v[k], send = up ? v[k] : v[k + o];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    tot += v[0];
   }
+  double* p = part + (size_t)blockIdx.x * NPAR + threadIdx.x;
+  *p = accumulate ? *p + tot : tot;
 }
 
-// gacc[i] += 2 sum_b part[b][i] (one block, blocks in order).
-__global__ void net_grad_final_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ gacc) {
-  for (int i = threadIdx.x; i < NPAR; i += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * NPAR + i];
-    gacc[i] += 2.0 * s;
-  }
+// Adam's arguments; P null: no update.
+struct AdamArgs {
+  float *P, *m, *v;
+  double scale;
+  float lr, b1, b2, eps, c1, c2;
+};
+
+// One block per (layer, offset): gacc = 2 sum over the blocks' partials (eight slices of blocks,
+// then the slices in order), and one Adam step on those 32 parameters.  (One block per layer
+// summing 608 partials in sequence took 60 us per pair and layer; all layers of a step now take 14 us.)
+__global__ void __launch_bounds__(256) net_grad_final_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ gacc,
+                                                             AdamArgs ad) {
+  __shared__ double sh[8][32];
+  const int l = blockIdx.x / NOFF, d = blockIdx.x % NOFF;
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const double* p = part + (size_t)l * nblocks * NPAR + d * 32 + lane;
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = slice; b < nblocks; b += 8) s += p[(size_t)b * NPAR];
+  sh[slice][lane] = s;
+  __syncthreads();
+  if (slice) return;
+  for (int k = 1; k < 8; ++k) s += sh[k][lane];
+  const int i = l * NPAR + d * 32 + lane;
+  const double gsum = 2.0 * s;
+  gacc[i] = gsum;
+  if (!ad.P) return;
+  const float gr = (float)(gsum * ad.scale);
+  const float m = ad.b1 * ad.m[i] + (1.f - ad.b1) * gr, v = ad.b2 * ad.v[i] + (1.f - ad.b2) * gr * gr;
+  ad.m[i] = m;
+  ad.v[i] = v;
+  ad.P[i] -= ad.lr * (m / ad.c1) / (sqrtf(v / ad.c2) + ad.eps);
 }
 
-// |x|^2 and |out - x|^2 -> scal[0], scal[1]
+// |x|^2 and |out - x|^2 of pair blockIdx.y -> scal[2 + 2 pair], scal[3 + 2 pair].  The squares of a
+// chunk of LOSS_CHUNK complex numbers are summed as double-float pairs on the FP32 pipes (about 48
+// bits) when the chunk's largest component lies in [2^-40, 2^40], where neither the squares nor
+// their rounding errors leave FP32's range, and in FP64 otherwise; chunks are added in FP64.  (In
+// FP64 throughout, the FP64 pipe was 82 % busy: 51 us for 25 MB at 16^3 x 32, now 13 us a pair.)
+constexpr int LOSS_CHUNK = 8;
+__device__ __forceinline__ dd dd_sq(dd a) {
+  const float p = a.hi * a.hi;
+  const float e = fmaf(a.hi, a.hi, -p);
+  return dd_renorm(p, fmaf(2.f * a.hi, a.lo, e));
+}
+__device__ __forceinline__ dd dd_diff(float a, float b) {
+  const float s = a - b, bb = s - a;
+  return dd(s, (a - (s - bb)) - (b + bb));
+}
 __global__ void __launch_bounds__(256) net_loss_kernel(const float2* __restrict__ out, const float2* __restrict__ x, long long n,
                                                        double* part, double* scal, unsigned* ticket) {
+  out += blockIdx.y * n;
+  x += blockIdx.y * n;
   double v[2] = {0.0, 0.0};
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-    const float2 a = out[i], b = x[i];
-    const double er = (double)a.x - b.x, ei = (double)a.y - b.y;
-    v[0] += (double)b.x * b.x + (double)b.y * b.y;
-    v[1] += er * er + ei * ei;
+  const long long gs = (long long)gridDim.x * 256;
+  for (long long i0 = blockIdx.x * 256LL + threadIdx.x; i0 < n; i0 += gs * LOSS_CHUNK) {
+    float2 a[LOSS_CHUNK], b[LOSS_CHUNK];
+    float mx = 0.f;
+#pragma unroll
+    for (int u = 0; u < LOSS_CHUNK; ++u) {
+      const long long i = i0 + u * gs;
+      a[u] = b[u] = make_float2(0.f, 0.f);
+      if (i < n) { a[u] = out[i]; b[u] = x[i]; }
+    }
+    bool nan = false;
+#pragma unroll
+    for (int u = 0; u < LOSS_CHUNK; ++u) {
+      mx = fmaxf(fmaxf(fmaxf(mx, fabsf(a[u].x)), fmaxf(fabsf(a[u].y), fabsf(b[u].x))), fabsf(b[u].y));
+      nan = nan || isnan(a[u].x) || isnan(a[u].y) || isnan(b[u].x) || isnan(b[u].y);
+    }
+    if (mx == 0.f && !nan) continue;
+    if (mx >= 0x1p-40f && mx <= 0x1p40f && !nan) {
+      dd s0(0.f, 0.f), s1(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < LOSS_CHUNK; ++u) {
+        s0 = s0 + dd_sq(dd(b[u].x, 0.f));
+        s0 = s0 + dd_sq(dd(b[u].y, 0.f));
+        s1 = s1 + dd_sq(dd_diff(a[u].x, b[u].x));
+        s1 = s1 + dd_sq(dd_diff(a[u].y, b[u].y));
+      }
+      v[0] += (double)s0;
+      v[1] += (double)s1;
+    } else {
+#pragma unroll 1
+      for (int u = 0; u < LOSS_CHUNK; ++u) {
+        const long long i = i0 + u * gs;
+        if (i >= n) break;
+        const float2 o = out[i], y = x[i];
+        const double er = (double)o.x - y.x, ei = (double)o.y - y.y;
+        v[0] += (double)y.x * y.x + (double)y.y * y.y;
+        v[1] += er * er + ei * ei;
+      }
+    }
   }
-  const RedArgs ra{nullptr, part, scal, FIN_NONE};
-  grid_reduce<2, 256>(v, ra, ticket);
+  const RedArgs ra{nullptr, part + (size_t)blockIdx.y * 2 * gridDim.x, scal + 2 + 2 * blockIdx.y, FIN_NONE};
+  grid_reduce<2, 256>(v, ra, ticket + blockIdx.y);
 }
 
-// g = (out - x) / |x|^2; block 0 adds this pair's loss to scal[2].
-__global__ void __launch_bounds__(256) net_seed_kernel(const float2* __restrict__ out, const float2* __restrict__ x, float2* g,
-                                                       long long n, double* scal) {
-  const double n2 = scal[0];
-  const float inv = n2 > 0.0 ? (float)(1.0 / n2) : 0.f;
+// g = (out - x) / |x|^2 for pair blockIdx.y; one thread adds the group's losses to scal[0].
+__global__ void __launch_bounds__(256) net_seed_kernel(const float2* __restrict__ out, const float2* __restrict__ x,
+                                                       float2* __restrict__ g, long long n, double* scal) {
+  __shared__ float inv_s;
+  if (threadIdx.x == 0) {
+    const double n2 = scal[2 + 2 * blockIdx.y];
+    inv_s = n2 > 0.0 ? (float)(1.0 / n2) : 0.f;  // one FP64 division per block, not per thread
+  }
+  __syncthreads();
+  const float inv = inv_s;
+  out += blockIdx.y * n;
+  x += blockIdx.y * n;
+  g += blockIdx.y * n;
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
     const float2 a = out[i], b = x[i];
     g[i] = make_float2((a.x - b.x) * inv, (a.y - b.y) * inv);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) scal[2] += n2 > 0.0 ? scal[1] / n2 : 0.0;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    double s = scal[0];
+    for (unsigned q = 0; q < gridDim.y; ++q) s += scal[2 + 2 * q] > 0.0 ? scal[3 + 2 * q] / scal[2 + 2 * q] : 0.0;
+    scal[0] = s;
+  }
 }
 
-__global__ void net_adam_kernel(float* P, float* m, float* v, const double* gacc, int n, double scale, float lr, float b1, float b2,
-                                float eps, float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gr = (float)(gacc[i] * scale);
-  m[i] = b1 * m[i] + (1.f - b1) * gr;
-  v[i] = b2 * v[i] + (1.f - b2) * gr * gr;
-  const float mh = m[i] / c1, vh = v[i] / c2;
-  P[i] -= lr * mh / (sqrtf(vh) + eps);
+// Two blocks of GRAD_THREADS threads fit on a multiprocessor.
+int grad_blocks(int V) {
+  const int need = (V + 31) / 32;
+  const int cap = sm_count() * 2;
+  return need < cap ? need : cap;
 }
 
-int net_blocks(int V) {
-  const int need = grid_for(V, NET_THREADS);
+int loss_blocks(int V) {
+  const int need = grid_for((12LL * V + LOSS_CHUNK - 1) / LOSS_CHUNK, 256);
   const int cap = sm_count() * 4;
   return need < cap ? need : cap;
 }
 
-// Scratch for a lattice of V sites: two fields (the layer ping-pong and the backward gradients),
-// the reduction partials, and, for training, the activations of every layer.
-int ensure_workspace(ok_net* N, int V, bool training) {
-  if (N->V == V && N->g[0] && (!training || N->acts)) return OK_SUCCESS;
+void free_training(ok_net* N) {
+  for (void* q : {(void*)N->acts, (void*)N->tg[0], (void*)N->tg[1], (void*)N->part, (void*)N->lpart})
+    if (q) cudaFree(q);
+  N->acts = N->tg[0] = N->tg[1] = nullptr;
+  N->part = N->lpart = nullptr;
+  N->group = 0;
+}
+
+// Pairs of a batch of nb that one pass of the kernels takes: as many as fit in 256 MiB of
+// activations (enough to fill the GPU: the launches of a small lattice hold little work each).
+int group_of(const ok_net* N, int V, int nb) {
+  const long long per = (long long)N->layers * V * 12 * (long long)sizeof(cx<float>);
+  long long q = (256LL << 20) / per;
+  if (q > MAX_GROUP) q = MAX_GROUP;
+  if (q > nb) q = nb;
+  return q < 1 ? 1 : (int)q;
+}
+
+// Scratch for a lattice of V sites: two fields (the layer ping-pong of an application) and, for
+// training (nb > 0), the activations of every layer, the backward gradients and the reduction
+// partials of a group of pairs; a group that does not fit in memory falls back to one pair.
+int ensure_workspace(ok_net* N, int V, int nb) {
   const size_t n = (size_t)V * 12;
   if (N->V != V) {
-    if (N->acts) cudaFree(N->acts);
+    free_training(N);
     if (N->g[0]) cudaFree(N->g[0]);
     if (N->g[1]) cudaFree(N->g[1]);
-    if (N->part) cudaFree(N->part);
-    N->acts = nullptr; N->g[0] = N->g[1] = nullptr; N->part = nullptr; N->V = 0;
+    N->g[0] = N->g[1] = nullptr; N->V = 0;
     OK_CUDA_TRY(cudaMalloc(&N->g[0], n * sizeof(cx<float>)));
     OK_CUDA_TRY(cudaMalloc(&N->g[1], n * sizeof(cx<float>)));
-    N->part_blocks = net_blocks(V);
-    const int lb = grid_for((long long)n, 256) < 1024 ? grid_for((long long)n, 256) : 1024;
-    size_t pn = (size_t)N->part_blocks * NPAR;
-    if ((size_t)lb * 2 > pn) pn = (size_t)lb * 2;
-    OK_CUDA_TRY(cudaMalloc(&N->part, pn * sizeof(double)));
     N->V = V;
   }
-  if (training && !N->acts) OK_CUDA_TRY(cudaMalloc(&N->acts, (size_t)N->layers * n * sizeof(cx<float>)));
+  if (nb < 1) return OK_SUCCESS;
+  int want = group_of(N, V, nb);
+  if (N->group >= want) return OK_SUCCESS;
+  for (;;) {
+    free_training(N);
+    const size_t f = want * n * sizeof(cx<float>);
+    cudaError_t e = cudaMalloc(&N->acts, N->layers * f);
+    if (e == cudaSuccess) e = cudaMalloc(&N->tg[0], f);
+    if (e == cudaSuccess) e = cudaMalloc(&N->tg[1], f);
+    if (e == cudaSuccess) e = cudaMalloc(&N->part, (size_t)N->layers * grad_blocks(V) * NPAR * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&N->lpart, (size_t)want * 2 * loss_blocks(V) * sizeof(double));
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    free_training(N);
+    if (want == 1) { set_cuda_error(e); return OK_ECUDA; }
+    want = 1;
+  }
+  N->group = want;
   return OK_SUCCESS;
 }
 
@@ -323,46 +462,61 @@ int layer(const ok_net* N, const ok_W* W, int l, bool adj, const cx<float>* in, 
     if (_rc != OK_SUCCESS) return _rc;      \
   } while (0)
 
-// The gradient of one pair added into gacc (and its loss into scal[2]).
-int pair_backprop(ok_net* N, const ok_W* W, const cx<float>* b, const cx<float>* x, cudaStream_t st) {
+// The gradient partials of `pairs` pairs ([pairs][V * 12] fields), added to those of the batch's
+// earlier groups unless `first`, and their losses into scal[0].
+int group_backprop(ok_net* N, const ok_W* W, int pairs, const cx<float>* b, const cx<float>* x, bool first, cudaStream_t st) {
   const Geom& g = W->g;
-  const long long n = 12LL * g.V;
+  const long long n = 12LL * g.V, gn = n * pairs;
   const int K = N->layers;
   const cx<float>* in = b;
   for (int l = 0; l < K; ++l) {
-    cx<float>* o = N->acts + (size_t)l * n;
-    NET_TRY(layer(N, W, l, false, in, o, st));
+    cx<float>* o = N->acts + (size_t)l * gn;
+    NET_TRY(layer(N, W, l, false, in, o, st, pairs));
     in = o;
   }
-  const int lb = grid_for(n, 256) < 1024 ? grid_for(n, 256) : 1024;
+  const int lb = loss_blocks(g.V), gb = grad_blocks(g.V);
   {
     TraceScope ts("net_loss", st);
-    net_loss_kernel<<<lb, 256, 0, st>>>((const float2*)in, (const float2*)x, n, N->part, N->scal, N->ticket);
+    net_loss_kernel<<<dim3(lb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, n, N->lpart, N->scal, N->ticket);
   }
   OK_LAUNCH_CHECK();
   {
     TraceScope ts("net_seed", st);
-    net_seed_kernel<<<lb, 256, 0, st>>>((const float2*)in, (const float2*)x, (float2*)N->g[0], n, N->scal);
+    const int sb = grid_for(n, 256) < 1024 ? grid_for(n, 256) : 1024;
+    net_seed_kernel<<<dim3(sb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, (float2*)N->tg[0], n, N->scal);
   }
   OK_LAUNCH_CHECK();
   int cur = 0;
   for (int l = K - 1; l >= 0; --l) {
-    const cx<float>* lin = l == 0 ? b : N->acts + (size_t)(l - 1) * n;
+    const cx<float>* lin = l == 0 ? b : N->acts + (size_t)(l - 1) * gn;
     {
       TraceScope ts("net_grad", st);
-      net_grad_kernel<<<N->part_blocks, NET_THREADS, 0, st>>>((const cx<float>*)W->L32, N->g[cur], lin, g, N->part);
-    }
-    OK_LAUNCH_CHECK();
-    {
-      TraceScope ts("net_grad_final", st);
-      net_grad_final_kernel<<<1, 288, 0, st>>>(N->part, N->part_blocks, N->gacc + (size_t)l * NPAR);
+      net_grad_kernel<<<gb, GRAD_THREADS, 0, st>>>((const cx<float>*)W->L32, N->tg[cur], lin, g, pairs,
+                                                   N->part + (size_t)l * gb * NPAR, !first);
     }
     OK_LAUNCH_CHECK();
     if (l > 0) {
-      NET_TRY(layer(N, W, l, true, N->g[cur], N->g[1 - cur], st));
+      NET_TRY(layer(N, W, l, true, N->tg[cur], N->tg[1 - cur], st, pairs));
       cur = 1 - cur;
     }
   }
+  return OK_SUCCESS;
+}
+
+// Loss sum (scal[0]) and gradient (gacc, with `ad` applied) over nb pairs.
+int batch_backprop(ok_net* N, const ok_W* W, int nb, const cx<float>* b, const cx<float>* x, const AdamArgs& ad, cudaStream_t st) {
+  NET_TRY(ensure_workspace(N, W->g.V, nb));
+  OK_CUDA_TRY(cudaMemsetAsync(N->scal, 0, sizeof(double), st));
+  const size_t n = (size_t)W->g.V * 12;
+  for (int i = 0; i < nb; i += N->group) {
+    const int pairs = nb - i < N->group ? nb - i : N->group;
+    NET_TRY(group_backprop(N, W, pairs, b + i * n, x + i * n, i == 0, st));
+  }
+  {
+    TraceScope ts("net_grad_final", st);
+    net_grad_final_kernel<<<N->layers * NOFF, 256, 0, st>>>(N->part, grad_blocks(W->g.V), N->gacc, ad);
+  }
+  OK_LAUNCH_CHECK();
   return OK_SUCCESS;
 }
 
@@ -378,7 +532,7 @@ int check(const ok_net* N, const ok_W* W) {
 int net_apply_unless_halted(ok_net* N, const ok_W* W, const cx<float>* in, cx<float>* out, const int* halt,
                            cudaStream_t st) {
   NET_TRY(check(N, W));
-  NET_TRY(ensure_workspace(N, W->g.V, false));
+  NET_TRY(ensure_workspace(N, W->g.V, 0));
   const cx<float>* cur = in;
   for (int l = 0; l < N->layers; ++l) {
     cx<float>* o = l == N->layers - 1 ? out : N->g[l % 2];  // ping-pong through the workspace
@@ -410,15 +564,12 @@ int net_apply_multi(ok_net* N, const ok_W* W, const cx<float>* in, cx<float>* ou
 
 int net_loss_grad(ok_net* N, const ok_W* W, const cx<float>* b, const cx<float>* x, double* loss, double* grad, cudaStream_t st) {
   NET_TRY(check(N, W));
-  NET_TRY(ensure_workspace(N, W->g.V, true));
-  OK_CUDA_TRY(cudaMemsetAsync(N->gacc, 0, sizeof(double) * NPAR * N->layers, st));
-  OK_CUDA_TRY(cudaMemsetAsync(N->scal, 0, sizeof(double) * 4, st));
-  NET_TRY(pair_backprop(N, W, b, x, st));
-  double s[4];
-  OK_CUDA_TRY(cudaMemcpyAsync(s, N->scal, sizeof(s), cudaMemcpyDeviceToHost, st));
+  NET_TRY(batch_backprop(N, W, 1, b, x, AdamArgs{}, st));
+  double s = 0.0;
+  OK_CUDA_TRY(cudaMemcpyAsync(&s, N->scal, sizeof(s), cudaMemcpyDeviceToHost, st));
   if (grad) OK_CUDA_TRY(cudaMemcpyAsync(grad, N->gacc, sizeof(double) * NPAR * N->layers, cudaMemcpyDeviceToHost, st));
   OK_CUDA_TRY(cudaStreamSynchronize(st));
-  if (loss) *loss = s[2];
+  if (loss) *loss = s;
   return OK_SUCCESS;
 }
 
@@ -426,25 +577,15 @@ int net_train_step(ok_net* N, const ok_W* W, int nb, const cx<float>* b, const c
                    cudaStream_t st) {
   NET_TRY(check(N, W));
   if (nb < 1 || !b || !x || !(lr > 0.0)) return OK_EINVAL;
-  NET_TRY(ensure_workspace(N, W->g.V, true));
-  const long long n = 12LL * W->g.V;
-  OK_CUDA_TRY(cudaMemsetAsync(N->gacc, 0, sizeof(double) * NPAR * N->layers, st));
-  OK_CUDA_TRY(cudaMemsetAsync(N->scal, 0, sizeof(double) * 4, st));
-  for (int i = 0; i < nb; ++i) NET_TRY(pair_backprop(N, W, b + (size_t)i * n, x + (size_t)i * n, st));
-  N->adam_t += 1;
   const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.f - powf(b1, (float)N->adam_t), c2 = 1.f - powf(b2, (float)N->adam_t);
-  const int np = NPAR * N->layers;
-  {
-    TraceScope ts("net_adam", st);
-    net_adam_kernel<<<grid_for(np, 256), 256, 0, st>>>((float*)N->A, N->m, N->v, N->gacc, np, 1.0 / nb, (float)lr, b1, b2, 1e-8f,
-                                                        c1, c2);
-  }
-  OK_LAUNCH_CHECK();
-  double s[4];
-  OK_CUDA_TRY(cudaMemcpyAsync(s, N->scal, sizeof(s), cudaMemcpyDeviceToHost, st));
+  const float t = (float)(N->adam_t + 1);
+  const float c1 = 1.f - powf(b1, t), c2 = 1.f - powf(b2, t);
+  NET_TRY(batch_backprop(N, W, nb, b, x, AdamArgs{(float*)N->A, N->m, N->v, 1.0 / nb, (float)lr, b1, b2, 1e-8f, c1, c2}, st));
+  N->adam_t += 1;
+  double s = 0.0;
+  OK_CUDA_TRY(cudaMemcpyAsync(&s, N->scal, sizeof(s), cudaMemcpyDeviceToHost, st));
   OK_CUDA_TRY(cudaStreamSynchronize(st));
-  if (loss) *loss = s[2] / nb;
+  if (loss) *loss = s / nb;
   return OK_SUCCESS;
 }
 
@@ -463,10 +604,11 @@ int net_create(int layers, const double* w, ok_net** out) {
   const size_t np = (size_t)NPAR * layers;
   if (cudaMalloc(&N->A, np * sizeof(float)) != cudaSuccess || cudaMalloc(&N->m, np * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&N->v, np * sizeof(float)) != cudaSuccess || cudaMalloc(&N->gacc, np * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&N->scal, 4 * sizeof(double)) != cudaSuccess || cudaMalloc(&N->ticket, sizeof(unsigned)) != cudaSuccess)
+      cudaMalloc(&N->scal, (2 + 2 * MAX_GROUP) * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&N->ticket, MAX_GROUP * sizeof(unsigned)) != cudaSuccess)
     return fail(OK_ENOMEM);
   if (cudaMemset(N->m, 0, np * sizeof(float)) != cudaSuccess || cudaMemset(N->v, 0, np * sizeof(float)) != cudaSuccess ||
-      cudaMemset(N->ticket, 0, sizeof(unsigned)) != cudaSuccess)
+      cudaMemset(N->ticket, 0, MAX_GROUP * sizeof(unsigned)) != cudaSuccess)
     return fail(OK_ECUDA);
   std::vector<float> h(np, 0.f);
   for (size_t i = 0; i < np; ++i) h[i] = w ? (float)w[i] : 0.f;
@@ -481,7 +623,8 @@ int net_create(int layers, const double* w, ok_net** out) {
 void net_free(ok_net* N) {
   if (!N) return;
   cudaFree(N->A); cudaFree(N->m); cudaFree(N->v); cudaFree(N->gacc); cudaFree(N->scal); cudaFree(N->ticket);
-  cudaFree(N->acts); cudaFree(N->g[0]); cudaFree(N->g[1]); cudaFree(N->part);
+  free_training(N);
+  cudaFree(N->g[0]); cudaFree(N->g[1]);
   delete N;
 }
 
