@@ -4,9 +4,12 @@ import pytest
 
 import synth
 from oracle import precond
-from gpu_common import ok, rel_l2, to_dev, torch
+from tests.gpu_common import rel_l2, to_dev
 
 pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+ok = pytest.importorskip("paper_1311_5029_gb300")
 
 
 def _weights(layers, seed):
