@@ -4,11 +4,12 @@
 // the neighbour (Eqs. conjugate and opp_diag_pre_mat: W^-_{mu,x} = gamma5 W^{+ dagger}_{mu,x-mu}
 // gamma5 and so on).
 //
-// Spin handling.  With psi = (u, l) its upper and lower 2-spin halves, every hop except W^0 is
-// block diagonal in h+- = u +- l, so the kernel accumulates
-//   acc+ = (out_u + out_l) / 2,   acc- = (out_u - out_l) / 2
-// (the 1/2 is folded into the stored matrices) and writes out_u = acc+ + acc-,
-// out_l = acc+ - acc- at the end.  W^0 is block diagonal in u -+ i l instead.  In this basis the
+// Spin handling.  With psi = (u, l) its upper and lower 2-spin halves, the nearest spatial hops are
+// block diagonal in h+- = u +- l: the stored (D +- S) / 2 act on h+- and add to
+//   acc+ = (out_u + out_l) / 2,   acc- = (out_u - out_l) / 2.
+// W^0 is block diagonal in u -+ i l.  The temporal, two-hop and diagonal hops are [[A, B], [B, D]] with
+// A, B, D spin matrices times one colour matrix, so they act on u and l as they are and add to the
+// half outputs D_u = out_u / 2, D_l = out_l / 2 (the stored matrices hold the 1/2).  In these bases the
 // 148 colour matrix-vector products per site are the only dense work.
 //
 // Precision R = double or float: loads, arithmetic and stores in R.  Fused epilogues feed the
@@ -51,101 +52,163 @@ __device__ __forceinline__ void hop_spatial(const cx<R>* __restrict__ W, const c
   block2<R, true>(W, n, mp, hm, am);
 }
 
-// Temporal nearest neighbours: W^+_4 = [[0, S], [S, -U]], W^-_4 = [[-U^dag, -S^dag], [-S^dag, 0]].
+// The halves u, l of the neighbour at offset d, with the boundary sign.
+template <typename R, int D0, int D1, int D2, int D3>
+__device__ __forceinline__ int gather_ul(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, Half<R>& u, Half<R>& l) {
+  bool neg;
+  const int n = nbr_site<D0, D1, D2, D3>(c, g, neg);
+  cx<R> v[12];
+  load_spinor<R>(psi, n, v);
+  if (neg) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = -v[k];
+  }
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      u.v[s][a] = v[3 * s + a];
+      l.v[s][a] = v[3 * (s + 2) + a];
+    }
+  return n;
+}
+
+// Temporal nearest neighbours on (u, l): W^+_4 = [[0, S], [S, -U]] at x, W^-_4 = [[-U^dag, -S^dag], [-S^dag, 0]]
+// from x - t, S = [[s3, n1], [n2, -s3]].
 template <typename R>
 __device__ __forceinline__ void hop_time(const cx<R>* __restrict__ W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                         const Geom& g, int s, Half<R>& ap, Half<R>& am) {
-  Half<R> hp, hm, lo, up, w;
-  // forward at x: acc+ += S h+ - U l, acc- += U l - S h- (stored halves)
-  gather_h<R, 0, 0, 0, 1>(psi, c, g, hp, hm, nullptr, &lo);
-  {
-    M3<R> U = wmat(W, s, M_UT);
-    colour2<R, false>(w, U, lo);
+                                         const Geom& g, int s, Half<R>& du, Half<R>& dl) {
+  Half<R> u, l;
+  gather_ul<R, 0, 0, 0, 1>(psi, c, g, u, l);
+  M3<R> A = wmat(W, s, M_UT);
+  mv_sub(dl.v[0], A, l.v[0]); mv_sub(dl.v[1], A, l.v[1]);
+  A = wmat(W, s, M_ST + 0);
+  mv_add(du.v[0], A, l.v[0]); mv_sub(du.v[1], A, l.v[1]);
+  mv_add(dl.v[0], A, u.v[0]); mv_sub(dl.v[1], A, u.v[1]);
+  A = wmat(W, s, M_ST + 1);
+  mv_add(du.v[0], A, l.v[1]); mv_add(dl.v[0], A, u.v[1]);
+  A = wmat(W, s, M_ST + 2);
+  mv_add(du.v[1], A, l.v[0]); mv_add(dl.v[1], A, u.v[0]);
+  const int n = gather_ul<R, 0, 0, 0, -1>(psi, c, g, u, l);
+  // S^dag = [[s3^dag, n2^dag], [n1^dag, -s3^dag]]
+  A = wmat(W, n, M_UT);
+  mdv_sub(du.v[0], A, u.v[0]); mdv_sub(du.v[1], A, u.v[1]);
+  A = wmat(W, n, M_ST + 0);
+  mdv_sub(du.v[0], A, l.v[0]); mdv_add(du.v[1], A, l.v[1]);
+  mdv_sub(dl.v[0], A, u.v[0]); mdv_add(dl.v[1], A, u.v[1]);
+  A = wmat(W, n, M_ST + 2);
+  mdv_sub(du.v[0], A, l.v[1]); mdv_sub(dl.v[0], A, u.v[1]);
+  A = wmat(W, n, M_ST + 1);
+  mdv_sub(du.v[1], A, l.v[0]); mdv_sub(dl.v[1], A, u.v[0]);
+}
+
+// sigma_k y.
+template <typename R>
+__device__ __forceinline__ void sigma_half(int k, const Half<R>& y, Half<R>& s) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) { ap.v[q][a] = ap.v[q][a] - w.v[q][a]; am.v[q][a] = am.v[q][a] + w.v[q][a]; }
-    M3<R> s3 = wmat(W, s, M_ST + 0);
-    mv_add(ap.v[0], s3, hp.v[0]); mv_sub(ap.v[1], s3, hp.v[1]);
-    mv_sub(am.v[0], s3, hm.v[0]); mv_add(am.v[1], s3, hm.v[1]);
-    M3<R> n1 = wmat(W, s, M_ST + 1);
-    mv_add(ap.v[0], n1, hp.v[1]); mv_sub(am.v[0], n1, hm.v[1]);
-    M3<R> n2 = wmat(W, s, M_ST + 2);
-    mv_add(ap.v[1], n2, hp.v[0]); mv_sub(am.v[1], n2, hm.v[0]);
-  }
-  // backward from x - t: acc+ += -U^dag u - S^dag h+, acc- += -U^dag u + S^dag h-
-  int n = gather_h<R, 0, 0, 0, -1>(psi, c, g, hp, hm, &up, nullptr);
-  {
-    M3<R> U = wmat(W, n, M_UT);
-    colour2<R, true>(w, U, up);
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) { ap.v[q][a] = ap.v[q][a] - w.v[q][a]; am.v[q][a] = am.v[q][a] - w.v[q][a]; }
-    // S^dag = [[s3^dag, n2^dag], [n1^dag, -s3^dag]]
-    M3<R> s3 = wmat(W, n, M_ST + 0);
-    mdv_sub(ap.v[0], s3, hp.v[0]); mdv_add(ap.v[1], s3, hp.v[1]);
-    mdv_add(am.v[0], s3, hm.v[0]); mdv_sub(am.v[1], s3, hm.v[1]);
-    M3<R> n1 = wmat(W, n, M_ST + 1);
-    mdv_sub(ap.v[1], n1, hp.v[0]); mdv_add(am.v[1], n1, hm.v[0]);
-    M3<R> n2 = wmat(W, n, M_ST + 2);
-    mdv_sub(ap.v[0], n2, hp.v[1]); mdv_add(am.v[0], n2, hm.v[1]);
+  for (int a = 0; a < 3; ++a) {
+    s.v[0][a] = k == 0 ? y.v[1][a] : k == 1 ? tmi(y.v[1][a]) : y.v[0][a];
+    s.v[1][a] = k == 0 ? y.v[0][a] : k == 1 ? ti(y.v[0][a]) : -y.v[1][a];
   }
 }
 
-// Straight two-hop neighbours x +- 2I: W^{++}_ii = (a + b sigma_i) V on h+, (a - b sigma_i) V on h-.
+// The spin part of a straight two-hop term, applied to the spinor before the colour matrix:
+// a u + b sigma l = big (u + r sigma l) when |a| >= |b| (a_big), else big (r u + sigma l), |r| <= 1.  One
+// multiply-add per component; the factor big multiplies the sum of the six terms once.
+template <typename R> struct TwoHop { R big, r; bool a_big; };
+template <typename R>
+__device__ __forceinline__ Half<R> two_combine(const TwoHop<R>& q, R r, const Half<R>& u, const Half<R>& sl, bool minus) {
+  Half<R> w;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const cx<R> b = minus ? -sl.v[s][a] : sl.v[s][a];
+      const cx<R> x = q.a_big ? u.v[s][a] : b, y = q.a_big ? b : u.v[s][a];
+      w.v[s][a] = mk<R>(fma(r, y.re, x.re), fma(r, y.im, x.im));
+    }
+  return w;
+}
+
+// Straight two-hop neighbours x +- 2I: [[a, +-b sigma_i], [+-b sigma_i, a]] (x) V (at x), V^dag (at x - 2I),
+// without the factor q.big.
 template <typename R, int I>
 __device__ __forceinline__ void hop_two(const cx<R>* __restrict__ W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                        const Geom& g, int s, R a, R b, Half<R>& ap, Half<R>& am) {
-  Half<R> hp, hm, y;
-  gather_h<R, 2 * (I == 0), 2 * (I == 1), 2 * (I == 2), 0>(psi, c, g, hp, hm);
-  M3<R> V = wmat(W, s, M_VII + I);
-  colour2<R, false>(y, V, hp);
-  add_scaled(ap, a, y); add_sigma(ap, I, y, b);
-  colour2<R, false>(y, V, hm);
-  add_scaled(am, a, y); add_sigma(am, I, y, -b);
-  int n = gather_h<R, -2 * (I == 0), -2 * (I == 1), -2 * (I == 2), 0>(psi, c, g, hp, hm);
-  V = wmat(W, n, M_VII + I);
-  colour2<R, true>(y, V, hp);
-  add_scaled(ap, a, y); add_sigma(ap, I, y, -b);
-  colour2<R, true>(y, V, hm);
-  add_scaled(am, a, y); add_sigma(am, I, y, b);
+                                        const Geom& g, int s, const TwoHop<R>& q, Half<R>& du, Half<R>& dl) {
+  Half<R> u, l, t;
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    int n = s;
+    if (f == 0) gather_ul<R, 2 * (I == 0), 2 * (I == 1), 2 * (I == 2), 0>(psi, c, g, u, l);
+    else n = gather_ul<R, -2 * (I == 0), -2 * (I == 1), -2 * (I == 2), 0>(psi, c, g, u, l);
+    const M3<R> V = wmat(W, n, M_VII + I);
+    sigma_half(I, l, t);
+    const Half<R> wu = two_combine(q, q.r, u, t, f == 1);
+    sigma_half(I, u, t);
+    const Half<R> wl = two_combine(q, q.r, l, t, f == 1);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      if (f == 0) { mv_add(du.v[p], V, wu.v[p]); mv_add(dl.v[p], V, wl.v[p]); }
+      else { mdv_add(du.v[p], V, wu.v[p]); mdv_add(dl.v[p], V, wl.v[p]); }
+    }
+  }
 }
 
-// Diagonal neighbours of the pair (I, J), I < J, P = pair index:
-//   x+I+J: acc+ += (s_I + s_J) V h+, acc- -= (s_I + s_J) V h-             (V at x)
-//   x-I-J: acc+ -= (s_I + s_J) V^dag h+, acc- += (s_I + s_J) V^dag h-     (V at x-I-J)
-//   x+I-J: acc+ += (s_I - s_J) X h+, acc- -= (s_I - s_J) X h-             (X at x)
-//   x-I+J: acc+ -= (s_I - s_J) X^dag h+, acc- += (s_I - s_J) X^dag h-     (X at x-I+J)
+// w = (sigma_I + SG sigma_J) y, I < J.
+template <typename R, int I, int J, int SG>
+__device__ __forceinline__ Half<R> sigma_sum(const Half<R>& y) {
+  Half<R> w;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cx<R> p = y.v[0][a], q = y.v[1][a];
+    if constexpr (I == 0 && J == 1) {
+      w.v[0][a] = SG > 0 ? q + tmi(q) : q + ti(q);
+      w.v[1][a] = SG > 0 ? p + ti(p) : p + tmi(p);
+    } else if constexpr (I == 0) {
+      w.v[0][a] = SG > 0 ? q + p : q - p;
+      w.v[1][a] = SG > 0 ? p - q : p + q;
+    } else {
+      w.v[0][a] = SG > 0 ? tmi(q) + p : tmi(q) - p;
+      w.v[1][a] = SG > 0 ? ti(p) - q : ti(p) + q;
+    }
+  }
+  return w;
+}
+
+// Diagonal neighbours of the pair (I, J), I < J, P = pair index: [[0, S], [S, 0]] with
+// S = (s_I + s_J) (x) V from x+I+J and (s_I - s_J) (x) X from x+I-J, minus the adjoints from x-I-J, x-I+J.
 template <typename R, int I, int J, int P>
 __device__ __forceinline__ void hop_diag(const cx<R>* __restrict__ W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                         const Geom& g, int s, Half<R>& ap, Half<R>& am) {
+                                         const Geom& g, int s, Half<R>& du, Half<R>& dl) {
   constexpr int A0 = (I == 0) + (J == 0), A1 = (I == 1) + (J == 1), A2 = (I == 2) + (J == 2);
   constexpr int B0 = (I == 0) - (J == 0), B1 = (I == 1) - (J == 1), B2 = (I == 2) - (J == 2);
-  Half<R> hp, hm, y;
-  M3<R> V;
-  gather_h<R, A0, A1, A2, 0>(psi, c, g, hp, hm);
-  V = wmat(W, s, M_VIJ + P);
-  colour2<R, false>(y, V, hp); add_sigma(ap, I, y, R(1)); add_sigma(ap, J, y, R(1));
-  colour2<R, false>(y, V, hm); add_sigma(am, I, y, R(-1)); add_sigma(am, J, y, R(-1));
-  int n = gather_h<R, -A0, -A1, -A2, 0>(psi, c, g, hp, hm);
+  Half<R> u, l, w;
+  gather_ul<R, A0, A1, A2, 0>(psi, c, g, u, l);
+  M3<R> V = wmat(W, s, M_VIJ + P);
+  w = sigma_sum<R, I, J, 1>(l); mv_add(du.v[0], V, w.v[0]); mv_add(du.v[1], V, w.v[1]);
+  w = sigma_sum<R, I, J, 1>(u); mv_add(dl.v[0], V, w.v[0]); mv_add(dl.v[1], V, w.v[1]);
+  int n = gather_ul<R, -A0, -A1, -A2, 0>(psi, c, g, u, l);
   V = wmat(W, n, M_VIJ + P);
-  colour2<R, true>(y, V, hp); add_sigma(ap, I, y, R(-1)); add_sigma(ap, J, y, R(-1));
-  colour2<R, true>(y, V, hm); add_sigma(am, I, y, R(1)); add_sigma(am, J, y, R(1));
-  gather_h<R, B0, B1, B2, 0>(psi, c, g, hp, hm);
+  w = sigma_sum<R, I, J, 1>(l); mdv_sub(du.v[0], V, w.v[0]); mdv_sub(du.v[1], V, w.v[1]);
+  w = sigma_sum<R, I, J, 1>(u); mdv_sub(dl.v[0], V, w.v[0]); mdv_sub(dl.v[1], V, w.v[1]);
+  gather_ul<R, B0, B1, B2, 0>(psi, c, g, u, l);
   V = wmat(W, s, M_XIJ + P);
-  colour2<R, false>(y, V, hp); add_sigma(ap, I, y, R(1)); add_sigma(ap, J, y, R(-1));
-  colour2<R, false>(y, V, hm); add_sigma(am, I, y, R(-1)); add_sigma(am, J, y, R(1));
-  n = gather_h<R, -B0, -B1, -B2, 0>(psi, c, g, hp, hm);
+  w = sigma_sum<R, I, J, -1>(l); mv_add(du.v[0], V, w.v[0]); mv_add(du.v[1], V, w.v[1]);
+  w = sigma_sum<R, I, J, -1>(u); mv_add(dl.v[0], V, w.v[0]); mv_add(dl.v[1], V, w.v[1]);
+  n = gather_ul<R, -B0, -B1, -B2, 0>(psi, c, g, u, l);
   V = wmat(W, n, M_XIJ + P);
-  colour2<R, true>(y, V, hp); add_sigma(ap, I, y, R(-1)); add_sigma(ap, J, y, R(1));
-  colour2<R, true>(y, V, hm); add_sigma(am, I, y, R(1)); add_sigma(am, J, y, R(-1));
+  w = sigma_sum<R, I, J, -1>(l); mdv_sub(du.v[0], V, w.v[0]); mdv_sub(du.v[1], V, w.v[1]);
+  w = sigma_sum<R, I, J, -1>(u); mdv_sub(dl.v[0], V, w.v[0]); mdv_sub(dl.v[1], V, w.v[1]);
 }
 
 // ---------------------------------------------------------------------------- the kernel
+// One thread per site, for FP64: the FP64 pipe runs at 1/58 of the FP32 rate and bounds the kernel, so
+// what counts is the number of FP64 operations.  5328 of them per site are the products'
+// multiply-adds; acting on u and l wherever a hop allows leaves about 750 additions beside them, where
+// the h+- basis throughout took about 1600 (16^3 x 32: 1625 us before, 1401 us now).
 template <typename R, int EPI>
 __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(const cx<R>* __restrict__ W, const cx<R>* __restrict__ psi,
-                                                              cx<R>* __restrict__ out, Geom g, R c0q, R a_ii, R b_ii,
+                                                              cx<R>* __restrict__ out, Geom g, R c0q, TwoHop<R> two,
                                                               EpiArgs<R> ep) {
   if (ep.halt && *ep.halt) return;
   const int s = blockIdx.x * APPLY_THREADS + threadIdx.x;
@@ -159,10 +222,38 @@ __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(const cx<R>* __res
       c[2] = r % g.L[2]; c[3] = r / g.L[2];
     }
     Half<R> ap, am;
-    cx<R> x0[12];
-    // on-site: a = u - i l, b = u + i l; A = Y+ a, B = Y- b; acc+- = (A + B) +- i (A - B)
-    load_spinor<R>(psi, s, x0);
     {
+      Half<R> du, dl;
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) du.v[q][k] = dl.v[q][k] = mk<R>(0, 0);
+      hop_two<R, 0>(W, psi, c, g, s, two, du, dl);
+      hop_two<R, 1>(W, psi, c, g, s, two, du, dl);
+      hop_two<R, 2>(W, psi, c, g, s, two, du, dl);
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          du.v[q][k] = two.big * du.v[q][k];
+          dl.v[q][k] = two.big * dl.v[q][k];
+        }
+      hop_time<R>(W, psi, c, g, s, du, dl);
+      hop_diag<R, 0, 1, 0>(W, psi, c, g, s, du, dl);
+      hop_diag<R, 0, 2, 1>(W, psi, c, g, s, du, dl);
+      hop_diag<R, 1, 2, 2>(W, psi, c, g, s, du, dl);
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          ap.v[q][k] = du.v[q][k] + dl.v[q][k];
+          am.v[q][k] = du.v[q][k] - dl.v[q][k];
+        }
+    }
+    // on-site: a = u - i l, b = u + i l; A = Y+ a, B = Y- b; acc+- += (A + B) +- i (A - B)
+    {
+      cx<R> x0[12];
+      load_spinor<R>(psi, s, x0);
       Half<R> a, b, A, B;
 #pragma unroll
       for (int q = 0; q < 2; ++q)
@@ -189,21 +280,14 @@ __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(const cx<R>* __res
       for (int q = 0; q < 2; ++q)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          cx<R> P = A.v[q][k] + B.v[q][k], Q = A.v[q][k] - B.v[q][k];
-          ap.v[q][k] = P + ti(Q);
-          am.v[q][k] = P - ti(Q);
+          const cx<R> P = A.v[q][k] + B.v[q][k], Q = A.v[q][k] - B.v[q][k];
+          ap.v[q][k] = ap.v[q][k] + (P + ti(Q));
+          am.v[q][k] = am.v[q][k] + (P - ti(Q));
         }
     }
     hop_spatial<R, 0>(W, psi, c, g, s, ap, am);
     hop_spatial<R, 1>(W, psi, c, g, s, ap, am);
     hop_spatial<R, 2>(W, psi, c, g, s, ap, am);
-    hop_time<R>(W, psi, c, g, s, ap, am);
-    hop_two<R, 0>(W, psi, c, g, s, a_ii, b_ii, ap, am);
-    hop_two<R, 1>(W, psi, c, g, s, a_ii, b_ii, ap, am);
-    hop_two<R, 2>(W, psi, c, g, s, a_ii, b_ii, ap, am);
-    hop_diag<R, 0, 1, 0>(W, psi, c, g, s, ap, am);
-    hop_diag<R, 0, 2, 1>(W, psi, c, g, s, ap, am);
-    hop_diag<R, 1, 2, 2>(W, psi, c, g, s, ap, am);
 
     cx<R> o[12];
 #pragma unroll
@@ -235,6 +319,8 @@ __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(const cx<R>* __res
       red[0] = d.re;
       red[1] = d.im;
     } else if constexpr (EPI == EPI_TS) {
+      cx<R> x0[12];
+      load_spinor<R>(psi, s, x0);
       cx<R> d = mk<R>(0, 0);
       R n2 = 0;
 #pragma unroll
@@ -781,8 +867,12 @@ static void launch_variant(const cx<R>* W, const cx<R>* psi, cx<R>* out, const G
   }
   else if constexpr (v == 1)
     apply_pair_kernel<R, EPI><<<grid_for(2LL * g.V, APPLY_THREADS), APPLY_THREADS, 0, st>>>(W, psi, out, g, c0q, a, b, ep);
-  else
-    apply_kernel<R, EPI><<<grid_for(g.V, APPLY_THREADS), APPLY_THREADS, 0, st>>>(W, psi, out, g, c0q, a, b, ep);
+  else {
+    const bool a_big = fabs(a) >= fabs(b);
+    const R big = a_big ? a : b, small = a_big ? b : a;
+    const TwoHop<R> two{big, big != R(0) ? small / big : R(0), a_big};
+    apply_kernel<R, EPI><<<grid_for(g.V, APPLY_THREADS), APPLY_THREADS, 0, st>>>(W, psi, out, g, c0q, two, ep);
+  }
 }
 
 template <typename R>
