@@ -283,14 +283,16 @@ ok_solve_params ok_default_solve_params(double tol, int maxiter);
 int ok_true_residual(const ok_W* W, const void* b, const void* x, double* relres, void* stream);
 
 /* Inspection: one application of M with the fused inner products that a BiCGStab half-iteration
- * takes from it (the paper's bi-stabilized CG, Sec. 2.3; van der Vorst 1992): the launch the
- * solver runs for v = M p (kind OK_REDUCE_DOT) and for t = M s (kind OK_REDUCE_TS).
+ * takes from it (the paper's bi-stabilized CG, Sec. 2.3; van der Vorst 1992), as the solver runs
+ * them for v = M p (kind OK_REDUCE_DOT) and for t = M s (kind OK_REDUCE_TS): one fused launch in
+ * FP64, the application and a pass of inner products in FP32.
  *   out = M psi, and
  *   OK_REDUCE_DOT: sums[0] + i sums[1] = <y, M psi> = sum conj(y) (M psi); sums[2] = 0;
  *   OK_REDUCE_TS:  sums[0] + i sums[1] = <M psi, y>, sums[2] = |M psi|^2.
  * prec OK_F64 (complex128 fields, OK_W_F64; OK_REDUCE_TS then needs y == psi), OK_F32 (complex64,
  * OK_W_F32) or OK_F32_W16 (complex64, OK_W_F16).  psi, y, out: device [V][4][3]; out must not
- * overlap psi or y; sums: host, 3 doubles.  The partial sums are FP64 and summed in a fixed order.
+ * overlap psi or y; sums: host, 3 doubles.  The partial sums are FP64
+ * (FP32 fields: FP32 chunks of a few elements, then double-float) and summed in a fixed order.
  * Allocates stream-ordered scratch and synchronises `stream`.
  * Errors: OK_EINVAL (null or misaligned pointers, overlap, a missing copy, an unknown kind),
  * OK_ENOMEM, OK_ECUDA. */

@@ -341,162 +341,32 @@ __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(const cx<R>* __res
   }
 }
 
-#ifndef OK_APPLY_MINB
-#define OK_APPLY_MINB 1
-#endif
-
-template <typename R, int EPI>
-__global__ void __launch_bounds__(APPLY_THREADS, OK_APPLY_MINB) apply_pair_kernel(const cx<R>* __restrict__ W, const cx<R>* __restrict__ psi,
-                                                                   cx<R>* __restrict__ out, Geom g, R c0q, R a_ii, R b_ii,
-                                                                   EpiArgs<R> ep) {
-  if (ep.halt && *ep.halt) return;
-  const int tid = blockIdx.x * APPLY_THREADS + threadIdx.x;
-  const int s = tid >> 1;
-  Pair pr;
-  pr.p = threadIdx.x & 1;
-  pr.mask = 3u << (threadIdx.x & 30);
-  double red[3] = {0.0, 0.0, 0.0};
-  if (s < g.V) {
-    int c[4];
-    {
-      int r = s;
-      c[0] = r % g.L[0]; r /= g.L[0];
-      c[1] = r % g.L[1]; r /= g.L[1];
-      c[2] = r % g.L[2]; c[3] = r / g.L[2];
-    }
-    H6<R> acc;
-    {
-      // on-site: p = 0 forms A = Y+ (u - i l), p = 1 forms B = Y- (u + i l); acc = (A + B) + i (A - B)
-      // for p = 0 and (A + B) - i (A - B) for p = 1, i.e. acc = (R + Rp) + i (R - Rp) for both.
-      H6<R> mine, oth, v, Rm;
-      load_half<R>(psi, s, pr.p, mine);
-      oth = partner(mine, pr.mask);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          cx<R> u = pr.p ? oth.v[q][k] : mine.v[q][k];
-          cx<R> l = pr.p ? mine.v[q][k] : oth.v[q][k];
-          v.v[q][k] = pr.p ? u + ti(l) : u - ti(l);
-          Rm.v[q][k] = c0q * v.v[q][k];
-        }
-      const int m0 = pr.p ? M_Y0M : M_Y0P;
-      M3<R> y = wmat(W, s, m0 + 0);
-      mv_add(Rm.v[0], y, v.v[0]); mv_sub(Rm.v[1], y, v.v[1]);
-      y = wmat(W, s, m0 + 1);
-      mv_add(Rm.v[0], y, v.v[1]);
-      y = wmat(W, s, m0 + 2);
-      mv_add(Rm.v[1], y, v.v[0]);
-      H6<R> Rp = partner(Rm, pr.mask);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) acc.v[q][k] = (Rm.v[q][k] + Rp.v[q][k]) + ti(Rm.v[q][k] - Rp.v[q][k]);
-    }
-    const GlobalW<R> Wg{W};
-    pair_spatial<R, 0>(Wg, psi, c, g, s, pr, acc);
-    pair_spatial<R, 1>(Wg, psi, c, g, s, pr, acc);
-    pair_spatial<R, 2>(Wg, psi, c, g, s, pr, acc);
-    pair_time<R>(Wg, psi, c, g, s, pr, acc);
-    pair_two<R, 0>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-    pair_two<R, 1>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-    pair_two<R, 2>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-    pair_diag<R, 0, 1, 0>(Wg, psi, c, g, s, pr, acc);
-    pair_diag<R, 0, 2, 1>(Wg, psi, c, g, s, pr, acc);
-    pair_diag<R, 1, 2, 2>(Wg, psi, c, g, s, pr, acc);
-
-    // out_u = acc+ + acc- (p = 0 writes it), out_l = acc+ - acc- (p = 1)
-    H6<R> ap = partner(acc, pr.mask), o;
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) o.v[q][k] = pr.p ? ap.v[q][k] - acc.v[q][k] : acc.v[q][k] + ap.v[q][k];
-    if (EPI == EPI_RESID) {
-      H6<R> bv;
-      load_half<R>(ep.b, s, pr.p, bv);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          o.v[q][k] = bv.v[q][k] - o.v[q][k];
-          red[0] += (double)o.v[q][k].re * o.v[q][k].re + (double)o.v[q][k].im * o.v[q][k].im;
-          red[1] += (double)bv.v[q][k].re * bv.v[q][k].re + (double)bv.v[q][k].im * bv.v[q][k].im;
-        }
-    }
-    store_half<R>(out, s, pr.p, o);
-    if (EPI == EPI_DOT) {
-      H6<R> rh;
-      load_half<R>(ep.rhat, s, pr.p, rh);
-      cx<R> d = mk<R>(0, 0);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) d = fma_cj(rh.v[q][k], o.v[q][k], d);
-      red[0] = d.re;
-      red[1] = d.im;
-    } else if (EPI == EPI_TS) {
-      H6<R> x0;
-      load_half<R>(psi, s, pr.p, x0);
-      cx<R> d = mk<R>(0, 0);
-      R n2 = 0;
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          d = fma_cj(o.v[q][k], x0.v[q][k], d);
-          n2 += o.v[q][k].re * o.v[q][k].re + o.v[q][k].im * o.v[q][k].im;
-        }
-      red[0] = d.re;
-      red[1] = d.im;
-      red[2] = n2;
-    }
-  }
-  if (EPI == EPI_DOT || EPI == EPI_RESID) {
-    double v2[2] = {red[0], red[1]};
-    grid_reduce<2, APPLY_THREADS>(v2, ep.ra, ep.ticket);
-  } else if (EPI == EPI_TS) {
-    grid_reduce<3, APPLY_THREADS>(red, ep.ra, ep.ticket);
-  }
-}
-
-// ============================================================================ split kernel
-// A block of 128 threads covers 32 sites.  Warps 0-1 (thread pairs as above) do the on-site term
-// and the 13 forward hops, warps 2-3 the 13 backward hops of the same sites; the backward half
-// hands its partial sums over through shared memory.  Each thread's chain of dependent
-// load-then-multiply rounds is half as long as in the pair kernel, so twice as many global loads
-// are in flight per resident site.
+// ============================================================================ staged split kernel
+// FP32 arithmetic, the alternative to the pipelined kernel of ok_apply_pipe.cu that ok_autotune times
+// (and ok_set_launch_shape pins).  A block of 128 threads covers 32 sites.  Warps 0-1 (thread pairs as in
+// ok_pair.cuh) do the on-site term and the 13 forward hops, warps 2-3 the 13 backward hops of the same
+// sites; the backward half hands its partial sums over through shared memory.
 //
-// Staged form (STAGED = true): the forward half reads its own tile's W record from shared memory.
-// The record of a 32-site tile is contiguous in the site-blocked layout, so the Tensor Memory
-// Accelerator streams it (cp.async.bulk: one thread issues, an mbarrier counts the bytes) in
-// NCHUNK chunks, one per group of hops, through OK_STAGES shared-memory slots.  The copy of chunk
-// q + OK_STAGES is issued as soon as both forward warps are done with chunk q, across the block's
-// tiles, so the DRAM stream of W is kept in flight by the copy engine instead of by registers.
-// The backward half gathers the neighbours' matrices with ordinary loads: the block that owns
-// that tile streamed them shortly before, so they are L2 hits.
+// The forward half reads its own tile's W record from shared memory.  The record of a 32-site tile is
+// contiguous in the site-blocked layout, so the Tensor Memory Accelerator streams it (cp.async.bulk:
+// one thread issues, an mbarrier counts the bytes) in NCHUNK chunks, one per group of hops, through
+// OK_STAGES shared-memory slots.  The copy of chunk q + OK_STAGES is issued as soon as both forward
+// warps are done with chunk q, across the block's tiles, so the DRAM stream of W is kept in flight by
+// the copy engine instead of by registers.  The backward half gathers the neighbours' matrices with
+// ordinary loads: the block that owns that tile streamed them shortly before, so they are L2 hits.
 constexpr int SPLIT_THREADS = 128;
 constexpr int SPLIT_SITES = 32;
 static_assert(SPLIT_SITES == LANES, "a tile is one site block of the W layout");
 
-// 4 resident blocks per SM (128 registers per thread): measured best on 16^3 x 32 for the
-// unstaged form (102 us against 119 us with 2 blocks and 117 us with 5).
-#ifndef OK_SPLIT_MINB
-#define OK_SPLIT_MINB 4
-#endif
-// Resident blocks for the variants with a fused reduction (they hold a few more live values).
-#ifndef OK_SPLIT_MINB_EPI
-#define OK_SPLIT_MINB_EPI 4
-#endif
-
 #ifndef OK_STAGES
 #define OK_STAGES 2
 #endif
-constexpr int NCHUNK = 7;     // W0 | W+t | W+x | W+y | W+z | W++ii | W++ij, W+-ij
+constexpr int NCHUNK = 7;     // W+t | W++ii | W++ij, W+-ij | W0 | W+x | W+y | W+z (the order of use)
 constexpr int CHUNK_MAX = 8;  // matrices in the largest chunk
 __device__ __forceinline__ int chunk_first(int c) {
-  return c == 0 ? M_Y0P : c == 1 ? M_UT : c == 5 ? M_VII : c == 6 ? M_VIJ : M_WP + 8 * (c - 2);
+  return c == 0 ? M_UT : c == 1 ? M_VII : c == 2 ? M_VIJ : c == 3 ? M_Y0P : M_WP + 8 * (c - 4);
 }
-__device__ __forceinline__ int chunk_count(int c) { return c == 0 ? 6 : c == 1 ? 4 : c == 5 ? 3 : c == 6 ? 6 : 8; }
+__device__ __forceinline__ int chunk_count(int c) { return c == 0 ? 4 : c == 1 ? 3 : c == 2 || c == 3 ? 6 : 8; }
 // A staged matrix occupies its own 9 x 32 elements plus 16 bytes: the two threads of a pair read
 // matrices 4 apart, which this shift puts in different shared-memory banks.
 template <typename WT> constexpr int smat_elems() { return 9 * LANES + 16 / (int)sizeof(cx<WT>); }
@@ -555,20 +425,28 @@ template <typename WT> struct StagedW {
   const cx<WT>* slot;
   int m0;
   __device__ __forceinline__ M3<typename WReal<WT>::type> operator()(int site, int m) const {
-    const cx<WT>* q = slot + (m - m0) * smat_elems<WT>() + (site & (LANES - 1));
+    const cx<WT>* q = slot + (m - m0) * smat_elems<WT>();
+    const int l = site & (LANES - 1);
     M3<typename WReal<WT>::type> a;
+    if constexpr (std::is_same<WT, __half>::value) {
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      if constexpr (std::is_same<WT, __half>::value) {
-        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(q + e * LANES));
-        a.e[e] = mk<float>(f.x, f.y);
-      } else if constexpr (std::is_same<WT, float>::value) {
-        const float2 f = *reinterpret_cast<const float2*>(q + e * LANES);
-        a.e[e] = mk<float>(f.x, f.y);
-      } else {
-        const double2 f = *reinterpret_cast<const double2*>(q + e * LANES);
-        a.e[e] = mk<double>(f.x, f.y);
+      for (int k = 0; k < 2; ++k) {
+        const uint4 u = reinterpret_cast<const uint4*>(q)[k * LANES + l];
+        a.e[4 * k] = widen(u.x);
+        a.e[4 * k + 1] = widen(u.y);
+        a.e[4 * k + 2] = widen(u.z);
+        a.e[4 * k + 3] = widen(u.w);
       }
+      a.e[8] = widen(reinterpret_cast<const unsigned*>(q)[8 * LANES + l]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 f = reinterpret_cast<const float4*>(q)[k * LANES + l];
+        a.e[2 * k] = mk<float>(f.x, f.y);
+        a.e[2 * k + 1] = mk<float>(f.z, f.w);
+      }
+      const float2 f = reinterpret_cast<const float2*>(q)[8 * LANES + l];
+      a.e[8] = mk<float>(f.x, f.y);
     }
     return a;
   }
@@ -605,18 +483,18 @@ __device__ __forceinline__ void issue_chunk(const cx<WT>* __restrict__ W, cx<WT>
              W + ((size_t)tile * NMAT + m0 + j) * (9 * LANES), mbytes, &full[slot]);
 }
 
-template <typename R, int EPI, typename WT, bool STAGED>
-__global__ void __launch_bounds__(SPLIT_THREADS, EPI == EPI_NONE ? OK_SPLIT_MINB : OK_SPLIT_MINB_EPI) apply_split_kernel(const cx<WT>* __restrict__ W, const cx<R>* __restrict__ psi,
-                                                                                   cx<R>* __restrict__ out, Geom g, R c0q, R a_ii, R b_ii,
-                                                                                   EpiArgs<R> ep) {
-  if (ep.halt && *ep.halt) return;
-  // Persistent: each block walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...  The hand-off buffer
-  // is double-buffered by tile parity, so one barrier per tile suffices: the backward half writes
+template <typename WT>
+__global__ void __launch_bounds__(SPLIT_THREADS, 4)
+    apply_staged_kernel(const cx<WT>* __restrict__ W, const cx<float>* __restrict__ psi, cx<float>* __restrict__ out, Geom g,
+                        float c0q, float a_ii, float b_ii, const int* halt) {
+  using R = float;
+  if (halt && *halt) return;
+  // Persistent: each block walks tiles rank, rank + gridDim.x, ...  The hand-off buffer is
+  // double-buffered by tile parity, so one barrier per tile suffices: the backward half writes
   // buffer k & 1 for tile k only after the barrier of tile k - 1, which the forward half passes
   // only after it has read buffer (k - 2) & 1 = k & 1.
   __shared__ cx<R> xch[2][64][6];
-  __shared__ __align__(16) cx<R> xev[EPI == EPI_NONE ? 1 : 2][64][6];
-  __shared__ __align__(8) unsigned long long full[STAGED ? OK_STAGES : 1];
+  __shared__ __align__(8) unsigned long long full[OK_STAGES];
   extern __shared__ __align__(128) unsigned char stage_raw[];
   cx<WT>* stage = reinterpret_cast<cx<WT>*>(stage_raw);
   const int half = threadIdx.x >> 6;  // warp-uniform: 0 forward, 1 backward
@@ -625,12 +503,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, EPI == EPI_NONE ? OK_SPLIT_MINB
   pr.p = t & 1;
   pr.mask = 3u << (threadIdx.x & 30);
   const GlobalW<WT> Wg{W};
-  // Per-thread partial sums over this thread's few sites stay in the field's precision (fewer
-  // registers); the block and grid reductions that follow are FP64.
-  R red[3] = {0, 0, 0};
   const int ntiles = (g.V + SPLIT_SITES - 1) / SPLIT_SITES;
   const int rank = tile_rank(g.sms);
-  const int nq = (STAGED && rank < ntiles) ? ((ntiles - 1 - rank) / (int)gridDim.x + 1) * NCHUNK : 0;
+  const int nq = rank < ntiles ? ((ntiles - 1 - rank) / (int)gridDim.x + 1) * NCHUNK : 0;
   int qc = 0;  // next chunk (forward warps)
   bool staged_ok = true;
   // Failure path: a wait that runs out sets stage_abort; no further chunk is issued, the block
@@ -639,16 +514,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS, EPI == EPI_NONE ? OK_SPLIT_MINB
   // copy is in flight when the block exits.
   __shared__ int stage_abort;
   int issued = 0, unwaited_from = -1;
-  if constexpr (STAGED) {
-    if (threadIdx.x == 0) {
-      for (int k = 0; k < OK_STAGES; ++k) mbar_init(&full[k], 1);
-      mbar_fence_init();
-      stage_abort = 0;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (; issued < OK_STAGES && issued < nq; ++issued) issue_chunk<WT>(W, stage, full, issued, rank);
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < OK_STAGES; ++k) mbar_init(&full[k], 1);
+    mbar_fence_init();
+    stage_abort = 0;
   }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (; issued < OK_STAGES && issued < nq; ++issued) issue_chunk<WT>(W, stage, full, issued, rank);
   // Wait for chunk qc; the forward warps then read it through a StagedW.
   auto chunk = [&](int m0) {
     const int slot = qc % OK_STAGES;
@@ -687,72 +560,51 @@ __global__ void __launch_bounds__(SPLIT_THREADS, EPI == EPI_NONE ? OK_SPLIT_MINB
     c[2] = r % g.L[2]; c[3] = r / g.L[2];
   }
   if (half == 0) {
-    if constexpr (STAGED) {
-      // Every forward thread takes part in the waits and barriers, active or not.
-      { auto w = chunk(M_Y0P); if (active) pair_onsite<R>(w, psi, s, pr, c0q, acc); release(); }
-      { auto w = chunk(M_UT); if (active) pair_time<R, true, false>(w, psi, c, g, s, pr, acc); release(); }
-      { auto w = chunk(M_WP + 0); if (active) pair_spatial<R, 0, true, false>(w, psi, c, g, s, pr, acc); release(); }
-      { auto w = chunk(M_WP + 8); if (active) pair_spatial<R, 1, true, false>(w, psi, c, g, s, pr, acc); release(); }
-      { auto w = chunk(M_WP + 16); if (active) pair_spatial<R, 2, true, false>(w, psi, c, g, s, pr, acc); release(); }
-      {
-        auto w = chunk(M_VII);
-        if (active) {
-          pair_two<R, 0, true, false>(w, psi, c, g, s, pr, a_ii, b_ii, acc);
-          pair_two<R, 1, true, false>(w, psi, c, g, s, pr, a_ii, b_ii, acc);
-          pair_two<R, 2, true, false>(w, psi, c, g, s, pr, a_ii, b_ii, acc);
-        }
-        release();
+    Halves<R> hs;
+    zero_halves(hs);
+    // Every forward thread takes part in the waits and barriers, active or not.
+    { auto w = chunk(M_UT); if (active) pair_time<R, true, true>(w, psi, c, g, s, pr, hs); release(); }
+    {
+      auto w = chunk(M_VII);
+      if (active) {
+        pair_two<R, 0, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
+        pair_two<R, 1, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
+        pair_two<R, 2, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
       }
-      {
-        auto w = chunk(M_VIJ);
-        if (active) {
-          pair_diag<R, 0, 1, 0, true, false>(w, psi, c, g, s, pr, acc);
-          pair_diag<R, 0, 2, 1, true, false>(w, psi, c, g, s, pr, acc);
-          pair_diag<R, 1, 2, 2, true, false>(w, psi, c, g, s, pr, acc);
-        }
-        release();
-      }
-    } else if (active) {
-      pair_onsite<R>(Wg, psi, s, pr, c0q, acc);
-      pair_spatial<R, 0, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_spatial<R, 1, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_spatial<R, 2, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_time<R, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_two<R, 0, true, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_two<R, 1, true, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_two<R, 2, true, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_diag<R, 0, 1, 0, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_diag<R, 0, 2, 1, true, false>(Wg, psi, c, g, s, pr, acc);
-      pair_diag<R, 1, 2, 2, true, false>(Wg, psi, c, g, s, pr, acc);
+      release();
     }
-  } else if (active) {
-      // The epilogue's own half-spinor (rhat, b, or the y of <out, y>) is copied into shared memory
-      // asynchronously (cp.async, no registers held) while this half works through its hops.
-      if constexpr (EPI != EPI_NONE) {
-        const cx<R>* src = EPI == EPI_DOT ? ep.rhat : EPI == EPI_RESID ? ep.b : (ep.rhat ? ep.rhat : psi);
-        const char* gsrc = reinterpret_cast<const char*>(src + (size_t)s * 12 + 6 * pr.p);
-        char* dst = reinterpret_cast<char*>(&xev[kb][t][0]);
-#pragma unroll
-        for (int k = 0; k < (int)(6 * sizeof(cx<R>)) / 16; ++k)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst + 16 * k)), "l"(gsrc + 16 * k)
-                       : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    {
+      auto w = chunk(M_VIJ);
+      if (active) {
+        pair_diag<R, 0, 1, 0, true, true>(w, psi, c, g, s, pr, hs);
+        pair_diag<R, 0, 2, 1, true, true>(w, psi, c, g, s, pr, hs);
+        pair_diag<R, 1, 2, 2, true, true>(w, psi, c, g, s, pr, hs);
+        to_h(hs, pr, acc);
       }
-      pair_spatial<R, 0, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_spatial<R, 1, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_spatial<R, 2, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_time<R, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_two<R, 0, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_two<R, 1, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_two<R, 2, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, acc);
-      pair_diag<R, 0, 1, 0, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_diag<R, 0, 2, 1, false, true>(Wg, psi, c, g, s, pr, acc);
-      pair_diag<R, 1, 2, 2, false, true>(Wg, psi, c, g, s, pr, acc);
+      release();
+    }
+    { auto w = chunk(M_Y0P); if (active) pair_onsite<R>(w, psi, s, pr, c0q, acc); release(); }
+    { auto w = chunk(M_WP + 0); if (active) pair_spatial<R, 0, true, true>(w, psi, c, g, s, pr, acc); release(); }
+    { auto w = chunk(M_WP + 8); if (active) pair_spatial<R, 1, true, true>(w, psi, c, g, s, pr, acc); release(); }
+    { auto w = chunk(M_WP + 16); if (active) pair_spatial<R, 2, true, true>(w, psi, c, g, s, pr, acc); release(); }
+  } else if (active) {
+    Halves<R> hs;
+    zero_halves(hs);
+    pair_time<R, false, true>(Wg, psi, c, g, s, pr, hs);
+    pair_two<R, 0, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_two<R, 1, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_two<R, 2, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_diag<R, 0, 1, 0, false, true>(Wg, psi, c, g, s, pr, hs);
+    pair_diag<R, 0, 2, 1, false, true>(Wg, psi, c, g, s, pr, hs);
+    pair_diag<R, 1, 2, 2, false, true>(Wg, psi, c, g, s, pr, hs);
+    to_h(hs, pr, acc);
+    pair_spatial<R, 0, false, true>(Wg, psi, c, g, s, pr, acc);
+    pair_spatial<R, 1, false, true>(Wg, psi, c, g, s, pr, acc);
+    pair_spatial<R, 2, false, true>(Wg, psi, c, g, s, pr, acc);
 #pragma unroll
-      for (int qq = 0; qq < 2; ++qq)
+    for (int qq = 0; qq < 2; ++qq)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) xch[kb][t][3 * qq + k] = acc.v[qq][k];
-      if constexpr (EPI != EPI_NONE) asm volatile("cp.async.wait_all;" ::: "memory");
+      for (int k = 0; k < 3; ++k) xch[kb][t][3 * qq + k] = acc.v[qq][k];
   }
   __syncthreads();
   if (half == 0 && active) {
@@ -761,89 +613,28 @@ __global__ void __launch_bounds__(SPLIT_THREADS, EPI == EPI_NONE ? OK_SPLIT_MINB
 #pragma unroll
       for (int k = 0; k < 3; ++k) acc.v[q][k] = acc.v[q][k] + xch[kb][t][3 * q + k];
     // out_u = acc+ + acc- (p = 0 writes it), out_l = acc+ - acc- (p = 1)
-    H6<R> ap = partner(acc, pr.mask), o, ev;
+    H6<R> ap = partner(acc, pr.mask), o;
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        o.v[q][k] = pr.p ? ap.v[q][k] - acc.v[q][k] : acc.v[q][k] + ap.v[q][k];
-        if (EPI != EPI_NONE) ev.v[q][k] = xev[kb][t][3 * q + k];
-      }
-    if (EPI == EPI_RESID) {
-      const H6<R>& bv = ev;
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          o.v[q][k] = bv.v[q][k] - o.v[q][k];
-          red[0] += (double)o.v[q][k].re * o.v[q][k].re + (double)o.v[q][k].im * o.v[q][k].im;
-          red[1] += (double)bv.v[q][k].re * bv.v[q][k].re + (double)bv.v[q][k].im * bv.v[q][k].im;
-        }
-    }
+      for (int k = 0; k < 3; ++k) o.v[q][k] = pr.p ? ap.v[q][k] - acc.v[q][k] : acc.v[q][k] + ap.v[q][k];
     store_half<R>(out, s, pr.p, o);
-    if (EPI == EPI_DOT) {
-      const H6<R>& rh = ev;
-      cx<R> d = mk<R>(0, 0);
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) d = fma_cj(rh.v[q][k], o.v[q][k], d);
-      red[0] += d.re;
-      red[1] += d.im;
-    } else if (EPI == EPI_TS) {
-      const H6<R>& x0 = ev;
-      cx<R> d = mk<R>(0, 0);
-      R n2 = 0;
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          d = fma_cj(o.v[q][k], x0.v[q][k], d);
-          n2 += o.v[q][k].re * o.v[q][k].re + o.v[q][k].im * o.v[q][k].im;
-        }
-      red[0] += d.re;
-      red[1] += d.im;
-      red[2] += n2;
-    }
   }
   }  // tiles
-  if constexpr (STAGED) {
-    if (threadIdx.x == 0 && unwaited_from >= 0)
-      for (int q = unwaited_from; q < issued; ++q) mbar_wait(&full[q % OK_STAGES], (q / OK_STAGES) & 1, 1LL << 24, false);
-  }
-  if (EPI == EPI_DOT || EPI == EPI_RESID) {
-    double v2[2] = {(double)red[0], (double)red[1]};
-    grid_reduce<2, SPLIT_THREADS>(v2, ep.ra, ep.ticket);
-  } else if (EPI == EPI_TS) {
-    double v3[3] = {(double)red[0], (double)red[1], (double)red[2]};
-    grid_reduce<3, SPLIT_THREADS>(v3, ep.ra, ep.ticket);
-  }
+  if (threadIdx.x == 0 && unwaited_from >= 0)
+    for (int q = unwaited_from; q < issued; ++q) mbar_wait(&full[q % OK_STAGES], (q / OK_STAGES) & 1, 1LL << 24, false);
 }
 
 // ---------------------------------------------------------------------------- launchers
-// Kernel variant per precision: 0 = one thread per site, 1 = thread pair per site, 2 = split
-// (forward and backward halves in different warps).  FP64 is bound by the FP64 pipe, where one
-// thread per site does the least arithmetic; FP32 is bound by memory latency, where the split
-// kernel keeps the most loads in flight.
-#ifndef OK_APPLY64_VARIANT
-#define OK_APPLY64_VARIANT 0
-#endif
-#ifndef OK_APPLY32_VARIANT
-#define OK_APPLY32_VARIANT 2
-#endif
-template <typename R> constexpr int apply_variant() { return sizeof(R) == 8 ? OK_APPLY64_VARIANT : OK_APPLY32_VARIANT; }
-
-// Persistent grid of the split kernel: as many blocks as fit on the device at once (from the
-// occupancy calculator for this instantiation and its dynamic shared memory), at most one per tile.
-template <typename R, int EPI, typename WT, bool STAGED>
-static void launch_split(const cx<WT>* W, const cx<R>* psi, cx<R>* out, const Geom& g, R c0q, R a, R b,
-                         const EpiArgs<R>& ep, cudaStream_t st) {
+// Persistent grid: as many blocks as fit on the device at once, at most one per tile.
+template <typename WT>
+static void launch_staged(const cx<WT>* W, const cx<float>* psi, cx<float>* out, const Geom& g, float c0q, float a, float b,
+                          const int* halt, cudaStream_t st) {
   static int resident = 0;
-  const size_t dyn = STAGED ? staged_smem<WT>() : 0;
-  auto kern = apply_split_kernel<R, EPI, WT, STAGED>;
+  const size_t dyn = staged_smem<WT>();
+  auto kern = apply_staged_kernel<WT>;
   if (resident == 0) {
-    // Static plus dynamic shared memory above 48 KB needs the opt-in (the FP32 reducing variants).
-    if (dyn > 0) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, SPLIT_THREADS, dyn) != cudaSuccess || nb < 1) nb = 1;
     resident = nb * sm_count();
@@ -851,27 +642,31 @@ static void launch_split(const cx<WT>* W, const cx<R>* psi, cx<R>* out, const Ge
   const int tiles = grid_for(g.V, SPLIT_SITES);
   Geom gs = g;
   gs.sms = sm_count();
-  kern<<<tiles < resident ? tiles : resident, SPLIT_THREADS, dyn, st>>>(W, psi, out, gs, c0q, a, b, ep);
+  kern<<<tiles < resident ? tiles : resident, SPLIT_THREADS, dyn, st>>>(W, psi, out, gs, c0q, a, b, halt);
 }
 
-// The split kernel streams the forward W through shared memory by TMA when the handle's tuning
-// record says so (ok_autotune); the default reads it with ordinary loads, which measured faster
-// on 16^3 x 32 (the staging slots take L1 capacity that the neighbour spinors use).
-template <typename R, int EPI>
-static void launch_variant(const cx<R>* W, const cx<R>* psi, cx<R>* out, const Geom& g, R c0q, R a, R b,
-                           const EpiArgs<R>& ep, bool staged, cudaStream_t st) {
-  constexpr int v = apply_variant<R>();
-  if constexpr (v == 2) {
-    if (staged) launch_split<R, EPI, R, true>(W, psi, out, g, c0q, a, b, ep, st);
-    else launch_split<R, EPI, R, false>(W, psi, out, g, c0q, a, b, ep, st);
-  }
-  else if constexpr (v == 1)
-    apply_pair_kernel<R, EPI><<<grid_for(2LL * g.V, APPLY_THREADS), APPLY_THREADS, 0, st>>>(W, psi, out, g, c0q, a, b, ep);
-  else {
-    const bool a_big = fabs(a) >= fabs(b);
-    const R big = a_big ? a : b, small = a_big ? b : a;
-    const TwoHop<R> two{big, big != R(0) ? small / big : R(0), a_big};
-    apply_kernel<R, EPI><<<grid_for(g.V, APPLY_THREADS), APPLY_THREADS, 0, st>>>(W, psi, out, g, c0q, two, ep);
+// The staged form runs when the handle's tuning record says so (ok_autotune); the default, the
+// pipelined kernel, reads W with ordinary loads (16^3 x 32: 92 us against 128 us staged, whose slots take
+// L1 capacity that the neighbour spinors use).
+template <typename WT>
+static void launch_f32(const cx<WT>* W, const cx<float>* psi, cx<float>* out, const Geom& g, float c0q, float a, float b,
+                       const int* halt, bool staged, cudaStream_t st) {
+  if (staged) launch_staged<WT>(W, psi, out, g, c0q, a, b, halt, st);
+  else launch_pipe<WT>(W, psi, out, g, c0q, a, b, halt, st);
+}
+
+static void launch_f64(const cx<double>* W, const cx<double>* psi, cx<double>* out, const Geom& g, const WScalars& sc, int epi,
+                       const EpiArgs<double>& ep, cudaStream_t st) {
+  const double a = sc.a_ii, b = sc.b_ii;
+  const bool a_big = fabs(a) >= fabs(b);
+  const double big = a_big ? a : b, small = a_big ? b : a;
+  const TwoHop<double> two{big, big != 0.0 ? small / big : 0.0, a_big};
+  const int nb = grid_for(g.V, APPLY_THREADS);
+  switch (epi) {
+    case EPI_NONE: apply_kernel<double, EPI_NONE><<<nb, APPLY_THREADS, 0, st>>>(W, psi, out, g, sc.c0q, two, ep); break;
+    case EPI_DOT: apply_kernel<double, EPI_DOT><<<nb, APPLY_THREADS, 0, st>>>(W, psi, out, g, sc.c0q, two, ep); break;
+    case EPI_TS: apply_kernel<double, EPI_TS><<<nb, APPLY_THREADS, 0, st>>>(W, psi, out, g, sc.c0q, two, ep); break;
+    default: apply_kernel<double, EPI_RESID><<<nb, APPLY_THREADS, 0, st>>>(W, psi, out, g, sc.c0q, two, ep); break;
   }
 }
 
@@ -879,20 +674,13 @@ template <typename R>
 int launch_apply(const ok_W* Wh, const cx<R>* psi, cx<R>* out, int epi, const EpiArgs<R>& ep, cudaStream_t st) {
   const cx<R>* W = (const cx<R>*)(sizeof(R) == 8 ? Wh->W64 : Wh->W32);
   if (!W) return OK_EINVAL;
-  if (epi < EPI_NONE || epi > EPI_RESID) return OK_EINVAL;
-  const Geom& g = Wh->g;
-  R c0q = (R)Wh->sc.c0q, a = (R)Wh->sc.a_ii, b = (R)Wh->sc.b_ii;
-  const bool stg = sizeof(R) == 4 && Wh->tune.staged[0] == 1;
+  // FP32: no fused epilogue (the inner products run in passes of their own, launch_dots)
+  if (epi < EPI_NONE || epi > (sizeof(R) == 8 ? EPI_RESID : EPI_NONE)) return OK_EINVAL;
   static const char* n64[4] = {"apply_f64", "apply_f64_dot", "apply_f64_ts", "apply_f64_resid"};
-  static const char* n32[4] = {"apply_f32", "apply_f32_dot", "apply_f32_ts", "apply_f32_resid"};
   {
-    TraceScope ts(sizeof(R) == 8 ? n64[epi] : n32[epi], st);
-    switch (epi) {
-      case EPI_NONE: launch_variant<R, EPI_NONE>(W, psi, out, g, c0q, a, b, ep, stg, st); break;
-      case EPI_DOT: launch_variant<R, EPI_DOT>(W, psi, out, g, c0q, a, b, ep, stg, st); break;
-      case EPI_TS: launch_variant<R, EPI_TS>(W, psi, out, g, c0q, a, b, ep, stg, st); break;
-      default: launch_variant<R, EPI_RESID>(W, psi, out, g, c0q, a, b, ep, stg, st); break;
-    }
+    TraceScope ts(sizeof(R) == 8 ? n64[epi] : "apply_f32", st);
+    if constexpr (sizeof(R) == 8) launch_f64(W, psi, out, Wh->g, Wh->sc, epi, ep, st);
+    else launch_f32<R>(W, psi, out, Wh->g, (R)Wh->sc.c0q, (R)Wh->sc.a_ii, (R)Wh->sc.b_ii, ep.halt, Wh->tune.staged[0] == 1, st);
   }
   OK_LAUNCH_CHECK();
   return OK_SUCCESS;
@@ -901,31 +689,14 @@ int launch_apply(const ok_W* Wh, const cx<R>* psi, cx<R>* out, int epi, const Ep
 // Upper bound of the grid size of any apply variant (sizes the reduction partials).
 int apply_blocks_needed(const ok_W* Wh) { return grid_for(Wh->g.V, SPLIT_SITES); }
 
-// FP32 fields and arithmetic with the half-precision copy of W (split kernel, all epilogues).
+// FP32 fields and arithmetic with the half-precision copy of W.
 int launch_apply_w16(const ok_W* Wh, const cx<float>* psi, cx<float>* out, int epi, const EpiArgs<float>& ep, cudaStream_t st) {
   const cx<__half>* W = (const cx<__half>*)Wh->W16;
-  if (!W) return OK_EINVAL;
-  if (epi < EPI_NONE || epi > EPI_RESID) return OK_EINVAL;
-  const Geom& g = Wh->g;
-  const float c0q = (float)Wh->sc.c0q, a = (float)Wh->sc.a_ii, b = (float)Wh->sc.b_ii;
-  static const char* names[4] = {"apply_w16", "apply_w16_dot", "apply_w16_ts", "apply_w16_resid"};
+  if (!W || epi != EPI_NONE) return OK_EINVAL;
   {
-    TraceScope ts(names[epi], st);
-    if (Wh->tune.staged[1] == 1) {
-      switch (epi) {
-        case EPI_NONE: launch_split<float, EPI_NONE, __half, true>(W, psi, out, g, c0q, a, b, ep, st); break;
-        case EPI_DOT: launch_split<float, EPI_DOT, __half, true>(W, psi, out, g, c0q, a, b, ep, st); break;
-        case EPI_TS: launch_split<float, EPI_TS, __half, true>(W, psi, out, g, c0q, a, b, ep, st); break;
-        default: launch_split<float, EPI_RESID, __half, true>(W, psi, out, g, c0q, a, b, ep, st); break;
-      }
-    } else {
-      switch (epi) {
-        case EPI_NONE: launch_split<float, EPI_NONE, __half, false>(W, psi, out, g, c0q, a, b, ep, st); break;
-        case EPI_DOT: launch_split<float, EPI_DOT, __half, false>(W, psi, out, g, c0q, a, b, ep, st); break;
-        case EPI_TS: launch_split<float, EPI_TS, __half, false>(W, psi, out, g, c0q, a, b, ep, st); break;
-        default: launch_split<float, EPI_RESID, __half, false>(W, psi, out, g, c0q, a, b, ep, st); break;
-      }
-    }
+    TraceScope ts("apply_w16", st);
+    launch_f32<__half>(W, psi, out, Wh->g, (float)Wh->sc.c0q, (float)Wh->sc.a_ii, (float)Wh->sc.b_ii, ep.halt,
+                       Wh->tune.staged[1] == 1, st);
   }
   OK_LAUNCH_CHECK();
   return OK_SUCCESS;

@@ -358,10 +358,10 @@ int launch_update_xr(cx<R>* x, const cx<R>* p, const cx<R>* s, const cx<R>* t, c
 }
 
 template <typename R>
-int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm) {
+int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm, int fin) {
   using T = typename Unit<R>::T;
   long long nu = units_of<R>(n);
-  RedArgs ra{st, part, nullptr, omega ? FIN_OMEGA : FIN_ALPHA};
+  RedArgs ra{st, part, nullptr, fin >= 0 ? fin : omega ? FIN_OMEGA : FIN_ALPHA};
   {
     TraceScope ts(omega ? (sizeof(R) == 8 ? "dots_ts_f64" : "dots_ts_f32") : (sizeof(R) == 8 ? "dot_rv_f64" : "dot_rv_f32"), strm);
     if (omega)
@@ -493,8 +493,8 @@ int launch_norms(const cx<double>* x, const cx<double>* b, long long n, SolverSt
 
 template int launch_update_s<double>(const cx<double>*, const cx<double>*, cx<double>*, long long, const SolverState*, cudaStream_t);
 template int launch_update_s<float>(const cx<float>*, const cx<float>*, cx<float>*, long long, const SolverState*, cudaStream_t);
-template int launch_dots<float>(const cx<float>*, const cx<float>*, long long, bool, SolverState*, double*, cudaStream_t);
-template int launch_dots<double>(const cx<double>*, const cx<double>*, long long, bool, SolverState*, double*, cudaStream_t);
+template int launch_dots<float>(const cx<float>*, const cx<float>*, long long, bool, SolverState*, double*, cudaStream_t, int);
+template int launch_dots<double>(const cx<double>*, const cx<double>*, long long, bool, SolverState*, double*, cudaStream_t, int);
 template int launch_update_xr<double>(cx<double>*, const cx<double>*, const cx<double>*, const cx<double>*, cx<double>*, const cx<double>*, long long, SolverState*, double*, cudaStream_t, const cx<double>*);
 template int launch_update_xr<float>(cx<float>*, const cx<float>*, const cx<float>*, const cx<float>*, cx<float>*, const cx<float>*, long long, SolverState*, double*, cudaStream_t, const cx<float>*);
 template int launch_update_p<double>(cx<double>*, const cx<double>*, const cx<double>*, long long, const SolverState*, cudaStream_t);

@@ -121,12 +121,20 @@ template <typename R> __host__ __device__ __forceinline__ M3<R> m_rscale(R s, co
 
 // ---------------------------------------------------------------------------- W layout
 // Per site the stored forward set is NMAT colour matrices (see ok_precompute.cu for the list).
-// Sites are grouped in blocks of 32 consecutive sites; within a block, element e (0..8) of
-// matrix m of the site in lane l lives at ((blk * NMAT + m) * 9 + e) * 32 + l, so a warp
-// handling 32 consecutive sites reads each element as one contiguous 32-wide row.
+// Sites are grouped in blocks of 32 consecutive sites; within a block, matrix m takes 9 x 32 elements
+// from (blk * NMAT + m) * 9 * 32 on.  Its elements lie in 16-byte words, the words of the 32 lanes side
+// by side: K = 16 / sizeof(element) elements of a lane per word (1 in FP64 and double-float, 2 in FP32, 4
+// in FP16), and the ninth element, where K does not divide 9, in a row of single elements at the end.
+// A lane reads a matrix with 5 loads in FP32 and 3 in FP16, where rows of single elements took 9
+// (six right-hand sides at 12^3 x 24: 146 us with rows, 137 us with words).
 constexpr int NMAT = 43;
 constexpr int LANES = 32;
 constexpr int SITE_ELEMS = NMAT * 9;   // complex numbers stored per site
+// Index of element e of lane l inside its matrix.
+template <typename WT> __host__ __device__ __forceinline__ constexpr int w_elem(int e, int l) {
+  constexpr int K = 16 / (int)sizeof(cx<WT>);
+  return e < 9 / K * K ? (e / K) * (K * LANES) + l * K + e % K : e * LANES + l;
+}
 
 // Matrix indices inside a site record.
 constexpr int M_Y0P = 0;    // 1/4 (D0 + c0 + i S0): blocks (00 minus c0/4 part) y3, (01), (10)

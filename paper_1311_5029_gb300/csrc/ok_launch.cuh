@@ -14,7 +14,7 @@ enum : int {
 };
 
 template <typename R> struct EpiArgs {
-  const cx<R>* rhat;   // EPI_DOT; EPI_TS (split kernel): if set, the y of <out, y> instead of psi
+  const cx<R>* rhat;   // EPI_DOT
   const cx<R>* b;      // EPI_RESID
   RedArgs ra;
   unsigned* ticket;
@@ -24,8 +24,12 @@ template <typename R> struct EpiArgs {
 template <typename R>
 int launch_apply(const ok_W* W, const cx<R>* psi, cx<R>* out, int epi, const EpiArgs<R>& ep, cudaStream_t st);
 int apply_blocks_needed(const ok_W* W);
-// FP32 fields and arithmetic with the half-precision W copy (all epilogues).
+// FP32 fields and arithmetic with the half-precision W copy (EPI_NONE, as FP32 applications all).
 int launch_apply_w16(const ok_W* W, const cx<float>* psi, cx<float>* out, int epi, const EpiArgs<float>& ep, cudaStream_t st);
+// out = M psi in FP32 arithmetic with the FP32 or FP16 W (ok_apply_pipe.cu); nothing when *halt is set.
+template <typename WT>
+void launch_pipe(const cx<WT>* W, const cx<float>* psi, cx<float>* out, const Geom& g, float c0q, float a, float b,
+                 const int* halt, cudaStream_t st);
 // out = M psi in FP32 with every W matrix rebuilt from the handle's FP32 links and clover fields
 // (OK_W_OTF) inside the apply; OK_EINVAL without them.
 int launch_apply_otf(const ok_W* W, const cx<float>* psi, cx<float>* out, cudaStream_t st);
@@ -95,9 +99,11 @@ int launch_update_xr(cx<R>* x, const cx<R>* p, const cx<R>* s, const cx<R>* t, c
                      SolverState* st, double* part, cudaStream_t strm, const cx<R>* sx = nullptr);
 template <typename R>
 int launch_update_p(cx<R>* p, const cx<R>* r, const cx<R>* v, long long n, const SolverState* st, cudaStream_t strm);
-// <a, b> -> FIN_ALPHA (a = rhat, b = v), or with omega <a, b>, <a, a> -> FIN_OMEGA (a = t, b = s).
+// <a, b> -> FIN_ALPHA (a = rhat, b = v), or with omega <a, b>, <a, a> -> FIN_OMEGA (a = t, b = s); fin >= 0:
+// that finalisation instead.
 template <typename R>
-int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm);
+int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm,
+                int fin = -1);
 template <typename R>
 int launch_restart(const cx<R>* r, cx<R>* rhat, cx<R>* p, long long n, SolverState* st, double* part, cudaStream_t strm);
 int launch_demote(const cx<double>* r64, cx<float>* r32, cx<float>* rhat, cx<float>* p, long long n, bool restart,

@@ -24,34 +24,6 @@ constexpr int MR_SITES = 32;
 
 template <int NR> constexpr int mr_minb() { return NR <= 2 ? 4 : 2; }
 
-// h' = sg h (sg = +1 for p = 0, -1 for p = 1), l' = sg l and u of the neighbour at offset D.
-template <typename R, int D0, int D1, int D2, int D3>
-__device__ __forceinline__ int gather_signed(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
-                                             H6<R>& h, H6<R>* u, H6<R>* l) {
-  bool neg;
-  const int n = nbr_site<D0, D1, D2, D3>(c, g, neg);
-  H6<R> mine;
-  load_half<R>(psi, n, pr.p, mine);
-  if (neg) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) mine.v[s][a] = -mine.v[s][a];
-  }
-  const H6<R> oth = partner(mine, pr.mask);
-  const R sg = pr.p ? R(-1) : R(1);
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const cx<R> m = mine.v[s][a], o = oth.v[s][a];
-      h.v[s][a] = mk<R>(m.re + sg * o.re, m.im + sg * o.im);  // p = 0: u + l;  p = 1: l - u = -(u - l)
-      if (u) u->v[s][a] = pr.p ? o : m;
-      if (l) l->v[s][a] = pr.p ? -m : o;
-    }
-  return n;
-}
-
 // acc_r += 2x2 spin blocks of matrices m .. m + 3 (or their adjoints) times h_r, r < NR.
 template <typename R, int NR, bool DAG, typename WS>
 __device__ __forceinline__ void mr_block2h(const WS& W, int site, int m, const H6<R> (&h)[NR], H6<R> (&acc)[NR]) {
@@ -69,128 +41,109 @@ __device__ __forceinline__ void mr_block2h(const WS& W, int site, int m, const H
   for (int r = 0; r < NR; ++r) { if (DAG) mdv_add(acc[r].v[1], b, h[r].v[1]); else mv_add(acc[r].v[1], b, h[r].v[1]); }
 }
 
-template <typename R, int NR, int I, bool FWD, typename WS>
+template <typename R, int NR, int I, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void mr_spatial(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
                                            const Geom& g, int s, const Pair& pr, H6<R> (&acc)[NR]) {
   const int base = M_WP + 8 * I;
   H6<R> h[NR];
   if constexpr (FWD) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) gather_pair<R, I == 0, I == 1, I == 2, 0>(psi + r * rs, c, g, pr, h[r]);
+    for (int r = 0; r < NR; ++r) gather_pair<R, I == 0, I == 1, I == 2, 0, AP>(psi + r * rs, c, g, pr, h[r]);
     mr_block2h<R, NR, false>(W, s, base + 4 * pr.p, h, acc);
   } else {
     int n = 0;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) n = gather_pair<R, -(I == 0), -(I == 1), -(I == 2), 0>(psi + r * rs, c, g, pr, h[r]);
+    for (int r = 0; r < NR; ++r) n = gather_pair<R, -(I == 0), -(I == 1), -(I == 2), 0, AP>(psi + r * rs, c, g, pr, h[r]);
     mr_block2h<R, NR, true>(W, n, base + 4 * (1 - pr.p), h, acc);
   }
 }
 
-// Temporal hop with the thread's sign folded into the gathered spinors (see pair_time):
-//   forward   acc0 += s3 h'0 + n1 h'1 - U l'0,   acc1 += -s3 h'1 + n2 h'0 - U l'1
-//   backward  acc0 -= s3^ h'0 + n2^ h'1 + U^ u0, acc1 += s3^ h'1 - n1^ h'0 - U^ u1   (^ = adjoint)
-template <typename R, int NR, bool FWD, typename WS>
+// The hops without exchange between the threads (see pair_time, pair_two, pair_diag): each matrix is
+// applied to the thread's own halves of NR right-hand sides.
+template <typename R, int NR, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void mr_time(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
-                                        const Geom& g, int s, const Pair& pr, H6<R> (&acc)[NR]) {
-  H6<R> h[NR], x[NR];
+                                        const Geom& g, int s, const Pair& pr, Halves<R> (&d)[NR]) {
+  H6<R> m[NR];
   if constexpr (FWD) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) gather_signed<R, 0, 0, 0, 1>(psi + r * rs, c, g, pr, h[r], nullptr, &x[r]);
+    for (int r = 0; r < NR; ++r) gather_mine<R, 0, 0, 0, 1, AP>(psi + r * rs, c, g, pr, m[r]);
     M3<R> A = W(s, M_ST + 0);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) { mv_add(acc[r].v[0], A, h[r].v[0]); mv_sub(acc[r].v[1], A, h[r].v[1]); }
+    for (int r = 0; r < NR; ++r) { mv_add(d[r].cross.v[0], A, m[r].v[0]); mv_sub(d[r].cross.v[1], A, m[r].v[1]); }
     A = W(s, M_ST + 1);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) mv_add(acc[r].v[0], A, h[r].v[1]);
+    for (int r = 0; r < NR; ++r) mv_add(d[r].cross.v[0], A, m[r].v[1]);
     A = W(s, M_ST + 2);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) mv_add(acc[r].v[1], A, h[r].v[0]);
+    for (int r = 0; r < NR; ++r) mv_add(d[r].cross.v[1], A, m[r].v[0]);
     A = W(s, M_UT);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) { mv_sub(acc[r].v[0], A, x[r].v[0]); mv_sub(acc[r].v[1], A, x[r].v[1]); }
+    for (int r = 0; r < NR; ++r) { only(m[r], pr.p == 1); mv_sub(d[r].same.v[0], A, m[r].v[0]); mv_sub(d[r].same.v[1], A, m[r].v[1]); }
   } else {
     int n = 0;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) n = gather_signed<R, 0, 0, 0, -1>(psi + r * rs, c, g, pr, h[r], &x[r], nullptr);
+    for (int r = 0; r < NR; ++r) n = gather_mine<R, 0, 0, 0, -1, AP>(psi + r * rs, c, g, pr, m[r]);
     M3<R> A = W(n, M_ST + 0);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) { mdv_sub(acc[r].v[0], A, h[r].v[0]); mdv_add(acc[r].v[1], A, h[r].v[1]); }
+    for (int r = 0; r < NR; ++r) { mdv_sub(d[r].cross.v[0], A, m[r].v[0]); mdv_add(d[r].cross.v[1], A, m[r].v[1]); }
     A = W(n, M_ST + 2);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) mdv_sub(acc[r].v[0], A, h[r].v[1]);
+    for (int r = 0; r < NR; ++r) mdv_sub(d[r].cross.v[0], A, m[r].v[1]);
     A = W(n, M_ST + 1);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) mdv_sub(acc[r].v[1], A, h[r].v[0]);
+    for (int r = 0; r < NR; ++r) mdv_sub(d[r].cross.v[1], A, m[r].v[0]);
     A = W(n, M_UT);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) { mdv_sub(acc[r].v[0], A, x[r].v[0]); mdv_sub(acc[r].v[1], A, x[r].v[1]); }
+    for (int r = 0; r < NR; ++r) { only(m[r], pr.p == 0); mdv_sub(d[r].same.v[0], A, m[r].v[0]); mdv_sub(d[r].same.v[1], A, m[r].v[1]); }
   }
 }
 
-// W^{++}_ii: acc+- += (a +- b sigma_i) V h+-  forward,  (a -+ b sigma_i) V^dag h+-  backward.
-template <typename R, int NR, int I, bool FWD, typename WS>
+template <typename R, int NR, int I, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void mr_two(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
-                                       const Geom& g, int s, const Pair& pr, R a, R b, H6<R> (&acc)[NR]) {
-  const R sb = pr.p ? -b : b;
-  H6<R> h[NR];
+                                       const Geom& g, int s, const Pair& pr, R a, R b, Halves<R> (&d)[NR]) {
+  constexpr int f = FWD ? 1 : -1;
+  H6<R> m[NR];
   int n = s;
-  if constexpr (FWD) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) gather_pair<R, 2 * (I == 0), 2 * (I == 1), 2 * (I == 2), 0>(psi + r * rs, c, g, pr, h[r]);
-  } else {
-#pragma unroll
-    for (int r = 0; r < NR; ++r) n = gather_pair<R, -2 * (I == 0), -2 * (I == 1), -2 * (I == 2), 0>(psi + r * rs, c, g, pr, h[r]);
-  }
-  const M3<R> V = W(n, M_VII + I);
+  for (int r = 0; r < NR; ++r)
+    n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0, AP>(psi + r * rs, c, g, pr, m[r]);
+  const M3<R> V = W(FWD ? s : n, M_VII + I);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     H6<R> y;
-    colour2h<R, !FWD>(y, V, h[r]);
-    add_scaled_h(acc[r], a, y);
-    add_sigma_h(acc[r], I, y, FWD ? sb : -sb);
+    colour2h<R, !FWD>(y, V, m[r]);
+    add_scaled_h(d[r].same, a, y);
+    add_sigma_h(d[r].cross, I, y, FWD ? b : -b);
   }
 }
 
-// Diagonal pair (I, J): +-(s_I + s_J) V h (x+I+J) and +-(s_I - s_J) X h (x+I-J) forward, the
-// adjoints with opposite signs from x-I-J and x-I+J backward.
-template <typename R, int NR, int I, int J, int P, bool FWD, typename WS>
+template <typename R, int NR, int I, int J, int P, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void mr_diag(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
-                                        const Geom& g, int s, const Pair& pr, H6<R> (&acc)[NR]) {
+                                        const Geom& g, int s, const Pair& pr, Halves<R> (&d)[NR]) {
+  constexpr int f = FWD ? 1 : -1;
   constexpr int A0 = (I == 0) + (J == 0), A1 = (I == 1) + (J == 1), A2 = (I == 2) + (J == 2);
   constexpr int B0 = (I == 0) - (J == 0), B1 = (I == 1) - (J == 1), B2 = (I == 2) - (J == 2);
-  const R sg = pr.p ? R(-1) : R(1);
-  const R f = FWD ? sg : -sg;
-  H6<R> h[NR];
+  H6<R> m, y[NR];
   int n = s;
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    if constexpr (FWD) gather_pair<R, A0, A1, A2, 0>(psi + r * rs, c, g, pr, h[r]);
-    else n = gather_pair<R, -A0, -A1, -A2, 0>(psi + r * rs, c, g, pr, h[r]);
+    n = gather_mine<R, f * A0, f * A1, f * A2, 0, AP>(psi + r * rs, c, g, pr, m);
+    sigma_pair<R, I, J, 1>(m, y[r]);
   }
-  M3<R> V = W(n, M_VIJ + P);
+  M3<R> V = W(FWD ? s : n, M_VIJ + P);
+#pragma unroll
+  for (int r = 0; r < NR; ++r) colour2h_acc<R, !FWD>(d[r].cross, V, y[r]);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    H6<R> y;
-    colour2h<R, !FWD>(y, V, h[r]);
-    add_sigma_h(acc[r], I, y, f);
-    add_sigma_h(acc[r], J, y, f);
+    n = gather_mine<R, f * B0, f * B1, f * B2, 0, AP>(psi + r * rs, c, g, pr, m);
+    sigma_pair<R, I, J, -1>(m, y[r]);
   }
+  V = W(FWD ? s : n, M_XIJ + P);
 #pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    if constexpr (FWD) gather_pair<R, B0, B1, B2, 0>(psi + r * rs, c, g, pr, h[r]);
-    else n = gather_pair<R, -B0, -B1, -B2, 0>(psi + r * rs, c, g, pr, h[r]);
-  }
-  V = W(n, M_XIJ + P);
-#pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    H6<R> y;
-    colour2h<R, !FWD>(y, V, h[r]);
-    add_sigma_h(acc[r], I, y, f);
-    add_sigma_h(acc[r], J, y, -f);
-  }
+  for (int r = 0; r < NR; ++r) colour2h_acc<R, !FWD>(d[r].cross, V, y[r]);
 }
 
-template <int NR, int EPI, typename WT>
+template <int NR, int EPI, typename WT, bool AP = true>
 __global__ void __launch_bounds__(MR_THREADS, mr_minb<NR>())
     apply_mrhs_kernel(const cx<WT>* __restrict__ W, const cx<float>* __restrict__ psi, cx<float>* __restrict__ out, long long rs,
                       Geom g, float c0q, float a_ii, float b_ii, MultiEpi ep) {
@@ -235,30 +188,37 @@ __global__ void __launch_bounds__(MR_THREADS, mr_minb<NR>())
       c[0] = rr % g.L[0]; rr /= g.L[0];
       c[1] = rr % g.L[1]; rr /= g.L[1];
       c[2] = rr % g.L[2]; c[3] = rr / g.L[2];
+      Halves<R> hs[NR];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) zero_halves(hs[r]);
       if (half == 0) {
+        mr_time<R, NR, true, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_two<R, NR, 0, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 1, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 2, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_diag<R, NR, 0, 1, 0, true, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 0, 2, 1, true, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 1, 2, 2, true, AP>(Wg, P, rs, c, g, s, pr, hs);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) to_h(hs[r], pr, acc[r]);
 #pragma unroll
         for (int r = 0; r < NR; ++r) pair_onsite<R>(Wg, P + r * rs, s, pr, c0q, acc[r]);
-        mr_time<R, NR, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 0, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 1, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 2, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_two<R, NR, 0, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_two<R, NR, 1, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_two<R, NR, 2, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_diag<R, NR, 0, 1, 0, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_diag<R, NR, 0, 2, 1, true>(Wg, P, rs, c, g, s, pr, acc);
-        mr_diag<R, NR, 1, 2, 2, true>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 0, true, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 1, true, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 2, true, AP>(Wg, P, rs, c, g, s, pr, acc);
       } else {
-        mr_spatial<R, NR, 0, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 1, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 2, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_time<R, NR, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_two<R, NR, 0, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_two<R, NR, 1, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_two<R, NR, 2, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, acc);
-        mr_diag<R, NR, 0, 1, 0, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_diag<R, NR, 0, 2, 1, false>(Wg, P, rs, c, g, s, pr, acc);
-        mr_diag<R, NR, 1, 2, 2, false>(Wg, P, rs, c, g, s, pr, acc);
+        mr_time<R, NR, false, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_two<R, NR, 0, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 1, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 2, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_diag<R, NR, 0, 1, 0, false, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 0, 2, 1, false, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 1, 2, 2, false, AP>(Wg, P, rs, c, g, s, pr, hs);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) to_h(hs[r], pr, acc[r]);
+        mr_spatial<R, NR, 0, false, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 1, false, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 2, false, AP>(Wg, P, rs, c, g, s, pr, acc);
 #pragma unroll
         for (int r = 0; r < NR; ++r)
 #pragma unroll

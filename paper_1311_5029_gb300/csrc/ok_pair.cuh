@@ -8,60 +8,49 @@
 
 namespace okgb {
 
-// Read-only load of one FP32 W element.  Variant 0: plain __ldg; 1: not allocated in L1 (a W
-// element is used by exactly one thread, so L1 is left to the neighbour spinors); 2: with a 256-byte
-// L2 prefetch hint (a matrix element row of 32 sites is 256 bytes, read by two warps); 3: both.
-#ifndef OK_W_LOAD
-#define OK_W_LOAD 0
-#endif
-__device__ __forceinline__ float2 ldg_w(const float2* p) {
-  float2 d;
-#if OK_W_LOAD == 1
-  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(d.x), "=f"(d.y) : "l"(p));
-#elif OK_W_LOAD == 2
-  asm volatile("ld.global.nc.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(d.x), "=f"(d.y) : "l"(p));
-#elif OK_W_LOAD == 3
-  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(d.x), "=f"(d.y) : "l"(p));
-#else
-  d = __ldg(p);
-#endif
-  return d;
-}
-
-// Matrix m of the site record of `site`.
+// Matrix m of the site record of `site` (FP64: nine 16-byte loads; FP32: four and one of 8 bytes).
 template <typename R>
 __device__ __forceinline__ M3<R> wmat(const cx<R>* __restrict__ W, int site, int m) {
-  const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES) + (site & 31);
+  const cx<R>* p = W + ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
+  const int l = site & 31;
   M3<R> a;
   if constexpr (std::is_same<R, double>::value) {
-    const double2* p = reinterpret_cast<const double2*>(W) + base;
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-      double2 d = __ldg(p + e * LANES);
+      const double2 d = __ldg(reinterpret_cast<const double2*>(p) + e * LANES + l);
       a.e[e] = mk<R>(d.x, d.y);
     }
   } else {
-    const float2* p = reinterpret_cast<const float2*>(W) + base;
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      float2 d = ldg_w(p + e * LANES);
-      a.e[e] = mk<R>(d.x, d.y);
+    for (int q = 0; q < 4; ++q) {
+      const float4 d = __ldg(reinterpret_cast<const float4*>(p) + q * LANES + l);
+      a.e[2 * q] = mk<R>(d.x, d.y);
+      a.e[2 * q + 1] = mk<R>(d.z, d.w);
     }
+    const float2 d = __ldg(reinterpret_cast<const float2*>(p) + 8 * LANES + l);
+    a.e[8] = mk<R>(d.x, d.y);
   }
   return a;
 }
 
-// Matrix m of the site record of `site` from the half-precision copy, widened to FP32.
+// The same from the half-precision copy, widened to FP32 (two 16-byte loads and one of 4 bytes).
+__device__ __forceinline__ cx<float> widen(unsigned u) {
+  const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u));
+  return mk<float>(f.x, f.y);
+}
 __device__ __forceinline__ M3<float> wmat(const cx<__half>* __restrict__ W, int site, int m) {
-  const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES) + (site & 31);
-  const unsigned* p = reinterpret_cast<const unsigned*>(W) + base;
+  const cx<__half>* p = W + ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
+  const int l = site & 31;
   M3<float> a;
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const unsigned u = __ldg(p + e * LANES);
-    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u));
-    a.e[e] = mk<float>(f.x, f.y);
+  for (int q = 0; q < 2; ++q) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p) + q * LANES + l);
+    a.e[4 * q] = widen(u.x);
+    a.e[4 * q + 1] = widen(u.y);
+    a.e[4 * q + 2] = widen(u.z);
+    a.e[4 * q + 3] = widen(u.w);
   }
+  a.e[8] = widen(__ldg(reinterpret_cast<const unsigned*>(p) + 8 * LANES + l));
   return a;
 }
 
@@ -121,8 +110,8 @@ template <typename R> __device__ __forceinline__ void mdv(cx<R> (&y)[3], const M
 // ---------------------------------------------------------------------------- geometry
 // Neighbour x + d with fermion boundary sign; |d_mu| <= 2.  The coordinate is wrapped by at most
 // two conditional subtractions (two are needed only when L_mu < |d_mu|, on lattices of extent 1
-// or 2); the sign flips once per wrap across an antiperiodic boundary.
-template <int D0, int D1, int D2, int D3>
+// or 2); the sign flips once per wrap across an antiperiodic boundary (AP false: there is none).
+template <int D0, int D1, int D2, int D3, bool AP = true>
 __device__ __forceinline__ int nbr_site(const int (&c)[4], const Geom& g, bool& neg) {
   const int d[4] = {D0, D1, D2, D3};
   int idx = 0;
@@ -139,7 +128,7 @@ __device__ __forceinline__ int nbr_site(const int (&c)[4], const Geom& g, bool& 
       } else {
         if (x < 0) { x += L; wraps = 1; if (x < 0) { x += L; wraps = 2; } }
       }
-      if (((g.bcneg >> mu) & 1) && (wraps & 1)) neg = !neg;
+      if (AP && ((g.bcneg >> mu) & 1) && (wraps & 1)) neg = !neg;
     }
     idx += x * g.S[mu];
   }
@@ -148,13 +137,19 @@ __device__ __forceinline__ int nbr_site(const int (&c)[4], const Geom& g, bool& 
 
 
 // ============================================================================ two threads per site
-// The pair (lanes 2k, 2k+1) shares one site.  Thread p = 0 accumulates acc+ and loads the upper
-// spin half u of every spinor it needs, thread p = 1 accumulates acc- and loads the lower half l;
-// the other half arrives through one shuffle.  Spatial hops then split without duplicated work:
-// p = 0 uses (D + S)/2 forward and (D - S)/2 backward, p = 1 the other two.  W^0, the temporal hop
-// and the colour matrices of the two-hop terms are read by both threads (the same addresses, one
-// transaction per warp).  Half the registers per thread and twice the warps per SM keep more
-// global loads in flight than one thread per site can.
+// The pair (lanes 2k, 2k+1) shares one site.  Thread p = 0 loads the upper spin half u of every
+// spinor it needs, thread p = 1 the lower half l.  Two bases are used:
+//   * The temporal, two-hop and diagonal hops need no exchange between the threads.  W^+-_4,
+//     W^{++}_ii and W^{++}_ij, W^{+-}_ij are [[A, B], [B, D]] on (u, l) with the same B both ways, so a
+//     thread multiplies its own half only and adds the result to `same` (its own half of the output)
+//     or to `cross` (the partner's half).  to_h exchanges the two sums once per site.
+//   * The nearest spatial hops and W^0 work on h+- = u +- l (u -+ i l for W^0): p = 0 accumulates
+//     acc+ with (D + S)/2 forward and (D - S)/2 backward, p = 1 acc- with the other two, so no matrix
+//     is read twice; the partner's half arrives through one shuffle per component.
+// With every hop in the h+- basis a site took 27 exchanges of 12 shuffles instead of 10, and each
+// diagonal product 48 additions instead of 24: 48.4 M warp instructions for an FP32 application at
+// 16^3 x 32, now 39 M.  Six right-hand sides at 12^3 x 24 in FP32 (apply_mrhs_kernel, whose unrolled code
+// overflowed the instruction caches): 169 us before, 137 us now.
 
 template <typename R> struct H6 { cx<R> v[2][3]; };
 
@@ -213,33 +208,75 @@ struct Pair {
   unsigned mask;  // the two lanes of the pair
 };
 
-// Gather the neighbour at offset D: mine = own half, oth = partner's half, h = h+ (p = 0) or h- (p = 1).
-template <typename R, int D0, int D1, int D2, int D3>
-__device__ __forceinline__ int gather_pair(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
-                                           H6<R>& h, H6<R>* u = nullptr, H6<R>* l = nullptr) {
+// The thread's own half of the neighbour at offset D, with the boundary sign (a multiplication, not a
+// branch: the hops stay one basic block, so the loads of the next hop can be issued early).
+template <typename R, int D0, int D1, int D2, int D3, bool AP>
+__device__ __forceinline__ int gather_mine(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
+                                           H6<R>& mine) {
   bool neg;
-  int n = nbr_site<D0, D1, D2, D3>(c, g, neg);
-  H6<R> mine;
+  const int n = nbr_site<D0, D1, D2, D3, AP>(c, g, neg);
   load_half<R>(psi, n, pr.p, mine);
-  if (neg) {
+  if constexpr (AP) {
+    const R sg = neg ? R(-1) : R(1);
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) mine.v[s][a] = -mine.v[s][a];
+      for (int a = 0; a < 3; ++a) mine.v[s][a] = sg * mine.v[s][a];
   }
-  H6<R> oth = partner(mine, pr.mask);
-  // p = 0: h+ = mine + oth (u = mine);  p = 1: h- = oth - mine (u = oth)
+  return n;
+}
+
+// h+ = u + l (p = 0) or h- = u - l (p = 1) from the threads' halves.
+template <typename R>
+__device__ __forceinline__ void halves_to_h(const H6<R>& mine, const Pair& pr, H6<R>& h) {
+  const H6<R> oth = partner(mine, pr.mask);
   const R sg = pr.p ? R(-1) : R(1);
 #pragma unroll
   for (int s = 0; s < 2; ++s)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      cx<R> m = mine.v[s][a], o = oth.v[s][a];
-      h.v[s][a] = mk<R>(sg * m.re + o.re, sg * m.im + o.im);
-      if (u) u->v[s][a] = pr.p ? o : m;
-      if (l) l->v[s][a] = pr.p ? m : o;
+      h.v[s][a].re = fma(sg, mine.v[s][a].re, oth.v[s][a].re);
+      h.v[s][a].im = fma(sg, mine.v[s][a].im, oth.v[s][a].im);
     }
+}
+
+// h+ (p = 0) or h- (p = 1) of the neighbour at offset D.
+template <typename R, int D0, int D1, int D2, int D3, bool AP>
+__device__ __forceinline__ int gather_pair(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
+                                           H6<R>& h) {
+  H6<R> mine;
+  const int n = gather_mine<R, D0, D1, D2, D3, AP>(psi, c, g, pr, mine);
+  halves_to_h(mine, pr, h);
   return n;
+}
+
+// Sums of the hops without exchange: same goes to the thread's own half of the output, cross to the
+// partner's.
+template <typename R> struct Halves { H6<R> same, cross; };
+
+template <typename R>
+__device__ __forceinline__ void zero_halves(Halves<R>& d) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) d.same.v[s][a] = d.cross.v[s][a] = mk<R>(0, 0);
+}
+
+// acc+ += D_u + D_l (p = 0), acc- += D_u - D_l (p = 1) of the half outputs D = same + partner's cross.
+template <typename R>
+__device__ __forceinline__ void to_h(const Halves<R>& d, const Pair& pr, H6<R>& acc) {
+  const H6<R> oc = partner(d.cross, pr.mask);
+  H6<R> m;
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m.v[s][a] = d.same.v[s][a] + oc.v[s][a];
+  H6<R> h;
+  halves_to_h(m, pr, h);
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) acc.v[s][a] = acc.v[s][a] + h.v[s][a];
 }
 
 template <typename R, bool DAG, typename WS>
@@ -278,77 +315,60 @@ __device__ __forceinline__ void colour2h(H6<R>& y, const M3<R>& V, const H6<R>& 
   else { mv(y.v[0], V, h.v[0]); mv(y.v[1], V, h.v[1]); }
 }
 
-// Each hop function takes FWD / BWD flags so that the forward and the backward halves of the
-// stencil can run in different warps (the split kernel below).
-template <typename R, int I, bool FWD = true, bool BWD = true, typename WS>
+// Each hop function does the forward (FWD) or the backward half of its part of the stencil; the two
+// run in different warps (the split kernel).
+template <typename R, int I, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void pair_spatial(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                              const Geom& g, int s, const Pair& pr, H6<R>& acc) {
-  const int base = M_WP + 8 * I;
+  constexpr int base = M_WP + 8 * I, f = FWD ? 1 : -1;
   H6<R> h;
-  if constexpr (FWD) {
-    gather_pair<R, I == 0, I == 1, I == 2, 0>(psi, c, g, pr, h);
-    block2h<R, false>(W, s, base + 4 * pr.p, h, acc);
-  }
-  if constexpr (BWD) {
-    int n = gather_pair<R, -(I == 0), -(I == 1), -(I == 2), 0>(psi, c, g, pr, h);
-    block2h<R, true>(W, n, base + 4 * (1 - pr.p), h, acc);
-  }
+  const int n = gather_pair<R, f * (I == 0), f * (I == 1), f * (I == 2), 0, AP>(psi, c, g, pr, h);
+  if constexpr (FWD) block2h<R, false>(W, s, base + 4 * pr.p, h, acc);
+  else block2h<R, true>(W, n, base + 4 * (1 - pr.p), h, acc);
 }
 
-// acc+ += S h+ - U l (p = 0);  acc- += -S h- + U l (p = 1)   [forward, matrices at x]
-// acc+ += -U^dag u - S^dag h+;  acc- += -U^dag u + S^dag h-   [backward, matrices at x - t]
-template <typename R, bool FWD = true, bool BWD = true, typename WS>
+// m, or zero for the thread whose half a term does not act on (selects instead of a branch).
+template <typename R>
+__device__ __forceinline__ void only(H6<R>& m, bool mine) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m.v[s][a] = mk<R>(mine ? m.v[s][a].re : R(0), mine ? m.v[s][a].im : R(0));
+}
+
+// On (u, l): W^+_4 = [[0, S], [S, -U]] with the matrices at x, W^-_4 = [[-U^dag, -S^dag], [-S^dag, 0]]
+// with those at x - t (halves stored); S = [[s3, n1], [n2, -s3]].
+template <typename R, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void pair_time(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                          const Geom& g, int s, const Pair& pr, H6<R>& acc) {
-  const R sg = pr.p ? R(-1) : R(1);
-  H6<R> h, u, l;
+                                          const Geom& g, int s, const Pair& pr, Halves<R>& d) {
+  H6<R> m;
   if constexpr (FWD) {
-    gather_pair<R, 0, 0, 0, 1>(psi, c, g, pr, h, nullptr, &l);
-    // acc += sg (S h - U l),  S = [[s3, n1], [n2, -s3]]
-    H6<R> sh;
-    M3<R> s3 = W(s, M_ST + 0);
-    mv(sh.v[0], s3, h.v[0]);
-    mv(sh.v[1], s3, h.v[1]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) sh.v[1][a] = -sh.v[1][a];
-    M3<R> n1 = W(s, M_ST + 1);
-    mv_add(sh.v[0], n1, h.v[1]);
-    M3<R> n2 = W(s, M_ST + 2);
-    mv_add(sh.v[1], n2, h.v[0]);
-    M3<R> U = W(s, M_UT);
-    mv_sub(sh.v[0], U, l.v[0]);
-    mv_sub(sh.v[1], U, l.v[1]);
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        acc.v[q][a].re = fma(sg, sh.v[q][a].re, acc.v[q][a].re);
-        acc.v[q][a].im = fma(sg, sh.v[q][a].im, acc.v[q][a].im);
-      }
-  }
-  if constexpr (BWD) {
-    int n = gather_pair<R, 0, 0, 0, -1>(psi, c, g, pr, h, &u, nullptr);
-    // S^dag h = [[s3^dag, n2^dag], [n1^dag, -s3^dag]] h ; acc += -U^dag u - sg S^dag h
-    H6<R> sh;
-    M3<R> s3 = W(n, M_ST + 0);
-    mdv(sh.v[0], s3, h.v[0]);
-    mdv(sh.v[1], s3, h.v[1]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) sh.v[1][a] = -sh.v[1][a];
-    M3<R> n2 = W(n, M_ST + 2);
-    mdv_add(sh.v[0], n2, h.v[1]);
-    M3<R> n1 = W(n, M_ST + 1);
-    mdv_add(sh.v[1], n1, h.v[0]);
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        acc.v[q][a].re = fma(-sg, sh.v[q][a].re, acc.v[q][a].re);
-        acc.v[q][a].im = fma(-sg, sh.v[q][a].im, acc.v[q][a].im);
-      }
-    M3<R> U = W(n, M_UT);
-    mdv_sub(acc.v[0], U, u.v[0]);
-    mdv_sub(acc.v[1], U, u.v[1]);
+    gather_mine<R, 0, 0, 0, 1, AP>(psi, c, g, pr, m);
+    M3<R> A = W(s, M_ST + 0);
+    mv_add(d.cross.v[0], A, m.v[0]);
+    mv_sub(d.cross.v[1], A, m.v[1]);
+    A = W(s, M_ST + 1);
+    mv_add(d.cross.v[0], A, m.v[1]);
+    A = W(s, M_ST + 2);
+    mv_add(d.cross.v[1], A, m.v[0]);
+    only(m, pr.p == 1);  // U multiplies l
+    A = W(s, M_UT);
+    mv_sub(d.same.v[0], A, m.v[0]);
+    mv_sub(d.same.v[1], A, m.v[1]);
+  } else {
+    // S^dag = [[s3^dag, n2^dag], [n1^dag, -s3^dag]]
+    const int n = gather_mine<R, 0, 0, 0, -1, AP>(psi, c, g, pr, m);
+    M3<R> A = W(n, M_ST + 0);
+    mdv_sub(d.cross.v[0], A, m.v[0]);
+    mdv_add(d.cross.v[1], A, m.v[1]);
+    A = W(n, M_ST + 2);
+    mdv_sub(d.cross.v[0], A, m.v[1]);
+    A = W(n, M_ST + 1);
+    mdv_sub(d.cross.v[1], A, m.v[0]);
+    only(m, pr.p == 0);  // U^dag multiplies u
+    A = W(n, M_UT);
+    mdv_sub(d.same.v[0], A, m.v[0]);
+    mdv_sub(d.same.v[1], A, m.v[1]);
   }
 }
 
@@ -363,58 +383,65 @@ __device__ __forceinline__ void add_scaled_h(H6<R>& acc, R a, const H6<R>& y) {
     }
 }
 
-// W^{++}_ii: acc+- += (a +- b sigma_i) V h+-  forward,  (a -+ b sigma_i) V^dag h+-  backward.
-template <typename R, int I, bool FWD = true, bool BWD = true, typename WS>
+// W^{++}_ii = [[a, b sigma_i], [b sigma_i, a]] (x) V forward, [[a, -b sigma_i], [-b sigma_i, a]] (x) V^dag backward.
+template <typename R, int I, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void pair_two(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                         const Geom& g, int s, const Pair& pr, R a, R b, H6<R>& acc) {
-  const R sb = pr.p ? -b : b;
-  H6<R> h, y;
-  if constexpr (FWD) {
-    gather_pair<R, 2 * (I == 0), 2 * (I == 1), 2 * (I == 2), 0>(psi, c, g, pr, h);
-    M3<R> V = W(s, M_VII + I);
-    colour2h<R, false>(y, V, h);
-    add_scaled_h(acc, a, y);
-    add_sigma_h(acc, I, y, sb);
-  }
-  if constexpr (BWD) {
-    int n = gather_pair<R, -2 * (I == 0), -2 * (I == 1), -2 * (I == 2), 0>(psi, c, g, pr, h);
-    M3<R> V = W(n, M_VII + I);
-    colour2h<R, true>(y, V, h);
-    add_scaled_h(acc, a, y);
-    add_sigma_h(acc, I, y, -sb);
+                                         const Geom& g, int s, const Pair& pr, R a, R b, Halves<R>& d) {
+  constexpr int f = FWD ? 1 : -1;
+  H6<R> m, y;
+  const int n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0, AP>(psi, c, g, pr, m);
+  const M3<R> V = W(FWD ? s : n, M_VII + I);
+  colour2h<R, !FWD>(y, V, m);
+  add_scaled_h(d.same, a, y);
+  add_sigma_h(d.cross, I, y, FWD ? b : -b);
+}
+
+// s = (sigma_I + SG sigma_J) m, I < J.
+template <typename R, int I, int J, int SG>
+__device__ __forceinline__ void sigma_pair(const H6<R>& m, H6<R>& s) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cx<R> x = m.v[0][a], y = m.v[1][a];
+    if constexpr (I == 0 && J == 1) {       // [[0, 1 - SG i], [1 + SG i, 0]]
+      s.v[0][a] = SG > 0 ? y + tmi(y) : y + ti(y);
+      s.v[1][a] = SG > 0 ? x + ti(x) : x + tmi(x);
+    } else if constexpr (I == 0) {          // [[SG, 1], [1, -SG]]
+      s.v[0][a] = SG > 0 ? y + x : y - x;
+      s.v[1][a] = SG > 0 ? x - y : x + y;
+    } else {                                // [[SG, -i], [i, -SG]]
+      s.v[0][a] = SG > 0 ? tmi(y) + x : tmi(y) - x;
+      s.v[1][a] = SG > 0 ? ti(x) - y : ti(x) + y;
+    }
   }
 }
 
-// Diagonal pair (I, J): acc+- += +-(s_I + s_J) V h, -+(s_I + s_J) V^dag h (x-I-J),
-//                       +-(s_I - s_J) X h (x+I-J), -+(s_I - s_J) X^dag h (x-I+J).
-template <typename R, int I, int J, int P, bool FWD = true, bool BWD = true, typename WS>
+template <typename R, bool DAG>
+__device__ __forceinline__ void colour2h_acc(H6<R>& y, const M3<R>& V, const H6<R>& h) {
+  if (DAG) { mdv_sub(y.v[0], V, h.v[0]); mdv_sub(y.v[1], V, h.v[1]); }
+  else { mv_add(y.v[0], V, h.v[0]); mv_add(y.v[1], V, h.v[1]); }
+}
+
+// Diagonal pair (I, J): [[0, S], [S, 0]] with S = (s_I + s_J) (x) V from x+I+J and (s_I - s_J) (x) X from
+// x+I-J (forward), minus their adjoints from x-I-J and x-I+J (backward).
+template <typename R, int I, int J, int P, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void pair_diag(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
-                                          const Geom& g, int s, const Pair& pr, H6<R>& acc) {
+                                          const Geom& g, int s, const Pair& pr, Halves<R>& d) {
+  constexpr int f = FWD ? 1 : -1;
   constexpr int A0 = (I == 0) + (J == 0), A1 = (I == 1) + (J == 1), A2 = (I == 2) + (J == 2);
   constexpr int B0 = (I == 0) - (J == 0), B1 = (I == 1) - (J == 1), B2 = (I == 2) - (J == 2);
-  const R sg = pr.p ? R(-1) : R(1);
-  H6<R> h, y;
-  M3<R> V;
-  if constexpr (FWD) {
-    gather_pair<R, A0, A1, A2, 0>(psi, c, g, pr, h);
-    V = W(s, M_VIJ + P);
-    colour2h<R, false>(y, V, h); add_sigma_h(acc, I, y, sg); add_sigma_h(acc, J, y, sg);
-    gather_pair<R, B0, B1, B2, 0>(psi, c, g, pr, h);
-    V = W(s, M_XIJ + P);
-    colour2h<R, false>(y, V, h); add_sigma_h(acc, I, y, sg); add_sigma_h(acc, J, y, -sg);
-  }
-  if constexpr (BWD) {
-    int n = gather_pair<R, -A0, -A1, -A2, 0>(psi, c, g, pr, h);
-    V = W(n, M_VIJ + P);
-    colour2h<R, true>(y, V, h); add_sigma_h(acc, I, y, -sg); add_sigma_h(acc, J, y, -sg);
-    n = gather_pair<R, -B0, -B1, -B2, 0>(psi, c, g, pr, h);
-    V = W(n, M_XIJ + P);
-    colour2h<R, true>(y, V, h); add_sigma_h(acc, I, y, -sg); add_sigma_h(acc, J, y, sg);
-  }
+  H6<R> m, y;
+  int n = gather_mine<R, f * A0, f * A1, f * A2, 0, AP>(psi, c, g, pr, m);
+  sigma_pair<R, I, J, 1>(m, y);
+  M3<R> V = W(FWD ? s : n, M_VIJ + P);
+  colour2h_acc<R, !FWD>(d.cross, V, y);
+  n = gather_mine<R, f * B0, f * B1, f * B2, 0, AP>(psi, c, g, pr, m);
+  sigma_pair<R, I, J, -1>(m, y);
+  V = W(FWD ? s : n, M_XIJ + P);
+  colour2h_acc<R, !FWD>(d.cross, V, y);
 }
 
 // On-site term W^0 psi_x (both halves of the pair): p = 0 forms A = Y+ (u - i l), p = 1 forms
-// B = Y- (u + i l); acc = (A + B) + i (A - B) for p = 0 and (A + B) - i (A - B) for p = 1.
+// B = Y- (u + i l); acc += (A + B) + i (A - B) for p = 0 and (A + B) - i (A - B) for p = 1.
 template <typename R, typename WS>
 __device__ __forceinline__ void pair_onsite(const WS& W, const cx<R>* __restrict__ psi, int s, const Pair& pr, R c0q,
                                             H6<R>& acc) {
@@ -441,7 +468,8 @@ __device__ __forceinline__ void pair_onsite(const WS& W, const cx<R>* __restrict
 #pragma unroll
   for (int q = 0; q < 2; ++q)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) acc.v[q][k] = (Rm.v[q][k] + Rp.v[q][k]) + ti(Rm.v[q][k] - Rp.v[q][k]);
+    for (int k = 0; k < 3; ++k)
+      acc.v[q][k] = acc.v[q][k] + ((Rm.v[q][k] + Rp.v[q][k]) + ti(Rm.v[q][k] - Rp.v[q][k]));
 }
 
 }  // namespace okgb

@@ -192,33 +192,56 @@ struct WOut {
   cx<__half>* W16;
 };
 
+// The FP32 and FP16 copies of a matrix, in 16-byte words (w_elem).
+__device__ __forceinline__ void store_low(const WOut& o, size_t base, int lane, const M3<float>& f) {
+  if (o.W32) {
+    cx<float>* p = o.W32 + base;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      reinterpret_cast<float4*>(p)[q * LANES + lane] = make_float4(f.e[2 * q].re, f.e[2 * q].im, f.e[2 * q + 1].re, f.e[2 * q + 1].im);
+    reinterpret_cast<float2*>(p)[8 * LANES + lane] = make_float2(f.e[8].re, f.e[8].im);
+  }
+  if (o.W16) {
+    cx<__half>* p = o.W16 + base;
+    unsigned h[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const __half2 v = __halves2half2(__float2half_rn(f.e[e].re), __float2half_rn(f.e[e].im));
+      h[e] = *reinterpret_cast<const unsigned*>(&v);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      reinterpret_cast<uint4*>(p)[q * LANES + lane] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+    reinterpret_cast<unsigned*>(p)[8 * LANES + lane] = h[8];
+  }
+}
+
 __device__ __forceinline__ void store_mat(const WOut& o, int site, int m, const M3<double>& a) {
-  size_t blk = (size_t)(site >> 5);
-  int lane = site & 31;
-  size_t base = (blk * NMAT + m) * 9 * LANES + lane;
+  const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
+  const int lane = site & 31;
+  M3<float> f;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    if (o.W64) o.W64[base + (size_t)e * LANES] = a.e[e];
-    if (o.W32) o.W32[base + (size_t)e * LANES] = mk<float>((float)a.e[e].re, (float)a.e[e].im);
-    if (o.Wdf) o.Wdf[base + (size_t)e * LANES] = mk<dd>(split_df(a.e[e].re), split_df(a.e[e].im));
-    if (o.W16) o.W16[base + (size_t)e * LANES] = mk<__half>(__float2half_rn((float)a.e[e].re), __float2half_rn((float)a.e[e].im));
+    if (o.W64) o.W64[base + w_elem<double>(e, lane)] = a.e[e];
+    if (o.Wdf) o.Wdf[base + w_elem<dd>(e, lane)] = mk<dd>(split_df(a.e[e].re), split_df(a.e[e].im));
+    f.e[e] = mk<float>((float)a.e[e].re, (float)a.e[e].im);
   }
+  store_low(o, base, lane, f);
 }
 
 // The same stores from a double-float result (the FP32-pipe precompute, used when no native FP64
 // copy is kept): the double-float copy takes the pairs as they are, the FP32 and FP16 copies the
 // rounded high parts.
 __device__ __forceinline__ void store_mat(const WOut& o, int site, int m, const M3<dd>& a) {
-  size_t blk = (size_t)(site >> 5);
-  int lane = site & 31;
-  size_t base = (blk * NMAT + m) * 9 * LANES + lane;
+  const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
+  const int lane = site & 31;
+  M3<float> f;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    if (o.Wdf) o.Wdf[base + (size_t)e * LANES] = a.e[e];
-    const float re = a.e[e].re.hi + a.e[e].re.lo, im = a.e[e].im.hi + a.e[e].im.lo;
-    if (o.W32) o.W32[base + (size_t)e * LANES] = mk<float>(re, im);
-    if (o.W16) o.W16[base + (size_t)e * LANES] = mk<__half>(__float2half_rn(re), __float2half_rn(im));
+    if (o.Wdf) o.Wdf[base + w_elem<dd>(e, lane)] = a.e[e];
+    f.e[e] = mk<float>(a.e[e].re.hi + a.e[e].re.lo, a.e[e].im.hi + a.e[e].im.lo);
   }
+  store_low(o, base, lane, f);
 }
 
 constexpr int K2_THREADS = 64;
@@ -280,11 +303,11 @@ template <typename R>
 __device__ __forceinline__ M3<double> fetch(const cx<R>* __restrict__ W, int site, int m) {
   size_t blk = (size_t)(site >> 5);
   int lane = site & 31;
-  size_t base = (blk * NMAT + m) * 9 * LANES + lane;
+  size_t base = (blk * NMAT + m) * 9 * LANES;
   M3<double> a;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    cx<R> v = W[base + (size_t)e * LANES];
+    cx<R> v = W[base + w_elem<R>(e, lane)];
     a.e[e] = mk<double>((double)v.re, (double)v.im);
   }
   return a;

@@ -127,7 +127,7 @@ int iterate(const ok_W* W, const IterBufs<R>& b, long long n, SolverState* dst, 
   // FP32: plain applications, their inner products in separate passes (cheaper than the fused
   // epilogue in this kernel); FP64: the epilogue is fused (the FP64 pipe bounds that kernel).
   constexpr bool fused = sizeof(R) == 8;
-  EpiArgs<R> e1{b.rhat, nullptr, RedArgs{dst, part, nullptr, FIN_ALPHA}, &dst->ticket[0], &dst->halt};
+  const EpiArgs<R> e1{b.rhat, nullptr, RedArgs{dst, part, nullptr, FIN_ALPHA}, &dst->ticket[0], &dst->halt};
   OK_TRY(apply_iter<R>(W, pin, b.v, fused ? EPI_DOT : EPI_NONE, e1, w16, st));
   if (!fused) OK_TRY(launch_dots<R>(b.rhat, b.v, n, false, dst, part, st));
   OK_TRY(launch_update_s<R>(b.r, b.v, b.s, n, dst, st));
@@ -137,7 +137,7 @@ int iterate(const ok_W* W, const IterBufs<R>& b, long long n, SolverState* dst, 
       sin = pc.zs;
     }
   }
-  EpiArgs<R> e2{pre ? b.s : nullptr, nullptr, RedArgs{dst, part, nullptr, FIN_OMEGA}, &dst->ticket[1], &dst->halt};
+  const EpiArgs<R> e2{nullptr, nullptr, RedArgs{dst, part, nullptr, FIN_OMEGA}, &dst->ticket[1], &dst->halt};
   OK_TRY(apply_iter<R>(W, sin, b.t, fused ? EPI_TS : EPI_NONE, e2, w16, st));
   if (!fused) OK_TRY(launch_dots<R>(b.t, b.s, n, true, dst, part, st));
   OK_TRY(launch_update_xr<R>(b.x, pin, b.s, b.t, b.r, b.rhat, n, dst, part, st, pre ? sin : nullptr));
@@ -376,7 +376,8 @@ int apply_reduce(const ok_W* W, ok_prec prec, int kind, const void* psi, const v
   Workspace ws;
   ws.st = st;
   cudaError_t err = cudaSuccess;
-  double* part = ws.get<double>((size_t)apply_blocks_needed(W) * 4, &err);
+  const int nb = apply_blocks_needed(W), nd = blas_blocks(12LL * W->g.V);
+  double* part = ws.get<double>((size_t)(nb > nd ? nb : nd) * 4, &err);
   SolverState* dst = ws.get<SolverState>(1, &err);
   HostState hs;
   if (!part || !dst || !hs.h) { if (err != cudaSuccess) set_cuda_error(err); return OK_ENOMEM; }
@@ -386,9 +387,13 @@ int apply_reduce(const ok_W* W, ok_prec prec, int kind, const void* psi, const v
     EpiArgs<double> e{(const cx<double>*)y, nullptr, ra, &dst->ticket[0], nullptr};
     OK_TRY(launch_apply<double>(W, (const cx<double>*)psi, (cx<double>*)out, epi, e, st));
   } else {
-    EpiArgs<float> e{(const cx<float>*)y, nullptr, ra, &dst->ticket[0], nullptr};
-    if (prec == OK_F32) OK_TRY(launch_apply<float>(W, (const cx<float>*)psi, (cx<float>*)out, epi, e, st));
-    else OK_TRY(launch_apply_w16(W, (const cx<float>*)psi, (cx<float>*)out, epi, e, st));
+    // as the FP32 iteration runs it: the plain application, then its inner products
+    const EpiArgs<float> e{};
+    if (prec == OK_F32) OK_TRY(launch_apply<float>(W, (const cx<float>*)psi, (cx<float>*)out, EPI_NONE, e, st));
+    else OK_TRY(launch_apply_w16(W, (const cx<float>*)psi, (cx<float>*)out, EPI_NONE, e, st));
+    const bool ts = kind == 2;  // <out, y>, <out, out>, else <y, out>
+    OK_TRY(launch_dots<float>((const cx<float>*)(ts ? out : y), (const cx<float>*)(ts ? y : out), 12LL * W->g.V, ts, dst, part, st,
+                              FIN_NONE));
   }
   OK_TRY(read_state(dst, hs.h, st));
   for (int k = 0; k < 3; ++k) sums[k] = kind == 1 && k == 2 ? 0.0 : hs.h->aux[k];
