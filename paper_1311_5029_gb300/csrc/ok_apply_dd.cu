@@ -1,23 +1,22 @@
-// FP64-accurate M psi on the FP32 pipes: double-float W (OK_W_DF64) and fields, one thread per
-// site, the stencil walked as a table.
+// FP64-accurate M psi on the FP32 pipes: double-float W (OK_W_DF64) and fields.
 //
-// The operator is the one of the other apply kernels (Eq. minFlopForm in the spin basis where
-// every hop except W^0 is block diagonal in h+- = u +- l; see ok_apply.cu): per site 27 offsets
-// and 148 colour matrix-vector products y = V h or V^dag h, each added to one or two of the four
-// accumulators acc+-(spin 0, 1) with a factor 1, a_ii or b_ii times a unit (+-1, +-i, +-1 +- i).
-// Written out with every product inlined, that is about 100 K FP32 instructions of straight-line
-// code per thread in double-float arithmetic, far beyond the instruction caches.  Here the
-// products are entries of a table in the kernel's parameter space and one compact loop body
-// executes them: the offset's neighbour spinor is gathered once into shared memory (three
-// half-spinor slots per thread), then every entry loads its matrix, multiplies and accumulates.
-// All threads of a block walk the same entries, so the table reads and the branches on an
-// entry's fields are uniform.
+// A block takes a 32-site tile of W; its four warps take the four sums per site of ok_dd_entries.cuh, lane
+// = site, and walk their 37 products with one compact loop body: gather one or two spin components of
+// the neighbour, combine them, multiply by the matrix, add to the warp's one sum.  All of a warp's
+// lanes walk the same entry, so the table reads and the branches on an entry's fields are uniform.
 //
 // Double-float: a row of a product sums six real products with TwoProd and TwoSum, deferring the
-// renormalisation to the end of the row (Joldes, Muller, Popescu, ACM TOMS 44 (2017), the
-// building blocks of ok_internal.cuh); accumulators are renormalised at every addition.
+// renormalisation to the addition of the row to the sum (Joldes, Muller, Popescu, ACM TOMS 44 (2017),
+// the building blocks of ok_internal.cuh).  Real and imaginary parts go through the same sequence
+// side by side, as the two halves of packed FP32 operations.
+//
+// What bounds it: the FP32 pipe, about 520 slots of packed operations per product and lane.  One thread
+// per site with four sums, up to two destinations and a scalar per product, and scalar operations took
+// 120 k instructions per site (issue 72 % busy): 602 us at 16^3 x 32 with x's conversion, now 475 us, and
+// the error against 64 bits 3.2e-15 instead of 8.9e-15 (fewer sums).
 #include "ok_dd.cuh"
-#include "ok_dd_table.cuh"
+#include "ok_dd_entries.cuh"
+#include "ok_split.cuh"
 
 namespace okgb {
 
@@ -25,98 +24,81 @@ namespace {
 
 constexpr int DD_THREADS = 128;
 #ifndef OK_DD_MINB
-#define OK_DD_MINB 4
+#define OK_DD_MINB 5   // 475 us at 16^3 x 32 with x's conversion; 482 and 516 us at 4 and 3 blocks per SM
 #endif
 
-using namespace ddtab;
+using namespace ddent;
 
-// ---------------------------------------------------------------------------- double-float pieces
-__device__ __forceinline__ cx<dd> ld4(const float4* p) {
-  const float4 v = __ldg(p);
-  return mk(dd(v.x, v.y), dd(v.z, v.w));
+// ---------------------------------------------------------------------------- packed double-float
+// A complex double-float: hi = (re.hi, im.hi), lo = (re.lo, im.lo).
+struct P2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+// a - b (one rounding: the product by -1 is exact)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ P2 norm2(float2 s, float2 e) {
+  P2 r;
+  r.hi = add2(s, e);
+  r.lo = sub2(e, sub2(r.hi, s));
+  return r;
 }
-// (s, t) = a * b as an unnormalised pair: s the rounded product of the high parts, t the rest.
-__device__ __forceinline__ void prod_first(float& s, float& t, dd a, dd b) {
-  s = a.hi * b.hi;
-  t = fmaf(a.hi, b.hi, -s);
-  t = fmaf(a.hi, b.lo, t);
-  t = fmaf(a.lo, b.hi, t);
+// a + (s, e), e the unnormalised low part
+__device__ __forceinline__ P2 add_row(P2 a, float2 s, float2 e) {
+  const float2 t = add2(a.hi, s), bb = sub2(t, a.hi);
+  float2 r = add2(sub2(a.hi, sub2(t, bb)), sub2(s, bb));
+  r = add2(r, add2(a.lo, e));
+  return norm2(t, r);
 }
-// (s, t) += a * b: TwoSum of the high parts, every low-order term into t.
-__device__ __forceinline__ void prod_acc(float& s, float& t, dd a, dd b) {
-  const float p = a.hi * b.hi;
-  float e = fmaf(a.hi, b.hi, -p);
-  e = fmaf(a.hi, b.lo, e);
-  e = fmaf(a.lo, b.hi, e);
-  const float s2 = s + p;
-  const float bb = s2 - s;
-  t += (s - (s2 - bb)) + (p - bb);
-  t += e;
+__device__ __forceinline__ P2 add(P2 a, P2 b) { return add_row(a, b.hi, b.lo); }
+__device__ __forceinline__ float2 flip2(float2 a, unsigned mx, unsigned my) {
+  return f2(__uint_as_float(__float_as_uint(a.x) ^ mx), __uint_as_float(__float_as_uint(a.y) ^ my));
+}
+__device__ __forceinline__ P2 flip(P2 a, unsigned mx, unsigned my) { return P2{flip2(a.hi, mx, my), flip2(a.lo, mx, my)}; }
+// i^k a (exact)
+__device__ __forceinline__ P2 times_i(P2 a, int k) {
+  const bool sw = k & 1;
+  const unsigned mr = ((k + 1) & 2) ? 0x80000000u : 0u, mi = (k & 2) ? 0x80000000u : 0u;
+  const P2 b = sw ? P2{f2(a.hi.y, a.hi.x), f2(a.lo.y, a.lo.x)} : a;
+  return flip(b, mr, mi);
+}
+// a times the real double-float f
+__device__ __forceinline__ P2 scale(P2 a, dd f) {
+  const float2 fh = f2(f.hi, f.hi), fl = f2(f.lo, f.lo), q = __fmul2_rn(a.hi, f2(-f.hi, -f.hi));  // -product
+  float2 e = __ffma2_rn(a.hi, fh, q);
+  e = __ffma2_rn(a.hi, fl, e);
+  e = __ffma2_rn(a.lo, fh, e);
+  return norm2(f2(-q.x, -q.y), e);
+}
+// (s, t) = or += a b by components: q is the negated product of the high parts (na = -a.hi).
+__device__ __forceinline__ void prod_first(float2& s, float2& t, float2 ah, float2 na, float2 al, float2 bh, float2 bl) {
+  s = __fmul2_rn(ah, bh);
+  const float2 q = __fmul2_rn(na, bh);
+  t = __ffma2_rn(ah, bh, q);
+  t = __ffma2_rn(ah, bl, t);
+  t = __ffma2_rn(al, bh, t);
+}
+__device__ __forceinline__ void prod_acc(float2& s, float2& t, float2 ah, float2 na, float2 al, float2 bh, float2 bl) {
+  const float2 q = __fmul2_rn(na, bh);
+  float2 e = __ffma2_rn(ah, bh, q);
+  e = __ffma2_rn(ah, bl, e);
+  e = __ffma2_rn(al, bh, e);
+  const float2 s2 = sub2(s, q), bb = sub2(s2, s);
+  t = add2(t, sub2(sub2(s, sub2(s2, bb)), add2(q, bb)));  // (s - (s2 - bb)) + (p - bb)
+  t = add2(t, e);
   s = s2;
 }
-__device__ __forceinline__ dd dneg(dd a) { return dd(-a.hi, -a.lo); }
 
-__device__ __forceinline__ dd dflip(dd a, unsigned m) {
-  return dd(__uint_as_float(__float_as_uint(a.hi) ^ m), __uint_as_float(__float_as_uint(a.lo) ^ m));
-}
-
-// y = V v, or V^dag v when adj, for the matrix at wp (element e at wp + e * LANES).  One body for
-// both forms: the adjoint reads element (c, r) for (r, c) and flips the sign of its imaginary
-// part; a row's three elements are loaded as the row starts.
-__device__ __forceinline__ void matvec(const float4* __restrict__ wp, bool adj, const cx<dd> (&v)[3], cx<dd> (&y)[3]) {
-  const int sr = adj ? 1 : 3, sc = adj ? 3 : 1;
-  const unsigned cj = adj ? 0x80000000u : 0u;
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    cx<dd> e[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      e[c] = ld4(wp + (r * sr + c * sc) * LANES);
-      e[c].im = dflip(e[c].im, cj);
-    }
-    float sr_, tr, si, ti_;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      // (a.re v.re - a.im v.im) + i (a.re v.im + a.im v.re)
-      if (c == 0) {
-        prod_first(sr_, tr, e[c].re, v[c].re);
-        prod_first(si, ti_, e[c].re, v[c].im);
-      } else {
-        prod_acc(sr_, tr, e[c].re, v[c].re);
-        prod_acc(si, ti_, e[c].re, v[c].im);
-      }
-      prod_acc(sr_, tr, dneg(e[c].im), v[c].im);
-      prod_acc(si, ti_, e[c].im, v[c].re);
-    }
-    y[r] = mk(dd_renorm(sr_, tr), dd_renorm(si, ti_));
-  }
-}
-
-// w = unit x y for the units 1, i, -1, -i (codes 0..3: a quarter turn per step, exact) and
-// 1 + i, 1 - i, -1 - i, -1 + i (codes 4..7: g (1 + s i), s = -1 for odd codes, g = -1 from 6 on).
-__device__ __forceinline__ void times_unit(const cx<dd> (&y)[3], int u, cx<dd> (&w)[3]) {
-  if (u < 4) {
-    const bool sw = u & 1;
-    const unsigned mr = (((u + 1) >> 1) & 1) ? 0x80000000u : 0u, mi = ((u >> 1) & 1) ? 0x80000000u : 0u;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) w[k] = mk(dflip(sw ? y[k].im : y[k].re, mr), dflip(sw ? y[k].re : y[k].im, mi));
-  } else {
-    const unsigned ms = (u & 1) ? 0x80000000u : 0u, mg = (u & 2) ? 0x80000000u : 0u;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      w[k] = mk(dflip(y[k].re - dflip(y[k].im, ms), mg), dflip(y[k].im + dflip(y[k].re, ms), mg));
-  }
-}
-
-// Neighbour x + d of the site with coordinates c, with the fermion sign of every wrap across an
-// antiperiodic boundary (|d_mu| <= 2, so at most two wraps per direction).
-__device__ __forceinline__ int nbr_of(const int (&c)[4], const Geom& g, const DDHop& hop, bool& neg) {
+// Neighbour x + d with the fermion sign of every wrap across an antiperiodic boundary (|d_mu| <= 2, so at
+// most two wraps per direction).
+__device__ __forceinline__ int nbr_of(const int (&c)[4], const Geom& g, const signed char* d, bool& neg) {
   int n = 0;
   neg = false;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const int L = g.L[mu];
-    int x = c[mu] + hop.d[mu];
+    int x = c[mu] + d[mu];
     int wraps = 0;
     if (x >= L) { x -= L; wraps = 1; if (x >= L) { x -= L; wraps = 2; } }
     if (x < 0) { x += L; wraps = 1; if (x < 0) { x += L; wraps = 2; } }
@@ -126,196 +108,200 @@ __device__ __forceinline__ int nbr_of(const int (&c)[4], const Geom& g, const DD
   return n;
 }
 
-// Prefetch into L1 (no registers held): the next entry's matrix, the next offset's spinor.
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
-__device__ __forceinline__ const float4* wmat_dd(const float4* W, int site, int m) {
-  return W + ((size_t)(site >> 5) * NMAT + m) * (9 * LANES) + (site & 31);
+// Fields of the apply: per block of 32 sites, component k = 3 spin + colour of lane l is the 16-byte word
+// (re.hi, im.hi, re.lo, im.lo) at (blk * 12 + k) * 32 + l, so a warp's gather of one component is a run of
+// consecutive words.
+__device__ __forceinline__ const float4* field(const float4* psi, int n, int spin) {
+  return psi + ((size_t)(n >> 5) * 12 + 3 * spin) * LANES + (n & 31);
 }
-__device__ __forceinline__ void prefetch_mat(const float4* wp) {
-#pragma unroll
-  for (int e = 0; e < 9; ++e) prefetch_l1(wp + e * LANES);
-}
-
-__device__ __forceinline__ void add_to(cx<dd> (&acc)[3], const cx<dd> (&w)[3]) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) acc[k] = mk(acc[k].re + w[k].re, acc[k].im + w[k].im);
-}
+__device__ __forceinline__ P2 unpack(float4 v) { return P2{f2(v.x, v.y), f2(v.z, v.w)}; }
 
 // ---------------------------------------------------------------------------- the kernel
 template <int EPI>
 __global__ void __launch_bounds__(DD_THREADS, OK_DD_MINB)
     apply_dd_kernel(const float4* __restrict__ W, const float4* __restrict__ psi, double2* __restrict__ out, Geom g,
-                    dd c0q2, dd a_ii, dd b_ii, const double2* __restrict__ rhs, RedArgs ra, unsigned* ticket,
-                    const int* halt, const __grid_constant__ DDTable tab) {
+                    dd c0q4, dd two_big, dd two_r, int a_big, const double2* __restrict__ rhs, RedArgs ra, unsigned* ticket,
+                    const int* halt, const __grid_constant__ Table tab) {
   if (EPI != EPI_NONE && halt && *halt) return;
-  // Three half-spinor slots per thread, [slot * 6 + spin * 3 + colour][thread]: a thread's
-  // accesses to one entry hit consecutive 16-byte words across the warp.
-  __shared__ float4 slot[18][DD_THREADS];
-  const int tid = threadIdx.x;
-  const int s = blockIdx.x * DD_THREADS + tid;
-  double red[2] = {0.0, 0.0};
-  if (s < g.V) {
-    int c[4];
+  __shared__ float4 sh[2][4][3][LANES];   // the S and O sums of the four warps
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int s0 = blockIdx.x * LANES + lane;
+  const int s = s0 < g.V ? s0 : g.V - 1;   // lanes past the last site repeat it and store nothing
+  int c[4];
+  {
+    int r = s;
+    c[0] = r % g.L[0]; r /= g.L[0];
+    c[1] = r % g.L[1]; r /= g.L[1];
+    c[2] = r % g.L[2]; c[3] = r / g.L[2];
+  }
+  P2 acc[3], D[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) acc[k] = P2{f2(0.f, 0.f), f2(0.f, 0.f)};
+  int hop = -1, n = s;
+  bool neg = false;
+#pragma unroll 1
+  for (int i = 0; i < N_ALL; ++i) {
+    const Entry E = tab.e[w][i];
+    if (E.hop != hop) {
+      hop = E.hop;
+      n = nbr_of(c, g, tab.d[hop], neg);
+    }
+    const bool adj = E.flags & 1;
+    const int site = adj ? n : s;
+    const float4* wp = W + ((size_t)(site >> 5) * NMAT + E.m) * (9 * LANES) + (site & 31);
+    const int unit = E.src >> 4;
+    float4 ve[9];
+    // the matrix in the order of use: row r's elements (r, c), of the adjoint (c, r)
+    const int sr = adj ? 1 : 3, sc = adj ? 3 : 1;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) ve[3 * r + k] = __ldg(wp + (r * sr + k * sc) * LANES);
+    P2 v[3];
     {
-      int r = s;
-      c[0] = r % g.L[0]; r /= g.L[0];
-      c[1] = r % g.L[1]; r /= g.L[1];
-      c[2] = r % g.L[2]; c[3] = r / g.L[2];
-    }
-    cx<dd> acc0[3], acc1[3], acc2[3], acc3[3];
-    bool neg_next;
-    int n_next = nbr_of(c, g, tab.hop[0], neg_next);
-#pragma unroll 1
-    for (int hh = 0; hh < DD_HOPS; ++hh) {
-      const DDHop hop = tab.hop[hh];
-      const int n = n_next;
-      const bool neg = neg_next;
-      // the next offset's neighbour: its spinor is prefetched now, its first matrix with this
-      // offset's last entry
-      if (hh + 1 < DD_HOPS) {
-        n_next = nbr_of(c, g, tab.hop[hh + 1], neg_next);
-        const float4* pn = psi + (size_t)n_next * 12;
-        prefetch_l1(pn);
-        prefetch_l1(pn + 8);
-        prefetch_l1(pn + 11);
-      }
-      {
-        const float4* pp = psi + (size_t)n * 12;
-        cx<dd> v[12];
+      const float4* p1 = field(psi, n, E.src & 3);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          v[k] = ld4(pp + k);
-          if (neg) v[k] = mk(dneg(v[k].re), dneg(v[k].im));
-        }
+      for (int k = 0; k < 3; ++k) v[k] = unpack(__ldg(p1 + k * LANES));
+      if (unit) {
+        const float4* p2 = field(psi, n, (E.src >> 2) & 3);
+        P2 y[3];
 #pragma unroll
-        for (int q = 0; q < 2; ++q)
+        for (int k = 0; k < 3; ++k) y[k] = times_i(unpack(__ldg(p2 + k * LANES)), unit - 1);
+        if (i < N_TWO) {
+          // a psi_s1 + b y = two_big (psi_s1 + r y), or two_big (r psi_s1 + y) when b is the larger
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            const cx<dd> u = v[3 * q + k], l = v[3 * (q + 2) + k];
-            cx<dd> h0, h1;
-            if (hop.kind == DD_ONSITE) {
-              h0 = mk(u.re + l.im, u.im - l.re);  // u - i l
-              h1 = mk(u.re - l.im, u.im + l.re);  // u + i l
-            } else {
-              h0 = mk(u.re + l.re, u.im + l.im);
-              h1 = mk(u.re - l.re, u.im - l.im);
-            }
-            slot[0 * 6 + 3 * q + k][tid] = make_float4(h0.re.hi, h0.re.lo, h0.im.hi, h0.im.lo);
-            slot[1 * 6 + 3 * q + k][tid] = make_float4(h1.re.hi, h1.re.lo, h1.im.hi, h1.im.lo);
-            if (hop.kind == DD_THIRD_L || hop.kind == DD_THIRD_U) {
-              const cx<dd> t3 = hop.kind == DD_THIRD_L ? l : u;
-              slot[2 * 6 + 3 * q + k][tid] = make_float4(t3.re.hi, t3.re.lo, t3.im.hi, t3.im.lo);
-            }
-          }
-        if (hop.kind == DD_ONSITE) {
-          // the c0q part of W^0: acc+ = 2 c0q (u + l), acc- = 2 c0q (u - l)
-#pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const cx<dd> u0 = v[k], u1 = v[3 + k], l0 = v[6 + k], l1 = v[9 + k];
-            acc0[k] = mk(c0q2 * (u0.re + l0.re), c0q2 * (u0.im + l0.im));
-            acc1[k] = mk(c0q2 * (u1.re + l1.re), c0q2 * (u1.im + l1.im));
-            acc2[k] = mk(c0q2 * (u0.re - l0.re), c0q2 * (u0.im - l0.im));
-            acc3[k] = mk(c0q2 * (u1.re - l1.re), c0q2 * (u1.im - l1.im));
+            if (a_big) y[k] = scale(y[k], two_r);
+            else v[k] = scale(v[k], two_r);
           }
         }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = add(v[k], y[k]);
       }
-      const int a_end = hop.first + hop.count;
-#pragma unroll 1
-      for (int ai = hop.first; ai < a_end; ++ai) {
-        const DDAct A = tab.act[ai];
-        const int ws = (A.flags & 1) ? n : s;
-        const int src = A.flags >> 2;
-        const float4* wp = wmat_dd(W, ws, A.m);
-        if (ai + 1 < a_end) {
-          const DDAct B = tab.act[ai + 1];
-          prefetch_mat(wmat_dd(W, (B.flags & 1) ? n : s, B.m));
-        } else if (hh + 1 < DD_HOPS) {
-          const DDAct B = tab.act[tab.hop[hh + 1].first];
-          prefetch_mat(wmat_dd(W, (B.flags & 1) ? n_next : s, B.m));
-        }
-        cx<dd> v[3], y[3];
+      const unsigned m = (neg != ((E.flags & 2) != 0)) ? 0x80000000u : 0u;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const float4 f = slot[src * 3 + k][tid];
-          v[k] = mk(dd(f.x, f.y), dd(f.z, f.w));
-        }
-        matvec(wp, A.flags & 2, v, y);
-        // the one or two accumulators, each with its scalar and unit (a rolled loop: one copy of
-        // the code)
-#pragma unroll 1
-        for (int j = 0; j < 2; ++j) {
-          const int d = j ? A.dst[1] : A.dst[0];
-          if (d < 0) break;
-          const int mul = j ? A.mul[1] : A.mul[0];
-          const int sc = mul & 3, un = mul >> 2;
-          cx<dd> w[3];
-          times_unit(y, un, w);
-          if (sc != S1) {
-            const dd f = sc == SA ? a_ii : b_ii;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) w[k] = mk(f * w[k].re, f * w[k].im);
-          }
-          switch (d) {
-            case 0: add_to(acc0, w); break;
-            case 1: add_to(acc1, w); break;
-            case 2: add_to(acc2, w); break;
-            default: add_to(acc3, w); break;
-          }
-        }
-      }
+      for (int k = 0; k < 3; ++k) v[k] = flip(v[k], m, m);
     }
-    // out_u = acc+ + acc-, out_l = acc+ - acc-, rounded to FP64
-    double2* op = out + (size_t)s * 12;
-    const double2* bp = EPI == EPI_RESID ? rhs + (size_t)s * 12 : nullptr;
+    const unsigned cj = adj ? 0x80000000u : 0u;
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
+    for (int r = 0; r < 3; ++r) {
+      float2 S, T;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const cx<dd> p = q == 0 ? acc0[k] : acc1[k];
-        const cx<dd> m = q == 0 ? acc2[k] : acc3[k];
-        const cx<dd> up = mk(p.re + m.re, p.im + m.im), lo = mk(p.re - m.re, p.im - m.im);
-        double2 ou = make_double2((double)up.re, (double)up.im);
-        double2 ol = make_double2((double)lo.re, (double)lo.im);
-        if (EPI == EPI_RESID) {
-          const double2 bu = bp[3 * q + k], bl = bp[3 * (q + 2) + k];
-          ou = make_double2(bu.x - ou.x, bu.y - ou.y);
-          ol = make_double2(bl.x - ol.x, bl.y - ol.y);
-          red[0] += ou.x * ou.x + ou.y * ou.y + ol.x * ol.x + ol.y * ol.y;
-          red[1] += bu.x * bu.x + bu.y * bu.y + bl.x * bl.x + bl.y * bl.y;
-        }
-        op[3 * q + k] = ou;
-        op[3 * (q + 2) + k] = ol;
+        const float4 e = ve[3 * r + k];   // (re.hi, re.lo, im.hi, im.lo)
+        const float ih = __uint_as_float(__float_as_uint(e.z) ^ cj), il = __uint_as_float(__float_as_uint(e.w) ^ cj);
+        const float2 ah = f2(e.x, e.x), an = f2(-e.x, -e.x), al = f2(e.y, e.y);
+        if (k == 0) prod_first(S, T, ah, an, al, v[k].hi, v[k].lo);
+        else prod_acc(S, T, ah, an, al, v[k].hi, v[k].lo);
+        // i im times (re, im) = im times (-im, re)
+        prod_acc(S, T, f2(-ih, ih), f2(ih, -ih), f2(-il, il), f2(v[k].hi.y, v[k].hi.x), f2(v[k].lo.y, v[k].lo.x));
       }
+      acc[r] = add_row(acc[r], S, T);
+    }
+    if (i == N_TWO - 1) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) acc[k] = scale(acc[k], two_big);
+    } else if (i == N_D - 1) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        D[k] = acc[k];
+        acc[k] = P2{f2(0.f, 0.f), f2(0.f, 0.f)};
+      }
+    } else if (i == N_S - 1) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sh[0][w][k][lane] = make_float4(acc[k].hi.x, acc[k].hi.y, acc[k].lo.x, acc[k].lo.y);
+        acc[k] = P2{f2(0.f, 0.f), f2(0.f, 0.f)};
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) sh[1][w][k][lane] = make_float4(acc[k].hi.x, acc[k].hi.y, acc[k].lo.x, acc[k].lo.y);
+  __syncthreads();
+  // out_u = S+ + S- + 2 D + 2 (A + B) + 4 c0q u,  out_l = S+ - S- + 2 D + 2 i (A - B) + 4 c0q l
+  double red[2] = {0.0, 0.0};
+  const int h = w >> 1, q = w & 1;
+  const float4* pp = field(psi, s, w);
+  double2* op = out + (size_t)s * 12 + 3 * w;
+  const double2* bp = EPI == EPI_RESID ? rhs + (size_t)s * 12 + 3 * w : nullptr;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const unsigned m = h ? 0x80000000u : 0u;
+    const P2 S = add(unpack(sh[0][q][k][lane]), flip(unpack(sh[0][2 + q][k][lane]), m, m));
+    P2 O = add(unpack(sh[1][q][k][lane]), flip(unpack(sh[1][2 + q][k][lane]), m, m));
+    if (h) O = times_i(O, 1);
+    P2 X = add(D[k], O);
+    X = P2{add2(X.hi, X.hi), add2(X.lo, X.lo)};
+    X = add(X, add(S, scale(unpack(__ldg(pp + k * LANES)), c0q4)));
+    double2 o = make_double2((double)X.hi.x + (double)X.lo.x, (double)X.hi.y + (double)X.lo.y);
+    if (EPI == EPI_RESID) {
+      const double2 b = bp[k];
+      o = make_double2(b.x - o.x, b.y - o.y);
+      if (s0 < g.V) {
+        red[0] += o.x * o.x + o.y * o.y;
+        red[1] += b.x * b.x + b.y * b.y;
+      }
+    }
+    if (s0 < g.V) op[k] = o;
   }
   if (EPI == EPI_RESID) grid_reduce<2, DD_THREADS>(red, ra, ticket);
 }
 
-// The table, built once on the host.
-const DDTable& dd_table() {
-  static const DDTable t = build_table();
+// FP64 canonical field -> the apply's fields (zero past the last site).
+__global__ void __launch_bounds__(384) to_dd_field_kernel(const double2* __restrict__ in, float4* __restrict__ out, int V) {
+  __shared__ float4 t[12 * LANES + 12];
+  const int i = threadIdx.x;                         // site i / 12 of the block, component i % 12
+  const size_t base = (size_t)blockIdx.x * (12 * LANES);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (base + i < (size_t)V * 12) {
+    const double2 d = in[base + i];
+    const dd re = split_df(d.x), im = split_df(d.y);
+    v = make_float4(re.hi, im.hi, re.lo, im.lo);
+  }
+  t[(i % 12) * (LANES + 1) + i / 12] = v;
+  __syncthreads();
+  out[base + i] = t[(i / LANES) * (LANES + 1) + (i & 31)];
+}
+
+const Table& dd_entries() {
+  static const Table t = build();
   return t;
 }
 
 }  // namespace
 
-int launch_apply_dd(const ok_W* Wh, const cx<dd>* psi_df, cx<double>* out, int epi, const EpiArgs<dd>& ep, cudaStream_t st) {
+size_t dd_field_bytes(const ok_W* W) { return (size_t)W->g.nblk * 12 * LANES * 16; }
+
+int launch_to_dd_field(const ok_W* W, const cx<double>* in, void* out, cudaStream_t st) {
+  {
+    TraceScope ts("to_df64", st);
+    to_dd_field_kernel<<<W->g.nblk, 12 * LANES, 0, st>>>((const double2*)in, (float4*)out, W->g.V);
+  }
+  OK_LAUNCH_CHECK();
+  return OK_SUCCESS;
+}
+
+int launch_apply_dd(const ok_W* Wh, const void* psi_dd, cx<double>* out, int epi, const EpiArgs<dd>& ep, cudaStream_t st) {
   if (!Wh->Wdf || (epi != EPI_NONE && epi != EPI_RESID)) return OK_EINVAL;
   if (epi == EPI_RESID && !ep.b) return OK_EINVAL;
-  const DDTable& tab = dd_table();
-  if (tab.hop[0].count == 0) return OK_EINTERNAL;
+  const Table& tab = dd_entries();
   const Geom& g = Wh->g;
-  const int nb = grid_for(g.V, DD_THREADS);
-  const dd c0q2(2.0 * Wh->sc.c0q), a(Wh->sc.a_ii), b(Wh->sc.b_ii);
+  const double a = Wh->sc.a_ii, b = Wh->sc.b_ii;
+  const int a_big = fabs(a) >= fabs(b);
+  const double big = a_big ? a : b, small = a_big ? b : a;
+  const dd c0q4(4.0 * Wh->sc.c0q), two_big(big), two_r(big != 0.0 ? small / big : 0.0);
   const float4* W = reinterpret_cast<const float4*>(Wh->Wdf);
-  const float4* psi = reinterpret_cast<const float4*>(psi_df);
+  const float4* psi = reinterpret_cast<const float4*>(psi_dd);
   double2* o = reinterpret_cast<double2*>(out);
   const double2* rhs = reinterpret_cast<const double2*>(ep.b);
   {
     TraceScope ts(epi == EPI_RESID ? "apply_df64_resid" : "apply_df64", st);
     if (epi == EPI_RESID)
-      apply_dd_kernel<EPI_RESID><<<nb, DD_THREADS, 0, st>>>(W, psi, o, g, c0q2, a, b, rhs, ep.ra, ep.ticket, ep.halt, tab);
+      apply_dd_kernel<EPI_RESID><<<g.nblk, DD_THREADS, 0, st>>>(W, psi, o, g, c0q4, two_big, two_r, a_big, rhs, ep.ra, ep.ticket,
+                                                                ep.halt, tab);
     else
-      apply_dd_kernel<EPI_NONE><<<nb, DD_THREADS, 0, st>>>(W, psi, o, g, c0q2, a, b, rhs, ep.ra, ep.ticket, ep.halt, tab);
+      apply_dd_kernel<EPI_NONE><<<g.nblk, DD_THREADS, 0, st>>>(W, psi, o, g, c0q4, two_big, two_r, a_big, rhs, ep.ra, ep.ticket,
+                                                               ep.halt, tab);
   }
   OK_LAUNCH_CHECK();
   return OK_SUCCESS;

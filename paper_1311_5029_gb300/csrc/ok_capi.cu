@@ -141,11 +141,11 @@ int ok_apply_M(const ok_W* W, ok_prec prec, const void* psi, void* out, void* st
     // double-float copy: convert psi into stream-ordered scratch, apply, release the scratch
     cudaStream_t st = (cudaStream_t)stream;
     void* psi_df = nullptr;
-    OK_CUDA_TRY(cudaMallocAsync(&psi_df, bytes, st));
-    int rc = launch_to_df((const cx<double>*)psi, (cx<dd>*)psi_df, 12LL * W->g.V, st);
+    OK_CUDA_TRY(cudaMallocAsync(&psi_df, dd_field_bytes(W), st));
+    int rc = launch_to_dd_field(W, (const cx<double>*)psi, psi_df, st);
     if (rc == OK_SUCCESS) {
       EpiArgs<dd> e{};
-      rc = launch_apply_dd(W, (const cx<dd>*)psi_df, (cx<double>*)out, EPI_NONE, e, st);
+      rc = launch_apply_dd(W, psi_df, (cx<double>*)out, EPI_NONE, e, st);
     }
     cudaError_t fe = cudaFreeAsync(psi_df, st);
     if (rc == OK_SUCCESS && fe != cudaSuccess) { set_cuda_error(fe); rc = OK_ECUDA; }

@@ -4,13 +4,17 @@
 
 namespace okgb {
 
+// The apply's input: a spinor field as double-float, in blocks of 32 sites (dd_field_bytes bytes).
+size_t dd_field_bytes(const ok_W* W);
+int launch_to_dd_field(const ok_W* W, const cx<double>* in, void* out, cudaStream_t st);
 // out = M psi (EPI_NONE) or out = b - M psi with <out, out>, <b, b> reduced (EPI_RESID), in
-// double-float arithmetic with the handle's OK_W_DF64 copy: psi double-float [V][12], b and out
-// FP64 [V][12].  OK_EINVAL without the copy or for another epilogue.
-int launch_apply_dd(const ok_W* W, const cx<dd>* psi_df, cx<double>* out, int epi, const EpiArgs<dd>& ep, cudaStream_t st);
+// double-float arithmetic with the handle's OK_W_DF64 copy: psi from launch_to_dd_field, b and out FP64
+// [V][12].  OK_EINVAL without the copy or for another epilogue.
+int launch_apply_dd(const ok_W* W, const void* psi_dd, cx<double>* out, int epi, const EpiArgs<dd>& ep, cudaStream_t st);
 
-// The stencil as the table the kernel walks: 27 offsets, each with its colour matrix-vector
-// products (built by ok_dd_table.cuh, passed to the kernel as a launch parameter).
+// The stencil as one list of 27 offsets with their colour matrix-vector products on the h+- halves
+// (ok_dd_table.cuh): the statement of the products that the entries of ok_dd_entries.cuh, which the
+// kernel walks, are tested against on the host.
 struct DDHop {
   signed char d[4];       // offset (x, y, z, t)
   unsigned char kind;     // DD_ONSITE, DD_PLAIN, DD_THIRD_L, DD_THIRD_U

@@ -87,8 +87,6 @@ int launch_tc_update_xr(cx<float>* x, const void* p16, const cx<float>* s, const
 int launch_tc_demote(const cx<double>* r64, cx<float>* r, cx<float>* rhat, cx<float>* p, int V, int nrhs, int k, bool restart,
                      SolverState* st, double* part, cudaStream_t strm);
 int launch_tc_accum(cx<double>* x64, cx<float>* x, int V, int nrhs, int k, cudaStream_t strm);
-// FP64 complex -> double-float complex (n complex numbers).
-int launch_to_df(const cx<double>* in, cx<dd>* out, long long n, cudaStream_t st);
 
 int blas_blocks(long long units);
 int sm_count();  // multiprocessors of the current device (cached)

@@ -146,13 +146,13 @@ int iterate(const ok_W* W, const IterBufs<R>& b, long long n, SolverState* dst, 
 }
 
 // out = b - M x in FP64 with |out|^2 in state aux[0] and |b|^2 in state bb (and aux[1]).  With the
-// double-float copy when the handle has one (x converted first into `xdf`, n complex double-floats
-// of scratch): on the FP32 pipes it is faster than the native FP64 copy, which is used otherwise.
+// double-float copy when the handle has one (x converted first into `xdf`, dd_field_bytes of scratch):
+// on the FP32 pipes it is faster than the native FP64 copy, which is used otherwise.
 int residual64(const ok_W* W, const cx<double>* bvec, const cx<double>* x, cx<double>* out, SolverState* dst, double* part,
-               cx<dd>* xdf, cudaStream_t st) {
+               void* xdf, cudaStream_t st) {
   if (W->Wdf) {
     if (!xdf) return OK_EINVAL;
-    OK_TRY(launch_to_df(x, xdf, 12LL * W->g.V, st));
+    OK_TRY(launch_to_dd_field(W, x, xdf, st));
     EpiArgs<dd> e{nullptr, reinterpret_cast<const cx<dd>*>(bvec), RedArgs{dst, part, nullptr, FIN_RESID}, &dst->ticket[5],
                   nullptr};
     return launch_apply_dd(W, xdf, out, EPI_RESID, e, st);
@@ -214,9 +214,9 @@ int bicgstab_impl(const ok_W* W, const cx<double>* bvec, cx<double>* x, const ok
   IterBufs<float> b32{};
   cx<double>* r64 = ws.get<cx<double>>(n, &err);
   if (!r64) { set_cuda_error(err); return OK_ENOMEM; }
-  cx<dd>* xdf = nullptr;
+  void* xdf = nullptr;
   if (W->Wdf) {
-    xdf = ws.get<cx<dd>>(n, &err);
+    xdf = ws.get<unsigned char>(dd_field_bytes(W), &err);
     if (!xdf) { set_cuda_error(err); return OK_ENOMEM; }
   }
   if (mode == OK_SOLVE_F64) {
@@ -353,7 +353,7 @@ int true_residual(const ok_W* W, const cx<double>* bvec, const cx<double>* x, do
   double* part = ws.get<double>((size_t)apply_blocks_needed(W) * 4, &err);
   SolverState* dst = ws.get<SolverState>(1, &err);
   cx<double>* r = ws.get<cx<double>>(n, &err);
-  cx<dd>* xdf = W->Wdf ? ws.get<cx<dd>>(n, &err) : nullptr;
+  void* xdf = W->Wdf ? ws.get<unsigned char>(dd_field_bytes(W), &err) : nullptr;
   HostState hs;
   if (!part || !dst || !r || !hs.h || (W->Wdf && !xdf)) { if (err != cudaSuccess) set_cuda_error(err); return OK_ENOMEM; }
   OK_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(SolverState), st));
@@ -488,7 +488,7 @@ int bicgstab_multi(const ok_W* W, int nrhs, const cx<double>* bvec, cx<double>* 
   if (tcp) OK_CUDA_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(unsigned), st));
   const int V = W->g.V;
   cx<double>* r64 = ws.get<cx<double>>(n, &err);
-  cx<dd>* xdf = W->Wdf ? ws.get<cx<dd>>(n, &err) : nullptr;
+  void* xdf = W->Wdf ? ws.get<unsigned char>(dd_field_bytes(W), &err) : nullptr;
   IterBufs<float> b{};
   b.x = ws.get<cx<float>>(N, &err); b.r = ws.get<cx<float>>(N, &err); b.rhat = ws.get<cx<float>>(N, &err);
   b.p = ws.get<cx<float>>(N, &err); b.v = ws.get<cx<float>>(N, &err); b.s = ws.get<cx<float>>(N, &err);
