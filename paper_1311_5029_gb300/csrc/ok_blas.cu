@@ -183,6 +183,213 @@ __global__ void __launch_bounds__(BLAS_THREADS) dots_kernel(const typename Unit<
   }
 }
 
+// ---------------------------------------------------------------------------- small systems
+// On a small lattice the five vector kernels of an FP32 iteration cost their launches, their grid
+// completions and their last block's tail, not their bytes (4^3 x 8: 36 us an iteration, 12 us of it
+// update_xr; now 25 us).  There one cluster of up to eight blocks does the work between two applications
+// in one launch: it takes the inner products, finalises the scalars and streams the update, with cluster
+// barriers in the place of kernel boundaries.  Block sums meet in the first block's shared memory and are
+// added in a fixed tree, so a solve is reproducible; the state is worked on in shared memory as well, as
+// its finalisation is one thread's chain of dependent accesses (20.0 -> 16.0 us for small_xrp).
+constexpr int CL_THREADS = 1024;
+constexpr int CL_MAX = 8;
+__device__ __forceinline__ unsigned cl_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ unsigned cl_size() { unsigned r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
+struct ClusterShared {
+  dd warp[3][CL_THREADS / 32];
+  dd part[3];
+  float sc[4];
+  int halt;
+  SolverState st;  // the first block's copy of the system's state: the finalisations work on it
+};
+static_assert(sizeof(SolverState) % 4 == 0 && sizeof(SolverState) / 4 <= CL_THREADS, "one word per thread");
+// Copies the state into the first block's shared memory, or back; every thread of the block calls it.
+__device__ __forceinline__ void cl_state(ClusterShared& sh, SolverState* st, bool load) {
+  if (cl_rank() != 0) return;
+  if (!load) __syncthreads();
+  if (threadIdx.x < sizeof(SolverState) / 4) {
+    unsigned* a = reinterpret_cast<unsigned*>(&sh.st) + threadIdx.x;
+    unsigned* b = reinterpret_cast<unsigned*>(st) + threadIdx.x;
+    if (load) *a = *b; else *b = *a;
+  }
+}
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A 32-bit word of shared memory at the same place in block `rank` of the cluster.
+__device__ __forceinline__ float cl_load(const void* p, unsigned rank) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), b;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(b) : "memory");
+  return v;
+}
+
+// Sums v over the cluster and finalises on sh.st; sc[0..3] and the halt flag as `publish` leaves them in the
+// first block's shared memory reach every block's.  Every thread of the cluster takes part.
+template <int NP, typename Publish>
+__device__ __forceinline__ void cl_finalise(dd (&v)[NP], ClusterShared& sh, int fin, Publish&& publish) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NP; ++k) {
+    dd x = v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = x + shfl_xor_dd(x, o);
+    if (lane == 0) sh.warp[k][warp] = x;
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      dd x = sh.warp[k][lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x = x + shfl_xor_dd(x, o);
+      if (lane == 0) sh.part[k] = x;
+    }
+  }
+  cl_sync();
+  const unsigned rank = cl_rank();
+  if (rank == 0 && warp == 0) {
+    double tot[4] = {0.0, 0.0, 0.0, 0.0};
+    dd x[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {   // lane r takes block r's sum
+      x[k] = dd(0.f, 0.f);
+      if (lane < (int)cl_size()) x[k] = dd(cl_load(&sh.part[k].hi, lane), cl_load(&sh.part[k].lo, lane));
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+#pragma unroll
+      for (int o = CL_MAX / 2; o > 0; o >>= 1) x[k] = x[k] + shfl_xor_dd(x[k], o);
+      tot[k] = (double)x[k];
+    }
+    if (lane == 0) {
+      finalise(&sh.st, fin, tot);
+      publish(sh.sc);
+      sh.halt = sh.st.halt;
+    }
+  }
+  cl_sync();
+  if (rank != 0 && threadIdx.x < 5) {
+    if (threadIdx.x < 4) sh.sc[threadIdx.x] = cl_load(&sh.sc[threadIdx.x], 0);
+    else sh.halt = __float_as_int(cl_load(&sh.halt, 0));
+  }
+  __syncthreads();
+}
+
+// <rhat, v> -> alpha;  s = r - alpha v.
+__global__ void __launch_bounds__(CL_THREADS, 1) small_s_kernel(const float4* __restrict__ rhat, const float4* __restrict__ v,
+                                                                const float4* __restrict__ r, float4* __restrict__ s, int nu,
+                                                                SolverState* __restrict__ st) {
+  __shared__ ClusterShared sh;
+  if (st->halt) return;  // set before this launch, so the same for every block
+  cl_state(sh, st, true);
+  using U = Unit<float>;
+  const int i0 = cl_rank() * CL_THREADS + threadIdx.x, step = cl_size() * CL_THREADS;
+  dd red[2] = {dd(0.f, 0.f), dd(0.f, 0.f)};
+  for (int i = i0; i < nu; i += step) {
+    cx<float> a[2], b[2], d = mk<float>(0, 0);
+    U::get(rhat[i], a);
+    U::get(v[i], b);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) d = fma_cj(a[k], b[k], d);
+    red_add(red[0], d.re);
+    red_add(red[1], d.im);
+  }
+  cl_finalise<2>(red, sh, FIN_ALPHA, [&](float* sc) { sc[0] = (float)sh.st.alpha.re; sc[1] = (float)sh.st.alpha.im; });
+  cl_state(sh, st, false);
+  if (!sh.halt) {
+    const cx<float> al = mk(sh.sc[0], sh.sc[1]);
+    for (int i = i0; i < nu; i += step) {
+      cx<float> a[2], b[2];
+      U::get(r[i], a);
+      U::get(v[i], b);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) a[k] = a[k] - al * b[k];
+      s[i] = U::put(a);
+    }
+  }
+  cl_sync();  // the first block's shared memory is read until here
+}
+
+// <t, s>, <t, t> -> omega;  x += alpha p + omega sx, r = s - omega t, <rhat, r>, <r, r> -> beta, convergence;
+// p = r + beta (p - omega v).  px, sx: the directions of the solution update (p and s, or P p and P s with a
+// right preconditioner P).
+__global__ void __launch_bounds__(CL_THREADS, 1) small_xrp_kernel(float4* __restrict__ x, float4* p, const float4* px,
+                                                                  const float4* __restrict__ s, const float4* sx,
+                                                                  const float4* __restrict__ t, float4* __restrict__ r,
+                                                                  const float4* __restrict__ rhat, const float4* __restrict__ v, int nu,
+                                                                  SolverState* __restrict__ st) {
+  __shared__ ClusterShared sh;
+  if (st->halt) return;
+  cl_state(sh, st, true);
+  using U = Unit<float>;
+  const int i0 = cl_rank() * CL_THREADS + threadIdx.x, step = cl_size() * CL_THREADS;
+  const cx<float> al = mk((float)st->alpha.re, (float)st->alpha.im);
+  dd red[3] = {dd(0.f, 0.f), dd(0.f, 0.f), dd(0.f, 0.f)};
+  for (int i = i0; i < nu; i += step) {
+    cx<float> a[2], b[2], d = mk<float>(0, 0);
+    float n2 = 0.f;
+    U::get(t[i], a);
+    U::get(s[i], b);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      d = fma_cj(a[k], b[k], d);
+      n2 += a[k].re * a[k].re + a[k].im * a[k].im;
+    }
+    red_add(red[0], d.re);
+    red_add(red[1], d.im);
+    red_add(red[2], n2);
+  }
+  cl_finalise<3>(red, sh, FIN_OMEGA, [&](float* sc) { sc[0] = (float)sh.st.omega.re; sc[1] = (float)sh.st.omega.im; });
+  const cx<float> om = mk(sh.sc[0], sh.sc[1]);
+  if (sh.halt) {  // the same in every block
+    cl_state(sh, st, false);
+    cl_sync();
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) red[k] = dd(0.f, 0.f);
+  for (int i = i0; i < nu; i += step) {
+    cx<float> xv[2], pv[2], sv[2], zv[2], tv[2], hv[2], d = mk<float>(0, 0);
+    float n2 = 0.f;
+    U::get(x[i], xv);
+    U::get(px[i], pv);
+    U::get(s[i], sv);
+    U::get(sx[i], zv);
+    U::get(t[i], tv);
+    U::get(rhat[i], hv);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      xv[k] = xv[k] + al * pv[k] + om * zv[k];
+      sv[k] = sv[k] - om * tv[k];
+      d = fma_cj(hv[k], sv[k], d);
+      n2 += sv[k].re * sv[k].re + sv[k].im * sv[k].im;
+    }
+    x[i] = U::put(xv);
+    r[i] = U::put(sv);
+    red_add(red[0], d.re);
+    red_add(red[1], d.im);
+    red_add(red[2], n2);
+  }
+  cl_sync();  // sc of omega is read; the sums' shared memory is free again
+  cl_finalise<3>(red, sh, FIN_XR, [&](float* sc) { sc[2] = (float)sh.st.beta.re; sc[3] = (float)sh.st.beta.im; });
+  cl_state(sh, st, false);
+  if (!sh.halt) {
+    const cx<float> be = mk(sh.sc[2], sh.sc[3]);
+    for (int i = i0; i < nu; i += step) {
+      cx<float> pv[2], rv[2], vv[2];
+      U::get(p[i], pv);
+      U::get(r[i], rv);
+      U::get(v[i], vv);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) pv[k] = rv[k] + be * (pv[k] - om * vv[k]);
+      p[i] = U::put(pv);
+    }
+  }
+  cl_sync();
+}
+
 // Restart: rhat = p = r (same precision), sum <r, r> -> FIN_RESTART.
 template <typename R>
 __global__ void __launch_bounds__(BLAS_THREADS) restart_kernel(const typename Unit<R>::T* __restrict__ r,
@@ -319,6 +526,53 @@ static int wave_blocks(K kern, long long units, bool reduces = false) {
 }
 
 template <typename R> long long units_of(long long ncomplex) { return ncomplex / Unit<R>::NC; }
+
+// One cluster of blocks, as many as give every thread a unit and a half, at most CL_MAX.
+// Up to 49152 units (8192 sites).  One solve, separate kernels / one cluster (us): 512 sites 2473 / 2088,
+// 4096 sites 2974 / 2516, 8192 sites 3192 / 3029, 16000 sites 3868 / 4347.
+constexpr long long CL_UNITS = 49152;
+bool small_system(long long n) { return units_of<float>(n) <= CL_UNITS; }
+
+template <typename... P, typename... A>
+static cudaError_t launch_cluster(void (*kern)(P...), int nu, cudaStream_t strm, A... args) {
+  int nr = (nu + CL_THREADS + CL_THREADS / 2 - 1) / (CL_THREADS + CL_THREADS / 2);
+  if (nr > CL_MAX) nr = CL_MAX;
+  if (nr < 1) nr = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nr);
+  cfg.blockDim = dim3(CL_THREADS);
+  cfg.stream = strm;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nr;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+int launch_small_s(const cx<float>* rhat, const cx<float>* v, const cx<float>* r, cx<float>* s, long long n, SolverState* st,
+                   cudaStream_t strm) {
+  const int nu = (int)units_of<float>(n);
+  {
+    TraceScope ts("small_s_f32", strm);
+    OK_CUDA_TRY(launch_cluster(small_s_kernel, nu, strm, (const float4*)rhat, (const float4*)v, (const float4*)r, (float4*)s, nu, st));
+  }
+  OK_LAUNCH_CHECK();
+  return OK_SUCCESS;
+}
+
+int launch_small_xrp(cx<float>* x, cx<float>* p, const cx<float>* px, const cx<float>* s, const cx<float>* sx, const cx<float>* t,
+                     cx<float>* r, const cx<float>* rhat, const cx<float>* v, long long n, SolverState* st, cudaStream_t strm) {
+  const int nu = (int)units_of<float>(n);
+  {
+    TraceScope ts("small_xrp_f32", strm);
+    OK_CUDA_TRY(launch_cluster(small_xrp_kernel, nu, strm, (float4*)x, (float4*)p, (const float4*)px, (const float4*)s,
+                               (const float4*)sx, (const float4*)t, (float4*)r, (const float4*)rhat, (const float4*)v, nu, st));
+  }
+  OK_LAUNCH_CHECK();
+  return OK_SUCCESS;
+}
 
 template <typename R>
 int launch_update_s(const cx<R>* r, const cx<R>* v, cx<R>* s, long long n, const SolverState* st, cudaStream_t strm) {

@@ -102,6 +102,13 @@ int launch_update_p(cx<R>* p, const cx<R>* r, const cx<R>* v, long long n, const
 template <typename R>
 int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm,
                 int fin = -1);
+// The work between two applications in one cluster launch each, for systems of few elements: the inner
+// product, alpha and s = r - alpha v; omega, x, r, beta and p.
+bool small_system(long long n);
+int launch_small_s(const cx<float>* rhat, const cx<float>* v, const cx<float>* r, cx<float>* s, long long n, SolverState* st,
+                   cudaStream_t strm);
+int launch_small_xrp(cx<float>* x, cx<float>* p, const cx<float>* px, const cx<float>* s, const cx<float>* sx, const cx<float>* t,
+                     cx<float>* r, const cx<float>* rhat, const cx<float>* v, long long n, SolverState* st, cudaStream_t strm);
 template <typename R>
 int launch_restart(const cx<R>* r, cx<R>* rhat, cx<R>* p, long long n, SolverState* st, double* part, cudaStream_t strm);
 int launch_demote(const cx<double>* r64, cx<float>* r32, cx<float>* rhat, cx<float>* p, long long n, bool restart,

@@ -15,9 +15,10 @@ struct dcx { double re, im; };
 
 __host__ __device__ __forceinline__ dcx dmk(double a, double b) { dcx z; z.re = a; z.im = b; return z; }
 __host__ __device__ __forceinline__ dcx dmul(dcx a, dcx b) { return dmk(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
+// One division: the finalisations run on one thread, where an FP64 division is a long chain.
 __host__ __device__ __forceinline__ dcx ddiv(dcx a, dcx b) {
-  double d = b.re * b.re + b.im * b.im;
-  return dmk((a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d);
+  const double d = 1.0 / (b.re * b.re + b.im * b.im);
+  return dmk((a.re * b.re + a.im * b.im) * d, (a.im * b.re - a.re * b.im) * d);
 }
 __host__ __device__ __forceinline__ double dabs2(dcx a) { return a.re * a.re + a.im * a.im; }
 __host__ __device__ __forceinline__ bool dfinite(dcx a) { return isfinite(a.re) && isfinite(a.im); }

@@ -42,8 +42,8 @@ __device__ __forceinline__ void block_sums_dd(dd (&v)[NP], dd (*sh)[THREADS / 32
   __syncthreads();
 }
 
-// grid_reduce (ok_reduce.cuh) in double-float: block partials stored as doubles (hi + lo, exact),
-// the last block sums them and finalises.
+// grid_reduce (ok_reduce.cuh) in double-float: block partials stored as pairs of floats in the slots of
+// the doubles (no FP64 conversion on the way), the last block sums them and finalises.
 template <int NP, int THREADS>
 __device__ __forceinline__ void grid_reduce_dd(dd (&v)[NP], const RedArgs& ra, unsigned* ticket) {
   __shared__ dd sh[NP][THREADS / 32];
@@ -51,7 +51,7 @@ __device__ __forceinline__ void grid_reduce_dd(dd (&v)[NP], const RedArgs& ra, u
   block_sums_dd<NP, THREADS>(v, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NP; ++k) ra.part[(size_t)blockIdx.x * NP + k] = (double)v[k];
+    for (int k = 0; k < NP; ++k) reinterpret_cast<float2*>(ra.part)[(size_t)blockIdx.x * NP + k] = make_float2(v[k].hi, v[k].lo);
     __threadfence();
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -63,7 +63,10 @@ __device__ __forceinline__ void grid_reduce_dd(dd (&v)[NP], const RedArgs& ra, u
   for (int k = 0; k < NP; ++k) w[k] = dd(0.f, 0.f);
   for (unsigned b = threadIdx.x; b < gridDim.x; b += THREADS)
 #pragma unroll
-    for (int k = 0; k < NP; ++k) w[k] = w[k] + dd(__ldcg(ra.part + (size_t)b * NP + k));
+    for (int k = 0; k < NP; ++k) {
+      const float2 f = __ldcg(reinterpret_cast<const float2*>(ra.part) + (size_t)b * NP + k);
+      w[k] = w[k] + dd(f.x, f.y);
+    }
   block_sums_dd<NP, THREADS>(w, sh);
   if (threadIdx.x == 0) {
     *ticket = 0u;

@@ -129,8 +129,14 @@ int iterate(const ok_W* W, const IterBufs<R>& b, long long n, SolverState* dst, 
   constexpr bool fused = sizeof(R) == 8;
   const EpiArgs<R> e1{b.rhat, nullptr, RedArgs{dst, part, nullptr, FIN_ALPHA}, &dst->ticket[0], &dst->halt};
   OK_TRY(apply_iter<R>(W, pin, b.v, fused ? EPI_DOT : EPI_NONE, e1, w16, st));
-  if (!fused) OK_TRY(launch_dots<R>(b.rhat, b.v, n, false, dst, part, st));
-  OK_TRY(launch_update_s<R>(b.r, b.v, b.s, n, dst, st));
+  bool small = false;
+  if constexpr (!fused) small = small_system(n);
+  if (small) {
+    if constexpr (!fused) OK_TRY(launch_small_s(b.rhat, b.v, b.r, b.s, n, dst, st));
+  } else {
+    if (!fused) OK_TRY(launch_dots<R>(b.rhat, b.v, n, false, dst, part, st));
+    OK_TRY(launch_update_s<R>(b.r, b.v, b.s, n, dst, st));
+  }
   if constexpr (sizeof(R) == 4) {
     if (pre) {
       OK_TRY(net_apply_unless_halted(pc.net, W, b.s, pc.zs, pc.halt, st));
@@ -139,7 +145,10 @@ int iterate(const ok_W* W, const IterBufs<R>& b, long long n, SolverState* dst, 
   }
   const EpiArgs<R> e2{nullptr, nullptr, RedArgs{dst, part, nullptr, FIN_OMEGA}, &dst->ticket[1], &dst->halt};
   OK_TRY(apply_iter<R>(W, sin, b.t, fused ? EPI_TS : EPI_NONE, e2, w16, st));
-  if (!fused) OK_TRY(launch_dots<R>(b.t, b.s, n, true, dst, part, st));
+  if constexpr (!fused) {
+    if (small) return launch_small_xrp(b.x, b.p, pin, b.s, sin, b.t, b.r, b.rhat, b.v, n, dst, st);
+    OK_TRY(launch_dots<R>(b.t, b.s, n, true, dst, part, st));
+  }
   OK_TRY(launch_update_xr<R>(b.x, pin, b.s, b.t, b.r, b.rhat, n, dst, part, st, pre ? sin : nullptr));
   OK_TRY(launch_update_p<R>(b.p, b.r, b.v, n, dst, st));
   return OK_SUCCESS;
