@@ -1,4 +1,4 @@
-// Double-float split of an FP64 value, for storing the OK_W_DF64 copy of W.
+// Conversions of FP64 values to narrower formats on the integer pipe.
 #pragma once
 #include <string.h>
 
@@ -6,43 +6,72 @@
 
 namespace okgb {
 
-// Double-float split of d: hi = RN_float(d), lo = RN_float(d - hi), the value dd(d) defines.  The
-// remainder is formed from the bits of d and hi with integer operations: GB300's FP64 pipe would
-// otherwise convert hi back, subtract and convert again for every stored component.  For
-// |d| in [2^-74, 2^127) (where lo is a normal float or zero) the result is bit for bit that of the
-// definition; outside that range, and for zero, the definition itself is used.
-__host__ __device__ __forceinline__ dd split_df(double d) {
-  const float hi = (float)d;
+// GB300's FP64 pipe, the conversions to and from FP64 with it, runs at 1/58 of the FP32 rate, so the
+// kernels that only pass FP64 data on are bound by their conversions.  These give bit for bit what
+// the conversion gives, from 32-bit integer operations, and use the conversion itself outside the
+// range where the integer form holds.
+__host__ __device__ __forceinline__ void double_words(double d, unsigned& hi, unsigned& lo) {
 #ifdef __CUDA_ARCH__
-  const long long D = __double_as_longlong(d);
-  const int H = __float_as_int(hi);
+  hi = (unsigned)__double2hiint(d);
+  lo = (unsigned)__double2loint(d);
 #else
-  long long D;
-  int H;
+  unsigned long long D;
   memcpy(&D, &d, sizeof D);
-  memcpy(&H, &hi, sizeof H);
+  hi = (unsigned)(D >> 32);
+  lo = (unsigned)D;
 #endif
-  const int ed = (int)((D >> 52) & 0x7ff);
-  if (ed < 1023 - 74 || ed > 1023 + 126) return dd(d);
-  // significands in units of 2^(ed - 1075): |d| = md, |hi| = mh (hi is d rounded to 24 bits, so it
-  // has d's exponent or, when d rounds up to a power of two, the next one)
-  const long long md = (D & ((1LL << 52) - 1)) | (1LL << 52);
-  const int eh = ((H >> 23) & 0xff) - 127 + 1023;
-  long long mh = (long long)((H & 0x7fffff) | 0x800000) << 29;
-  if (eh != ed) mh <<= 1;
-  int diff = (int)(md - mh);  // |diff| <= 2^28: half a float ulp
-  if (D < 0) diff = -diff;
-  // lo = diff * 2^(ed - 1075) (diff signed like d; zero stays +0), the power of two a normal float
-  const int scale_bits = (ed - 1075 + 127) << 23;
+}
+__host__ __device__ __forceinline__ float float_bits(unsigned u) {
 #ifdef __CUDA_ARCH__
-  const float scale = __int_as_float(scale_bits);
-  const float lo = __int2float_rn(diff) * scale;
+  return __uint_as_float(u);
 #else
-  float scale;
-  memcpy(&scale, &scale_bits, sizeof scale);
-  const float lo = (float)diff * scale;
+  float f;
+  memcpy(&f, &u, sizeof f);
+  return f;
 #endif
-  return dd(hi, lo);
+}
+
+// The 24 leading bits of |d|'s significand in place of a float's, biased exponent ed - 896 beside it; `low` the 29
+// bits that follow.  `ok`: |d| in [2^-74, 2^127).
+struct SplitBits {
+  unsigned top, low, sign, ed;
+  bool ok;
+};
+__host__ __device__ __forceinline__ SplitBits split_bits(double d) {
+  unsigned h, l;
+  double_words(d, h, l);
+  SplitBits s;
+  s.ed = (h >> 20) & 0x7ffu;
+  s.sign = h & 0x80000000u;
+  s.top = ((h & 0x7fffffffu) - (896u << 20)) << 3 | l >> 29;   // (exponent - 896) << 23 | 23 bits
+  s.low = l & 0x1fffffffu;
+  s.ok = s.ed - (1023u - 74u) <= 74u + 126u;
+  return s;
+}
+
+// d rounded to odd at 24 bits: rounding the result to 22 bits or fewer (to FP16) rounds d itself.
+__host__ __device__ __forceinline__ float float_odd_of(double d) {
+  const SplitBits s = split_bits(d);
+  if (!s.ok) return (float)d;   // |d| < 2^-74 is zero in FP16 and |d| >= 2^127 infinite, however rounded here
+  return float_bits(s.sign | s.top | (s.low != 0u));
+}
+
+// Double-float split of d: hi = RN_float(d), lo = RN_float(d - hi), the value dd(d) defines (lo is a
+// normal float or zero in the range of the integer form).
+__host__ __device__ __forceinline__ dd split_df(double d) {
+  const SplitBits s = split_bits(d);
+  if (!s.ok) return dd(d);
+  const unsigned up = s.low > 0x10000000u - (s.top & 1u);
+  int rem = (int)s.low - (int)(up << 29);   // |rem| <= 2^28: half a float ulp
+  if (s.sign) rem = -rem;
+  // lo = rem 2^(ed - 1075) (zero stays +0), the power of two a normal float
+  const float scale = float_bits((s.ed - 1075u + 127u) << 23);
+#ifdef __CUDA_ARCH__
+  const float lo = __int2float_rn(rem) * scale;
+#else
+  const float lo = (float)rem * scale;
+#endif
+  return dd(float_bits(s.sign | (s.top + up)), lo);
 }
 
 }  // namespace okgb

@@ -44,6 +44,7 @@
 // Q[(s, c)][(s', c')]; then U_t / 2 (9 words).  A lane reads the two entries it needs of a forward
 // block with one 8-byte load.
 #include "ok_pair.cuh"
+#include "ok_split.cuh"
 
 #include <cuda_fp16.h>
 
@@ -71,32 +72,27 @@ constexpr int MAX_RHS = 16;
 
 // ---------------------------------------------------------------------------- W copy
 __device__ __forceinline__ unsigned h2bits(cx<double> z) {
-  const __half2 h = __halves2half2(__double2half(z.re), __double2half(z.im));
+  const __half2 h = __floats2half2_rn(float_odd_of(z.re), float_odd_of(z.im));
   return *reinterpret_cast<const unsigned*>(&h);
-}
-
-// Pauli matrix entries sigma_k[r][c].
-__device__ __forceinline__ cx<double> pauli_e(int k, int r, int c) {
-  if (k == 0) return mk<double>(r != c ? 1.0 : 0.0, 0.0);
-  if (k == 1) return r == c ? mk<double>(0.0, 0.0) : mk<double>(0.0, r == 0 ? -1.0 : 1.0);
-  return r != c ? mk<double>(0.0, 0.0) : mk<double>(r == 0 ? 1.0 : -1.0, 0.0);
 }
 
 // One thread per site: the blocks Q of every forward hop, from the FP64 stored matrices (the
 // stored set keeps the factors 1/2 of the h+- basis of the FP32 kernels: the spatial P+- are
 // (D +- S) / 2, the temporal S and U are halves, W^0 = 2 (Y+ + Y-) (+) 2i (Y+ - Y-) ...).
+// Bound by the FP64 pipe: the spin factors are real or imaginary (or 2 (x +- i y)), so an entry takes two
+// products or sums, a factor 1 none, and the conversion to FP16 goes through integers; the four spin entries of
+// an element are one 16-byte store.
 __global__ void tc_build_kernel(const cx<double>* __restrict__ W, Geom g, const WScalars* __restrict__ scp,
                                 unsigned* __restrict__ out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   const WScalars sc = *scp;
   unsigned* o = out + (size_t)s * REC;
-  const cx<double> zero = mk<double>(0.0, 0.0);
-  // block `blk`, spin entry k: f * m
-  auto put = [&](int blk, int k, const M3<double>& m, cx<double> f) {
-    for (int e = 0; e < 9; ++e) o[blk * BLKW + 4 * e + k] = h2bits(f * m.e[e]);
+  auto put = [&](int blk, int e, const cx<double> (&z)[4]) {
+    *reinterpret_cast<uint4*>(o + blk * BLKW + 4 * e) = make_uint4(h2bits(z[0]), h2bits(z[1]), h2bits(z[2]), h2bits(z[3]));
   };
-  const cx<double> one = mk<double>(1.0, 0.0), two = mk<double>(2.0, 0.0);
+  auto rs = [](double f, cx<double> z) { return mk<double>(f * z.re, f * z.im); };
+  auto is = [](double f, cx<double> z) { return mk<double>(-f * z.im, f * z.re); };   // i f z
   // on-site: Y+- = [[a0 + c0, a1], [a2, c0 - a0]] (2x2 spin blocks of colour matrices);
   // W^0 = [[D', S'], [-S', D']], D' = 2 (Y+ + Y-), S' = -2i (Y+ - Y-); Q_{++} = Q_{--} = D', Q_{+-} = -S'.
   {
@@ -106,9 +102,16 @@ __global__ void tc_build_kernel(const cx<double>* __restrict__ W, Geom g, const 
     yp[0] = m_add(a0, c0); yp[1] = a1; yp[2] = a2; yp[3] = m_sub(c0, a0);
     const M3<double> b0 = wmat(W, s, M_Y0M), b1 = wmat(W, s, M_Y0M + 1), b2 = wmat(W, s, M_Y0M + 2);
     ym[0] = m_add(b0, c0); ym[1] = b1; ym[2] = b2; ym[3] = m_sub(c0, b0);
-    for (int k = 0; k < 4; ++k) {
-      put(B_E, k, m_add(yp[k], ym[k]), two);
-      put(B_F, k, m_sub(yp[k], ym[k]), mk<double>(0.0, 2.0));
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      cx<double> p[4], m[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        p[k] = rs(2.0, yp[k].e[e] + ym[k].e[e]);
+        m[k] = is(2.0, yp[k].e[e] - ym[k].e[e]);
+      }
+      put(B_E, e, p);
+      put(B_F, e, m);
     }
   }
   // temporal: W^+_4 = [[0, 2S], [2S, -2 U]] (S = [[t0, t1], [t2, -t0]], U = U_t / 2 stored):
@@ -116,43 +119,77 @@ __global__ void tc_build_kernel(const cx<double>* __restrict__ W, Geom g, const 
   {
     const M3<double> Uh = wmat(W, s, M_UT);
     const M3<double> t0 = wmat(W, s, M_ST), t1 = wmat(W, s, M_ST + 1), t2 = wmat(W, s, M_ST + 2);
-    const M3<double> S[4] = {t0, t1, t2, m_rscale(-1.0, t0)};
-    for (int k = 0; k < 4; ++k) {
-      const bool diag = k == 0 || k == 3;
-      put(B_TPP, k, diag ? m_sub(m_rscale(2.0, S[k]), Uh) : m_rscale(2.0, S[k]), one);
-      put(B_TMM, k, diag ? m_sub(m_rscale(-2.0, S[k]), Uh) : m_rscale(-2.0, S[k]), one);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const cx<double> S0 = rs(2.0, t0.e[e]), S1 = rs(2.0, t1.e[e]), S2 = rs(2.0, t2.e[e]), u = Uh.e[e];
+      const cx<double> p[4] = {S0 - u, S1, S2, -S0 - u}, m[4] = {-S0 - u, -S1, -S2, S0 - u};
+      put(B_TPP, e, p);
+      put(B_TMM, e, m);
     }
     for (int e = 0; e < 9; ++e) o[UHW + e] = h2bits(Uh.e[e]);
     for (int e = 9; e < REC - UHW; ++e) o[UHW + e] = 0u;  // padding to a 16-byte record
   }
   // spatial: stored P+- = (D +- S) / 2, so Q_{++} = 2 P+, Q_{--} = 2 P-.
-  for (int i = 0; i < 3; ++i)
-    for (int k = 0; k < 4; ++k) {
-      put(B_SP + 2 * i, k, wmat(W, s, M_WP + 8 * i + k), two);
-      put(B_SP + 2 * i + 1, k, wmat(W, s, M_WP + 8 * i + 4 + k), two);
+#pragma unroll 1
+  for (int b = 0; b < 6; ++b) {
+    M3<double> m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = wmat(W, s, M_WP + 4 * b + k);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const cx<double> z[4] = {rs(2.0, m[0].e[e]), rs(2.0, m[1].e[e]), rs(2.0, m[2].e[e]), rs(2.0, m[3].e[e])};
+      put(B_SP + b, e, z);
     }
+  }
   // two-hop: Q_{+-+-} = 2 (a +- b sigma_i) (x) V_ii.
+  const cx<double> zero = mk<double>(0.0, 0.0);
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     const M3<double> V = wmat(W, s, M_VII + i);
-    for (int k = 0; k < 4; ++k) {
-      const int sr = k >> 1, scc = k & 1;
-      const cx<double> a = mk<double>(sr == scc ? 2.0 * sc.a_ii : 0.0, 0.0);
-      const cx<double> b = (2.0 * sc.b_ii) * pauli_e(i, sr, scc);
-      put(B_II + 2 * i, k, V, a + b);
-      put(B_II + 2 * i + 1, k, V, a - b);
+    const double a = 2.0 * sc.a_ii, b = 2.0 * sc.b_ii;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const cx<double> v = V.e[e];
+      if (i == 2) {   // a +- b on the diagonal
+        const cx<double> x = rs(a + b, v), y = rs(a - b, v);
+        const cx<double> p[4] = {x, zero, zero, y}, m[4] = {y, zero, zero, x};
+        put(B_II + 4, e, p);
+        put(B_II + 5, e, m);
+      } else {
+        const cx<double> d = rs(a, v), y = i == 0 ? rs(b, v) : is(b, v);   // sigma_2 = [[0, -i], [i, 0]]
+        const cx<double> y1 = i == 0 ? y : -y;
+        const cx<double> p[4] = {d, y1, y, d}, m[4] = {d, -y1, -y, d};
+        put(B_II + 2 * i, e, p);
+        put(B_II + 2 * i + 1, e, m);
+      }
     }
   }
   // diagonal pair (I, J): Q_{++} = 2 (sigma_I +- sigma_J) (x) X for the offsets +I +-J.
+#pragma unroll
   for (int p = 0; p < 3; ++p) {
-    const int I = p == 2 ? 1 : 0, J = p == 0 ? 1 : 2;
-    const M3<double> Vij = wmat(W, s, M_VIJ + p), Xij = wmat(W, s, M_XIJ + p);
-    for (int k = 0; k < 4; ++k) {
-      const int sr = k >> 1, scc = k & 1;
-      put(B_VIJ + p, k, Vij, two * (pauli_e(I, sr, scc) + pauli_e(J, sr, scc)));
-      put(B_XIJ + p, k, Xij, two * (pauli_e(I, sr, scc) - pauli_e(J, sr, scc)));
+    const int I = p == 2 ? 1 : 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const M3<double> X = wmat(W, s, (h ? M_XIJ : M_VIJ) + p);
+      const double sg = h ? -1.0 : 1.0;
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        const cx<double> r = rs(2.0, X.e[e]), ir = mk<double>(-r.im, r.re);
+        cx<double> q[4];
+        if (p == 0) {   // sigma_1 +- sigma_2
+          q[0] = q[3] = zero;
+          q[1] = mk<double>(r.re - sg * ir.re, r.im - sg * ir.im);
+          q[2] = mk<double>(r.re + sg * ir.re, r.im + sg * ir.im);
+        } else {        // sigma_I +- sigma_3
+          q[0] = sg > 0 ? r : -r;
+          q[3] = sg > 0 ? -r : r;
+          q[1] = I == 0 ? r : -ir;
+          q[2] = I == 0 ? r : ir;
+        }
+        put((h ? B_XIJ : B_VIJ) + p, e, q);
+      }
     }
   }
-  (void)zero;
 }
 
 // The dense forward 12x12 matrix of one kind, rebuilt from the copy: W = T Q T / 2 in (u, l)
