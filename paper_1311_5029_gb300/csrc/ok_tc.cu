@@ -290,12 +290,8 @@ __device__ __forceinline__ BFrag neg(BFrag b) {
 // Per-lane constants.
 struct Lane {
   int g, t;            // groupID (lane >> 2), thread in group (lane & 3)
-  bool wact;           // this lane holds W entries (output column g < 6, input colour t < 3)
-  int off_f;           // forward: word offset of (Q[(s,c)][(0,t)], Q[(s,c)][(1,t)]) in a block
-  int uh_f, uh_b;      // U_t / 2 entries [c][t] and [t][c]
   int s;               // output spin of this lane's column
-  int a_off;           // offset 4 g + t of this lane's A-fragment word in a projection's tile
-  int e_b;             // word offset of the adjoint entries' element 3 t + c in a block (4 words)
+  int uh_f, uh_b;      // U_t / 2 entries [c][t] and [t][c], from the forward and the adjoint entries on
 };
 
 // FP16 input layout (the applied vectors, scaled): per (site, b) a 512-byte tile of 8 pairs x 4
@@ -307,18 +303,6 @@ struct Lane {
 constexpr int IN16_TILE_U4 = 32;   // 16-byte words per (site, projection) tile
 __host__ __device__ __forceinline__ size_t in16_index(int site, int b, int r, int c) {  // 8-byte units
   return ((((size_t)site * 2 + b) * IN16_TILE_U4) + 4 * (r & 7) + c) * 2 + (r >> 3);
-}
-
-// A fragments of the two projections of `site`.
-__device__ __forceinline__ void load_h(const uint4* __restrict__ f, int site, const Lane& L, AFrag& hp, AFrag& hm) {
-  const uint4* q = f + (size_t)site * (2 * IN16_TILE_U4) + L.a_off;
-  uint4 u = make_uint4(0u, 0u, 0u, 0u), v = u;
-  if (L.t < 3) {
-    u = __ldg(q);
-    v = __ldg(q + IN16_TILE_U4);
-  }
-  hp.r[0] = u.x; hp.r[2] = u.y; hp.r[1] = u.z; hp.r[3] = u.w;
-  hm.r[0] = v.x; hm.r[2] = v.y; hm.r[1] = v.z; hm.r[3] = v.w;
 }
 
 // Loads of W words that do not allocate in L1: every W byte is used once per application, so L1
@@ -417,16 +401,36 @@ __host__ __device__ constexpr HopDisp make_hop_disp() {
 }
 __constant__ HopDisp k_hop_disp = make_hop_disp();
 
+// x / L for the first three extents by multiplication: floor(x m / 2^s) with m = ceil(2^s / L), s = 31 + ceil(log2 L),
+// is the quotient for every x < 2^31 (Granlund and Montgomery, PLDI 1994).
+struct SiteDiv {
+  unsigned m[3];
+  int s[3];
+};
+static SiteDiv site_div(const Geom& g) {
+  SiteDiv d;
+  for (int mu = 0; mu < 3; ++mu) {
+    int l = 0;
+    while ((1LL << l) < g.L[mu]) ++l;
+    d.s[mu] = 31 + l;
+    d.m[mu] = (unsigned)(((1ULL << d.s[mu]) + g.L[mu] - 1) / g.L[mu]);
+  }
+  return d;
+}
+
 // Neighbour code of hop `lane` (lanes 0..26, in parallel): (neighbour site << 1) | 1 when the hop
 // crosses an antiperiodic boundary an odd number of times.
-__device__ __forceinline__ int nbr_code(int lane, int x, const Geom& g) {
+__device__ __forceinline__ int nbr_code(int lane, int x, const Geom& g, const SiteDiv& dv) {
   const unsigned w = k_hop_disp.d[lane & 31];
   int r = x, idx = 0, neg = 0;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     const int L = g.L[mu];
-    const int cm = mu < 3 ? r % L : r;
-    if (mu < 3) r /= L;
+    int cm = r;
+    if (mu < 3) {
+      r = (int)((unsigned long long)(unsigned)r * dv.m[mu] >> dv.s[mu]);
+      cm -= r * L;
+    }
     const int d = ((int)(w << (28 - 4 * mu))) >> 28;   // sign-extended 4-bit field
     int xm = cm + d, wraps = 0;
     if (xm >= L) { xm -= L; ++wraps; if (xm >= L) { xm -= L; ++wraps; } }
@@ -447,45 +451,50 @@ struct HopRaw {
 };
 
 struct Ctx {
-  const uint4* __restrict__ in;
-  const unsigned* __restrict__ W;
+  const uint4* in;      // input tiles, at this lane's word
+  const unsigned* Wx;   // the site's record, at this lane's forward entries
+  const unsigned* Wb;   // the first site's record, at this lane's adjoint entries
   int x;      // the site
   int code;   // this lane's neighbour code (nbr_code)
-  Lane L;
 };
 
+// The loads of one hop.  All lanes load: lanes that hold no entry (output column g >= 6, input slot t = 3) read
+// another lane's words, which meet a zero of the input tile's slot 3 or end in an output column that is
+// not stored.  Lanes that skipped theirs cost a move of zero for every register, which with the divisions of nbr_code
+// and a shuffle waited for in front of every hop's loads made 1388 us of 20^3 x 64 with 12 right-hand sides, now
+// 1266 us.  code: the hop's, from nbr_code.
 // AP: the lattice has an antiperiodic direction (else every boundary sign is +1).
 template <int J, bool AP>
-__device__ __forceinline__ void hop_load(const Ctx& C, HopRaw& R) {
+__device__ __forceinline__ void hop_load(const Ctx& C, const Lane& L, int code, HopRaw& R) {
   constexpr HopDesc d = hop_desc(J);
   int n = C.x;
   R.sm = 0u;
   if constexpr (d.mu >= 0) {
-    const int code = __shfl_sync(0xffffffffu, C.code, J);
     n = code >> 1;
     if constexpr (AP) R.sm = (code & 1) ? 0x80008000u : 0u;
   }
-  load_h(C.in, n, C.L, R.hp, R.hm);
-  constexpr bool at_nbr = d.ld[0].kind == LK_BWD;
-  const unsigned* rec = C.W + (size_t)(at_nbr ? n : C.x) * REC;
+  const uint4* q = C.in + (size_t)n * (2 * IN16_TILE_U4);
+  const uint4 u = __ldg(q), v = __ldg(q + IN16_TILE_U4);
+  R.hp.r[0] = u.x; R.hp.r[2] = u.y; R.hp.r[1] = u.z; R.hp.r[3] = u.w;
+  R.hm.r[0] = v.x; R.hm.r[2] = v.y; R.hm.r[1] = v.z; R.hm.r[3] = v.w;
+  const unsigned* nb = C.Wb + (size_t)n * REC;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    R.w[k][0] = R.w[k][1] = 0u;
     const int kind = d.ld[k].kind, blk = d.ld[k].blk;
-    if (kind == LK_NONE || !C.L.wact) continue;
+    if (kind == LK_NONE) continue;
     if (kind == LK_FWD) {
-      const uint2 z = ldw2(rec + blk * BLKW + C.L.off_f);
+      const uint2 z = ldw2(C.Wx + blk * BLKW);
       R.w[k][0] = z.x;
       R.w[k][1] = z.y;
     } else if (kind == LK_BWD) {
       // the four spin entries of element 3 t + c; this lane takes k = s and k = 2 + s
-      const uint4 z = ldw4(rec + blk * BLKW + C.L.e_b);
-      R.w[k][0] = C.L.s ? z.y : z.x;
-      R.w[k][1] = C.L.s ? z.w : z.z;
+      const uint4 z = ldw4(nb + blk * BLKW);
+      R.w[k][0] = L.s ? z.y : z.x;
+      R.w[k][1] = L.s ? z.w : z.z;
     } else {
-      const unsigned u = ldw1(rec + UHW + (kind == LK_UF ? C.L.uh_f : C.L.uh_b));
-      R.w[k][0] = C.L.s ? 0u : u;   // (U_t / 2) x 1 is diagonal in spin
-      R.w[k][1] = C.L.s ? u : 0u;
+      const unsigned u1 = kind == LK_UF ? ldw1(C.Wx + UHW + L.uh_f) : ldw1(nb + UHW + L.uh_b);
+      R.w[k][0] = L.s ? 0u : u1;   // (U_t / 2) x 1 is diagonal in spin
+      R.w[k][1] = L.s ? u1 : 0u;
     }
   }
 }
@@ -512,14 +521,17 @@ __device__ __forceinline__ void hop_compute(const HopRaw& R, Acc& A) {
 // hops already loaded.  Three register slots divide the 27 hops, so a hop's slot is a constant.
 constexpr int TC_SLOTS = 3;
 static_assert(NHOP % TC_SLOTS == 0, "hop slots must divide the hop count");
+// nc: the neighbour code of the hop whose loads come next, shuffled one hop ahead of its use.
 template <int J, bool AP>
-__device__ __forceinline__ void pipe(const Ctx& C, const Ctx& Cn, bool more, HopRaw (&R)[TC_SLOTS], Acc& A) {
+__device__ __forceinline__ void pipe(const Ctx& C, const Ctx& Cn, const Lane& L, bool more, int& nc, HopRaw (&R)[TC_SLOTS], Acc& A) {
   if constexpr (J < NHOP) {
     constexpr int JJ = J + TC_SLOTS - 1;
-    if constexpr (JJ < NHOP) hop_load<JJ, AP>(C, R[JJ % TC_SLOTS]);
-    else if (more) hop_load<JJ - NHOP, AP>(Cn, R[JJ % TC_SLOTS]);
+    const int code = nc;
+    nc = __shfl_sync(0xffffffffu, JJ + 1 < NHOP ? C.code : Cn.code, (JJ + 1) % NHOP);
+    if constexpr (JJ < NHOP) hop_load<JJ, AP>(C, L, code, R[JJ % TC_SLOTS]);
+    else if (more) hop_load<JJ - NHOP, AP>(Cn, L, code, R[JJ % TC_SLOTS]);
     hop_compute<J, AP>(R[J % TC_SLOTS], A);
-    pipe<J + 1, AP>(C, Cn, more, R, A);
+    pipe<J + 1, AP>(C, Cn, L, more, nc, R, A);
   }
 }
 
@@ -567,22 +579,15 @@ __device__ __forceinline__ void multi_finish(double (*bsum)[3], const bool* live
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-// Launch bounds: blocks per SM (4: 128 registers, 16 warps); L2 bulk prefetch of the next site's
-// record on (1) or off (0).
+// Blocks per SM: 4 (128 registers, 16 warps).  20^3 x 64, 12 right-hand sides: 1266 us; 1299 us at 5 (96 registers),
+// 1309 us at 3.
 #ifndef OK_TC_MINB
 #define OK_TC_MINB 4
 #endif
-#ifndef OK_TC_PF
-#define OK_TC_PF 1
-#endif
-// Bulk prefetch of a site's W record (3216 bytes, 16-byte aligned) into L2.
-__device__ __forceinline__ void prefetch_rec(const unsigned* p) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "n"(REC * 4) : "memory");
-}
 
 template <int EPI, bool AP>
 __global__ void __launch_bounds__(TC_THREADS, OK_TC_MINB) apply_tc_kernel(const unsigned* __restrict__ W, const uint4* __restrict__ in,
-                                                                 float4* __restrict__ out, Geom g, int nrhs, TcEpi ep) {
+                                                                 float4* __restrict__ out, Geom g, int nrhs, SiteDiv dv, TcEpi ep) {
   constexpr bool RED = EPI == EPI_DOT || EPI == EPI_TS;
   __shared__ bool live[MAX_RHS];
   __shared__ double bsum[MAX_RHS][3];
@@ -602,13 +607,11 @@ __global__ void __launch_bounds__(TC_THREADS, OK_TC_MINB) apply_tc_kernel(const 
   L.g = lane >> 2;
   L.t = lane & 3;
   L.s = L.g & 1;
-  L.wact = L.g < 6 && L.t < 3;
-  const int cc = L.g >> 1;
-  L.off_f = 4 * (3 * cc + L.t) + 2 * L.s;
-  L.uh_f = 3 * cc + L.t;
-  L.uh_b = 3 * L.t + cc;
-  L.a_off = 4 * L.g + L.t;
-  L.e_b = 4 * (3 * L.t + cc);
+  const int cc = (L.g < 6 ? L.g : 5) >> 1, tt = L.t < 3 ? L.t : 2;   // output column's and input's colour
+  const int off_f = 4 * (3 * cc + tt) + 2 * L.s;   // forward: (Q[(s,c)][(0,t)], Q[(s,c)][(1,t)]) in a block
+  const int off_b = 4 * (3 * tt + cc);             // adjoint: element 3 t + c (4 words)
+  L.uh_f = 3 * cc + tt - off_f;
+  L.uh_b = 3 * tt + cc - off_b;
   // 1 / sigma of the right-hand sides of this lane's rows (g and g + 8)
   float inv[2] = {1.f, 1.f};
 #pragma unroll
@@ -626,17 +629,16 @@ __global__ void __launch_bounds__(TC_THREADS, OK_TC_MINB) apply_tc_kernel(const 
   const int nw = G * TC_WARPS;
   int x = rank * TC_WARPS + warp;
   if (x < g.V) {
-    Ctx C{in, W, x, nbr_code(lane, x, g), L};
+    Ctx C{in + 4 * L.g + L.t, W + (size_t)x * REC + off_f, W + off_b, x, nbr_code(lane, x, g, dv)};
     HopRaw R[TC_SLOTS];
-    hop_load<0, AP>(C, R[0]);
-    hop_load<1, AP>(C, R[1]);
+    hop_load<0, AP>(C, L, 0, R[0]);
+    hop_load<1, AP>(C, L, __shfl_sync(0xffffffffu, C.code, 1), R[1]);
+    int nc = __shfl_sync(0xffffffffu, C.code, 2);
     for (;;) {
       const int xn = x + nw;
       const bool more = xn < g.V;
-      const Ctx Cn{in, W, more ? xn : x, more ? nbr_code(lane, xn, g) : C.code, L};
-      // the next site's own W record is read from DRAM once, block by block over its hops: have it
-      // in L2 before they start
-      if (OK_TC_PF && more && lane == 0) prefetch_rec(W + (size_t)xn * REC);
+      const int xm = more ? xn : x;
+      const Ctx Cn{C.in, W + (size_t)xm * REC + off_f, C.Wb, xm, nbr_code(lane, xm, g, dv)};
       if constexpr (RED) {
         // copy this site's epilogue operand units (FP32) into shared memory while the hops run
         if (L.t < 3) {
@@ -662,7 +664,7 @@ __global__ void __launch_bounds__(TC_THREADS, OK_TC_MINB) apply_tc_kernel(const 
         for (int p = 0; p < 2; ++p)
 #pragma unroll
           for (int k = 0; k < 4; ++k) A.v[a][p][k] = 0.f;
-      pipe<0, AP>(C, Cn, more, R, A);
+      pipe<0, AP>(C, Cn, L, more, nc, R, A);
       if constexpr (RED) asm volatile("cp.async.wait_all;" ::: "memory");
       if (L.t < 3) {
 #pragma unroll
@@ -1133,7 +1135,8 @@ int launch_apply_tc(const ok_W* W, const void* in16, cx<float>* out, int nrhs, i
     Geom gs = W->g;
     gs.sms = sm_count();
     const bool ap = gs.bcneg != 0;
-#define OK_TC_LAUNCH(E, AP) tc::apply_tc_kernel<E, AP><<<grid, tc::TC_THREADS, 0, st>>>(Wt, i4, o4, gs, nrhs, ep)
+    const tc::SiteDiv dv = tc::site_div(gs);
+#define OK_TC_LAUNCH(E, AP) tc::apply_tc_kernel<E, AP><<<grid, tc::TC_THREADS, 0, st>>>(Wt, i4, o4, gs, nrhs, dv, ep)
     if (epi == EPI_NONE) { if (ap) OK_TC_LAUNCH(EPI_NONE, true); else OK_TC_LAUNCH(EPI_NONE, false); }
     else if (epi == EPI_DOT) { if (ap) OK_TC_LAUNCH(EPI_DOT, true); else OK_TC_LAUNCH(EPI_DOT, false); }
     else { if (ap) OK_TC_LAUNCH(EPI_TS, true); else OK_TC_LAUNCH(EPI_TS, false); }
