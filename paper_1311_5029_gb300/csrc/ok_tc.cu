@@ -839,6 +839,20 @@ __device__ __forceinline__ void sys_scalars(const SolverState* st, int r, dcx& a
   halt = st[r].halt;
 }
 
+// Writes the FP16 unit (row, r, c), and with it the words beside it that belong to no right-hand side (slot 3,
+// absent right-hand sides; they stay zero), so that whole 32-byte sectors are written: partly written ones
+// are read first.  12 right-hand sides at 20^3 x 64, with VEC_BLOCKS: update_s 473 -> 355 us, update_p 530 -> 455 us.
+__device__ __forceinline__ void put16(uint2* __restrict__ f, long long row, int r, int c, int nrhs, uint2 w) {
+  uint2* q = f + in16_index((int)(row >> 1), (int)(row & 1), r, c);
+  if (r < 8 && r + 8 >= nrhs) {
+    *reinterpret_cast<uint4*>(q) = make_uint4(w.x, w.y, 0u, 0u);
+    if (c == 2) *reinterpret_cast<uint4*>(q + 2) = make_uint4(0u, 0u, 0u, 0u);
+  } else {
+    *q = w;
+    if (c == 2) q[2] = make_uint2(0u, 0u);
+  }
+}
+
 // s = r - alpha v, and its FP16 copy sigma s for the apply
 __global__ void tc_update_s_kernel(const float4* __restrict__ rv, const float4* __restrict__ v, float4* __restrict__ s,
                                    uint2* __restrict__ s16, int rows, int nrhs, const SolverState* __restrict__ st) {
@@ -856,8 +870,7 @@ __global__ void tc_update_s_kernel(const float4* __restrict__ rv, const float4* 
     const float4 o = make_float4(a.x - (ar * b.x - ai * b.y), a.y - (ar * b.y + ai * b.x), a.z - (ar * b.z - ai * b.w),
                                  a.w - (ar * b.w + ai * b.z));
     s[i] = o;
-    s16[in16_index((int)(row >> 1), (int)(row & 1), r, threadIdx.x - 3 * r)] =
-        make_uint2(pack_scaled(o.x, o.y, sc), pack_scaled(o.z, o.w, sc));
+    put16(s16, row, r, threadIdx.x - 3 * r, nrhs, make_uint2(pack_scaled(o.x, o.y, sc), pack_scaled(o.z, o.w, sc)));
   }
 }
 
@@ -866,37 +879,35 @@ __global__ void tc_update_s_kernel(const float4* __restrict__ rv, const float4* 
 __global__ void tc_update_p_kernel(float4* __restrict__ p, uint2* __restrict__ p16, const float4* __restrict__ rv,
                                    const float4* __restrict__ v, int rows, int nrhs, const SolverState* __restrict__ st,
                                    int only) {
-  const int r = threadIdx.x / 3;
+  const int r = (only >= 0 ? only : 0) + threadIdx.x / 3, tx = 3 * r + threadIdx.x % 3;
   dcx al, om, be;
   int halt;
   sys_scalars(st, r, al, om, be, halt);
-  if (halt || (only >= 0 && r != only)) return;
+  if (halt) return;
   const cx<float> B = mk<float>((float)be.re, (float)be.im), O = mk<float>((float)om.re, (float)om.im);
   const float sc = solve_scale(st[r].rr);
   const int L = 3 * nrhs;
   for (long long row = blockIdx.x * (long long)blockDim.y + threadIdx.y; row < rows; row += (long long)gridDim.x * blockDim.y) {
-    const size_t i = (size_t)row * L + threadIdx.x;
+    const size_t i = (size_t)row * L + tx;
     const float4 pp = p[i], rr = rv[i], vv = v[i];
     const cx<float> p0 = mk(pp.x, pp.y) - O * mk(vv.x, vv.y), p1 = mk(pp.z, pp.w) - O * mk(vv.z, vv.w);
     const cx<float> q0 = mk(rr.x, rr.y) + B * p0, q1 = mk(rr.z, rr.w) + B * p1;
     p[i] = make_float4(q0.re, q0.im, q1.re, q1.im);
-    p16[in16_index((int)(row >> 1), (int)(row & 1), r, threadIdx.x - 3 * r)] =
-        make_uint2(pack_scaled(q0.re, q0.im, sc), pack_scaled(q1.re, q1.im, sc));
+    put16(p16, row, r, tx - 3 * r, nrhs, make_uint2(pack_scaled(q0.re, q0.im, sc), pack_scaled(q1.re, q1.im, sc)));
   }
 }
 
 // FP16 copy sigma p of p for live systems (only >= 0: that system alone), after a restart.
 __global__ void tc_half_kernel(const float4* __restrict__ p, uint2* __restrict__ p16, int rows, int nrhs,
                                const SolverState* __restrict__ st, int only) {
-  const int r = threadIdx.x / 3;
-  if (st[r].halt || (only >= 0 && r != only)) return;
+  const int r = (only >= 0 ? only : 0) + threadIdx.x / 3, tx = 3 * r + threadIdx.x % 3;
+  if (st[r].halt) return;
   const float sc = solve_scale(st[r].rr);
   const int L = 3 * nrhs;
   for (long long row = blockIdx.x * (long long)blockDim.y + threadIdx.y; row < rows; row += (long long)gridDim.x * blockDim.y) {
-    const size_t i = (size_t)row * L + threadIdx.x;
+    const size_t i = (size_t)row * L + tx;
     const float4 q = p[i];
-    p16[in16_index((int)(row >> 1), (int)(row & 1), r, threadIdx.x - 3 * r)] =
-        make_uint2(pack_scaled(q.x, q.y, sc), pack_scaled(q.z, q.w, sc));
+    put16(p16, row, r, tx - 3 * r, nrhs, make_uint2(pack_scaled(q.x, q.y, sc), pack_scaled(q.z, q.w, sc)));
   }
 }
 
@@ -955,7 +966,7 @@ __global__ void tc_update_xr_kernel(float4* __restrict__ x, const uint2* __restr
     const long long gs = (long long)gridDim.x * blockDim.y;
     for (long long row0 = blockIdx.x * (long long)blockDim.y + threadIdx.y; row0 < rows; row0 += gs * TC_RED_CHUNK) {
     float c3[3] = {0.f, 0.f, 0.f};
-#pragma unroll
+#pragma unroll 1
     for (int u = 0; u < TC_RED_CHUNK; ++u) {
       const long long row = row0 + u * gs;
       if (row >= rows) break;
@@ -1175,6 +1186,11 @@ int launch_from_tc(const cx<float>* in, cx<float>* out, int V, int nrhs, cudaStr
 // Block shape and resident grid of the vector kernels for nrhs right-hand sides (occupancy looked
 // up once per kernel and nrhs).
 enum { VK_S = 0, VK_P = 1, VK_XR = 2 };
+// At most this many blocks per multiprocessor: with more streams at a time DRAM serves them worse.  12 right-hand
+// sides at 20^3 x 64 (us): update_s 355 / 379 / 397 at 5 / 4 / 3 blocks and 402 at the 6 its registers allow,
+// update_p 455 / 451 / 458 and 510 at 8.  update_xr takes 5 with its rows one by one (48 registers, 758 us) and 3
+// with the chunk unrolled (72 registers, 793 us).
+constexpr int VEC_BLOCKS = 5;
 static void vec_shape(int nrhs, dim3* block, int* grid, int which) {
   static std::atomic<int> cache[3][tc::MAX_RHS + 1];
   const int X = 3 * nrhs;
@@ -1188,6 +1204,7 @@ static void vec_shape(int nrhs, dim3* block, int* grid, int which) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, X * Y, 0) != cudaSuccess || nb < 1) nb = 1;
     cache[which][nrhs].store(nb, std::memory_order_relaxed);
   }
+  if (nb > VEC_BLOCKS) nb = VEC_BLOCKS;
   *grid = nb * sm_count();
 }
 
@@ -1215,7 +1232,7 @@ int launch_tc_update_p(cx<float>* p, void* p16, const cx<float>* r, const cx<flo
                        int only, cudaStream_t strm) {
   dim3 b;
   int g = 0;
-  vec_shape(nrhs, &b, &g, VK_P);
+  vec_shape(only >= 0 ? 1 : nrhs, &b, &g, VK_P);
   {
     TraceScope ts("update_p_tc", strm);
     tc::tc_update_p_kernel<<<g, b, 0, strm>>>((float4*)p, (uint2*)p16, (const float4*)r, (const float4*)v, 2 * V, nrhs, st,
@@ -1228,7 +1245,7 @@ int launch_tc_update_p(cx<float>* p, void* p16, const cx<float>* r, const cx<flo
 int launch_tc_half(const cx<float>* p, void* p16, int V, int nrhs, const SolverState* st, int only, cudaStream_t strm) {
   dim3 b;
   int g = 0;
-  vec_shape(nrhs, &b, &g, VK_P);
+  vec_shape(only >= 0 ? 1 : nrhs, &b, &g, VK_P);
   {
     TraceScope ts("half_tc", strm);
     tc::tc_half_kernel<<<g, b, 0, strm>>>((const float4*)p, (uint2*)p16, 2 * V, nrhs, st, only);
