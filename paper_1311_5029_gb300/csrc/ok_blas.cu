@@ -185,12 +185,12 @@ __global__ void __launch_bounds__(BLAS_THREADS) dots_kernel(const typename Unit<
 
 // ---------------------------------------------------------------------------- small systems
 // On a small lattice the five vector kernels of an FP32 iteration cost their launches, their grid
-// completions and their last block's tail, not their bytes (4^3 x 8: 36 us an iteration, 12 us of it
+// completions and their last block's tail, not their bytes (4^3 x 8: 43 us an iteration, 12 us of it
 // update_xr; now 25 us).  There one cluster of up to eight blocks does the work between two applications
 // in one launch: it takes the inner products, finalises the scalars and streams the update, with cluster
 // barriers in the place of kernel boundaries.  Block sums meet in the first block's shared memory and are
 // added in a fixed tree, so a solve is reproducible; the state is worked on in shared memory as well, as
-// its finalisation is one thread's chain of dependent accesses (20.0 -> 16.0 us for small_xrp).
+// its finalisation is one thread's chain of dependent accesses (18.2 -> 16.0 us for small_xrp).
 constexpr int CL_THREADS = 1024;
 constexpr int CL_MAX = 8;
 __device__ __forceinline__ unsigned cl_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
