@@ -204,14 +204,14 @@ def measured_peaks():
 
 def apply_source_hash():
     h = hashlib.sha256()
-    for f in ("ok_apply.cu", "ok_hops.cuh", "ok_pair.cuh", "ok_internal.cuh", "ok_reduce.cuh", "ok_launch.cuh"):
+    for f in ("ok_apply_pipe.cu", "ok_apply.cu", "ok_hops.cuh", "ok_pair.cuh", "ok_internal.cuh", "ok_reduce.cuh", "ok_launch.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1311_5029_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def ncu_traffic(kernel_key):
     """DRAM bytes per launch recorded by the committed ncu summary, if it still matches the source."""
-    path = os.path.join(ROOT, "profiles", "apply_f32_split_16x16x16x32.md")
+    path = os.path.join(ROOT, "profiles", "apply_f32_pipe_16x16x16x32.md")
     if not os.path.exists(path):
         return None
     text = open(path).read()

@@ -316,7 +316,7 @@ __device__ __forceinline__ void colour2h(H6<R>& y, const M3<R>& V, const H6<R>& 
 }
 
 // Each hop function does the forward (FWD) or the backward half of its part of the stencil; the two
-// run in different warps (the split kernel).
+// run in different warps.
 template <typename R, int I, bool FWD, bool AP, typename WS>
 __device__ __forceinline__ void pair_spatial(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                              const Geom& g, int s, const Pair& pr, H6<R>& acc) {

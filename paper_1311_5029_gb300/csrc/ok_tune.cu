@@ -1,5 +1,5 @@
 // Autotuner: picks launch shapes for a handle by timing the candidates on scratch fields.
-//   one right-hand side: the split kernel with the forward W read by ordinary loads or streamed
+//   one right-hand side: the pipelined kernel (ok_apply_pipe.cu), or the one with its forward W streamed
 //     into shared memory by TMA (which wins depends on the lattice and on L1 pressure);
 //   several right-hand sides: right-hand sides per thread NR (1, 2 or 4, dividing nrhs) and the
 //     width of the persistent grid (as many blocks as fit, or half of that).
