@@ -213,8 +213,10 @@ __device__ __forceinline__ void cl_state(ClusterShared& sh, SolverState* st, boo
     if (load) *a = *b; else *b = *a;
   }
 }
+// The form that counts threads, not warps: lane 0 alone finalises, and the last round of a loop over units need not take
+// a whole warp, so the lanes of a warp may arrive here apart (`.aligned` would want them converged).
 __device__ __forceinline__ void cl_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
 }
 // A 32-bit word of shared memory at the same place in block `rank` of the cluster.
 __device__ __forceinline__ float cl_load(const void* p, unsigned rank) {
