@@ -18,6 +18,7 @@
 //   Adam:     on the real and imaginary parts of every A entry, in the gradient's final sum.
 // A training step runs every kernel once for a group of its pairs, not once per pair.
 #include "ok_net.cuh"
+#include "ok_sum3.cuh"
 #include "ok_pair.cuh"
 
 #include <cmath>
@@ -286,21 +287,11 @@ __global__ void __launch_bounds__(256) net_grad_final_kernel(const double* __res
   ad.P[i] -= ad.lr * (m / ad.c1) / (sqrtf(v / ad.c2) + ad.eps);
 }
 
-// |x|^2 and |out - x|^2 of pair blockIdx.y -> scal[2 + 2 pair], scal[3 + 2 pair].  The squares of a
-// chunk of LOSS_CHUNK complex numbers are summed as double-float pairs on the FP32 pipes (about 48
-// bits) when the chunk's largest component lies in [2^-40, 2^40], where neither the squares nor
-// their rounding errors leave FP32's range, and in FP64 otherwise; chunks are added in FP64.  (In
-// FP64 throughout, the FP64 pipe was 82 % busy: 51 us for 25 MB at 16^3 x 32, now 13 us a pair.)
+// |x|^2 and |out - x|^2 of pair blockIdx.y -> scal[2 + 2 pair], scal[3 + 2 pair]: chunks of LOSS_CHUNK complex
+// numbers on the FP32 pipes with more than FP64's accuracy (ok_sum3.cuh), the chunks in FP64.  (In FP64 throughout
+// the FP64 pipe was 82 % busy: 51 us for 25 MB at 16^3 x 32, now 16 us a pair in a batch of four; pairs of floats, which
+// took 13 us, keep 48 bits and lose the squares of small differences.)
 constexpr int LOSS_CHUNK = 8;
-__device__ __forceinline__ dd dd_sq(dd a) {
-  const float p = a.hi * a.hi;
-  const float e = fmaf(a.hi, a.hi, -p);
-  return dd_renorm(p, fmaf(2.f * a.hi, a.lo, e));
-}
-__device__ __forceinline__ dd dd_diff(float a, float b) {
-  const float s = a - b, bb = s - a;
-  return dd(s, (a - (s - bb)) - (b + bb));
-}
 __global__ void __launch_bounds__(256) net_loss_kernel(const float2* __restrict__ out, const float2* __restrict__ x, long long n,
                                                        double* part, double* scal, unsigned* ticket) {
   out += blockIdx.y * n;
@@ -309,42 +300,13 @@ __global__ void __launch_bounds__(256) net_loss_kernel(const float2* __restrict_
   const long long gs = (long long)gridDim.x * 256;
   for (long long i0 = blockIdx.x * 256LL + threadIdx.x; i0 < n; i0 += gs * LOSS_CHUNK) {
     float2 a[LOSS_CHUNK], b[LOSS_CHUNK];
-    float mx = 0.f;
 #pragma unroll
     for (int u = 0; u < LOSS_CHUNK; ++u) {
       const long long i = i0 + u * gs;
       a[u] = b[u] = make_float2(0.f, 0.f);
       if (i < n) { a[u] = out[i]; b[u] = x[i]; }
     }
-    bool nan = false;
-#pragma unroll
-    for (int u = 0; u < LOSS_CHUNK; ++u) {
-      mx = fmaxf(fmaxf(fmaxf(mx, fabsf(a[u].x)), fmaxf(fabsf(a[u].y), fabsf(b[u].x))), fabsf(b[u].y));
-      nan = nan || isnan(a[u].x) || isnan(a[u].y) || isnan(b[u].x) || isnan(b[u].y);
-    }
-    if (mx == 0.f && !nan) continue;
-    if (mx >= 0x1p-40f && mx <= 0x1p40f && !nan) {
-      dd s0(0.f, 0.f), s1(0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < LOSS_CHUNK; ++u) {
-        s0 = s0 + dd_sq(dd(b[u].x, 0.f));
-        s0 = s0 + dd_sq(dd(b[u].y, 0.f));
-        s1 = s1 + dd_sq(dd_diff(a[u].x, b[u].x));
-        s1 = s1 + dd_sq(dd_diff(a[u].y, b[u].y));
-      }
-      v[0] += (double)s0;
-      v[1] += (double)s1;
-    } else {
-#pragma unroll 1
-      for (int u = 0; u < LOSS_CHUNK; ++u) {
-        const long long i = i0 + u * gs;
-        if (i >= n) break;
-        const float2 o = out[i], y = x[i];
-        const double er = (double)o.x - y.x, ei = (double)o.y - y.y;
-        v[0] += (double)y.x * y.x + (double)y.y * y.y;
-        v[1] += er * er + ei * ei;
-      }
-    }
+    loss_chunk(a, b, v);
   }
   const RedArgs ra{nullptr, part + (size_t)blockIdx.y * 2 * gridDim.x, scal + 2 + 2 * blockIdx.y, FIN_NONE};
   grid_reduce<2, 256>(v, ra, ticket + blockIdx.y);
