@@ -18,12 +18,24 @@
 //   Adam:     on the real and imaginary parts of every A entry, in the gradient's final sum.
 // A training step runs every kernel once for a group of its pairs, not once per pair.
 #include "ok_net.cuh"
+#include "ok_group.cuh"
 #include "ok_sum3.cuh"
 #include "ok_pair.cuh"
 
 #include <cmath>
 #include <cstring>
 #include <vector>
+
+namespace okgb {
+// Scratch of a training step for `group` pairs.
+struct TrainBufs {
+  int group = 0;                       // 0: none
+  cx<float>* acts = nullptr;           // [layers][group][V * 12]
+  cx<float>* tg[2] = {nullptr, nullptr};  // backward gradients [group][V * 12]; null for one pair (ok_net::g serves)
+  double* part = nullptr;              // gradient partials [layers][blocks][9][32]
+  double* lpart = nullptr;             // loss partials [group][2 * loss blocks]
+};
+}  // namespace okgb
 
 struct ok_net {
   int layers = 0;
@@ -37,11 +49,8 @@ struct ok_net {
   int V = 0;                // volume the workspace is sized for
   int device = 0;
   okgb::cx<float>* g[2] = {nullptr, nullptr};  // layer ping-pong of an application, [V * 12]
-  int group = 0;            // pairs the training workspace holds (0: none yet)
-  okgb::cx<float>* acts = nullptr;  // [layers][group][V * 12]
-  okgb::cx<float>* tg[2] = {nullptr, nullptr};  // backward gradients, [group][V * 12]
-  double* part = nullptr;   // gradient partials [layers][blocks][9][32]
-  double* lpart = nullptr;  // loss partials [group][2 * loss blocks]
+  okgb::TrainBufs t;        // of the pairs that train together
+  int most = 0;             // the largest group that fitted, once a larger one did not
 };
 
 namespace okgb {
@@ -349,12 +358,25 @@ int loss_blocks(int V) {
   return need < cap ? need : cap;
 }
 
-void free_training(ok_net* N) {
-  for (void* q : {(void*)N->acts, (void*)N->tg[0], (void*)N->tg[1], (void*)N->part, (void*)N->lpart})
+void free_training(TrainBufs& t) {
+  for (void* q : {(void*)t.acts, (void*)t.tg[0], (void*)t.tg[1], (void*)t.part, (void*)t.lpart})
     if (q) cudaFree(q);
-  N->acts = N->tg[0] = N->tg[1] = nullptr;
-  N->part = N->lpart = nullptr;
-  N->group = 0;
+  t = TrainBufs{};
+}
+
+cudaError_t alloc_training(const ok_net* N, int V, int pairs, TrainBufs& t) {
+  const size_t f = (size_t)pairs * V * 12 * sizeof(cx<float>);
+  cudaError_t e = cudaMalloc(&t.acts, N->layers * f);
+  for (int k = 0; k < 2 && pairs > 1 && e == cudaSuccess; ++k) e = cudaMalloc(&t.tg[k], f);
+  if (e == cudaSuccess) e = cudaMalloc(&t.part, (size_t)N->layers * grad_blocks(V) * NPAR * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&t.lpart, (size_t)pairs * 2 * loss_blocks(V) * sizeof(double));
+  if (e == cudaSuccess) {
+    t.group = pairs;
+  } else {
+    cudaGetLastError();
+    free_training(t);
+  }
+  return e;
 }
 
 // Pairs of a batch of nb that one pass of the kernels takes: as many as fit in 256 MiB of
@@ -367,13 +389,15 @@ int group_of(const ok_net* N, int V, int nb) {
   return q < 1 ? 1 : (int)q;
 }
 
-// Scratch for a lattice of V sites: two fields (the layer ping-pong of an application) and, for
-// training (nb > 0), the activations of every layer, the backward gradients and the reduction
-// partials of a group of pairs; a group that does not fit in memory falls back to one pair.
+// Scratch for a lattice of V sites: two fields (the layer ping-pong of an application, and the backward gradients of
+// one pair) and, for training (nb > 0), the activations of every layer, the backward gradients and the
+// reduction partials of a group of pairs.  A larger group's buffers are taken before the present ones are given
+// back; where they do not fit, a smaller group runs, down to one pair.
 int ensure_workspace(ok_net* N, int V, int nb) {
   const size_t n = (size_t)V * 12;
   if (N->V != V) {
-    free_training(N);
+    free_training(N->t);
+    N->most = 0;
     if (N->g[0]) cudaFree(N->g[0]);
     if (N->g[1]) cudaFree(N->g[1]);
     N->g[0] = N->g[1] = nullptr; N->V = 0;
@@ -382,23 +406,17 @@ int ensure_workspace(ok_net* N, int V, int nb) {
     N->V = V;
   }
   if (nb < 1) return OK_SUCCESS;
-  int want = group_of(N, V, nb);
-  if (N->group >= want) return OK_SUCCESS;
-  for (;;) {
-    free_training(N);
-    const size_t f = want * n * sizeof(cx<float>);
-    cudaError_t e = cudaMalloc(&N->acts, N->layers * f);
-    if (e == cudaSuccess) e = cudaMalloc(&N->tg[0], f);
-    if (e == cudaSuccess) e = cudaMalloc(&N->tg[1], f);
-    if (e == cudaSuccess) e = cudaMalloc(&N->part, (size_t)N->layers * grad_blocks(V) * NPAR * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&N->lpart, (size_t)want * 2 * loss_blocks(V) * sizeof(double));
-    if (e == cudaSuccess) break;
-    cudaGetLastError();
-    free_training(N);
-    if (want == 1) { set_cuda_error(e); return OK_ECUDA; }
-    want = 1;
+  TrainBufs t;
+  cudaError_t err = cudaSuccess;
+  const int group = grow_group(group_of(N, V, nb), N->t.group, N->most, [&](int q) {
+    err = alloc_training(N, V, q, t);
+    return err == cudaSuccess;
+  });
+  if (t.group) {
+    free_training(N->t);
+    N->t = t;
   }
-  N->group = want;
+  if (!group) { set_cuda_error(err); return OK_ECUDA; }
   return OK_SUCCESS;
 }
 
@@ -430,35 +448,36 @@ int group_backprop(ok_net* N, const ok_W* W, int pairs, const cx<float>* b, cons
   const Geom& g = W->g;
   const long long n = 12LL * g.V, gn = n * pairs;
   const int K = N->layers;
+  cx<float>* const tg[2] = {N->t.tg[0] ? N->t.tg[0] : N->g[0], N->t.tg[1] ? N->t.tg[1] : N->g[1]};
   const cx<float>* in = b;
   for (int l = 0; l < K; ++l) {
-    cx<float>* o = N->acts + (size_t)l * gn;
+    cx<float>* o = N->t.acts + (size_t)l * gn;
     NET_TRY(layer(N, W, l, false, in, o, st, pairs));
     in = o;
   }
   const int lb = loss_blocks(g.V), gb = grad_blocks(g.V);
   {
     TraceScope ts("net_loss", st);
-    net_loss_kernel<<<dim3(lb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, n, N->lpart, N->scal, N->ticket);
+    net_loss_kernel<<<dim3(lb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, n, N->t.lpart, N->scal, N->ticket);
   }
   OK_LAUNCH_CHECK();
   {
     TraceScope ts("net_seed", st);
     const int sb = grid_for(n, 256) < 1024 ? grid_for(n, 256) : 1024;
-    net_seed_kernel<<<dim3(sb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, (float2*)N->tg[0], n, N->scal);
+    net_seed_kernel<<<dim3(sb, pairs), 256, 0, st>>>((const float2*)in, (const float2*)x, (float2*)tg[0], n, N->scal);
   }
   OK_LAUNCH_CHECK();
   int cur = 0;
   for (int l = K - 1; l >= 0; --l) {
-    const cx<float>* lin = l == 0 ? b : N->acts + (size_t)(l - 1) * gn;
+    const cx<float>* lin = l == 0 ? b : N->t.acts + (size_t)(l - 1) * gn;
     {
       TraceScope ts("net_grad", st);
-      net_grad_kernel<<<gb, GRAD_THREADS, 0, st>>>((const cx<float>*)W->L32, N->tg[cur], lin, g, pairs,
-                                                   N->part + (size_t)l * gb * NPAR, !first);
+      net_grad_kernel<<<gb, GRAD_THREADS, 0, st>>>((const cx<float>*)W->L32, tg[cur], lin, g, pairs,
+                                                   N->t.part + (size_t)l * gb * NPAR, !first);
     }
     OK_LAUNCH_CHECK();
     if (l > 0) {
-      NET_TRY(layer(N, W, l, true, N->tg[cur], N->tg[1 - cur], st, pairs));
+      NET_TRY(layer(N, W, l, true, tg[cur], tg[1 - cur], st, pairs));
       cur = 1 - cur;
     }
   }
@@ -470,13 +489,13 @@ int batch_backprop(ok_net* N, const ok_W* W, int nb, const cx<float>* b, const c
   NET_TRY(ensure_workspace(N, W->g.V, nb));
   OK_CUDA_TRY(cudaMemsetAsync(N->scal, 0, sizeof(double), st));
   const size_t n = (size_t)W->g.V * 12;
-  for (int i = 0; i < nb; i += N->group) {
-    const int pairs = nb - i < N->group ? nb - i : N->group;
+  for (int i = 0; i < nb; i += N->t.group) {
+    const int pairs = nb - i < N->t.group ? nb - i : N->t.group;
     NET_TRY(group_backprop(N, W, pairs, b + i * n, x + i * n, i == 0, st));
   }
   {
     TraceScope ts("net_grad_final", st);
-    net_grad_final_kernel<<<N->layers * NOFF, 256, 0, st>>>(N->part, grad_blocks(W->g.V), N->gacc, ad);
+    net_grad_final_kernel<<<N->layers * NOFF, 256, 0, st>>>(N->t.part, grad_blocks(W->g.V), N->gacc, ad);
   }
   OK_LAUNCH_CHECK();
   return OK_SUCCESS;
@@ -585,7 +604,7 @@ int net_create(int layers, const double* w, ok_net** out) {
 void net_free(ok_net* N) {
   if (!N) return;
   cudaFree(N->A); cudaFree(N->m); cudaFree(N->v); cudaFree(N->gacc); cudaFree(N->scal); cudaFree(N->ticket);
-  free_training(N);
+  free_training(N->t);
   cudaFree(N->g[0]); cudaFree(N->g[1]);
   delete N;
 }
