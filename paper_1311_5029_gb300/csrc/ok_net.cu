@@ -194,34 +194,88 @@ __global__ void __launch_bounds__(NET_THREADS) net_layer_kernel(const cx<float>*
   }
 }
 
+// The lanes' floats summed over the warp: returns the sum of C[lane].  It transposes as it sums: each step adds the half of
+// the values that a lane keeps to the same half of its partner's, 31 additions instead of 160.  They are error-free
+// transformations on the FP32 pipes, which keep more bits than FP64 (ok_sum3.cuh), wherever their range allows: some
+// 200 cycles of a multiprocessor, where FP64's additions and conversions, at 1/58 of the FP32 rate, take 900.
+__device__ __forceinline__ double lane_sums(const float (&C)[32], int lane) {
+  constexpr unsigned full = 0xffffffffu;
+  float m = 0.f;   // (a NaN goes through either way)
+#pragma unroll
+  for (int k = 0; k < 32; ++k) m = fmaxf(m, fabsf(C[k]));
+  if (__any_sync(full, m > 0x1p100f)) {
+    double v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float keep = lane & 16 ? C[k + 16] : C[k], send = lane & 16 ? C[k] : C[k + 16];
+      v[k] = (double)keep + (double)__shfl_xor_sync(full, send, 16);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const double keep = lane & o ? v[k + o] : v[k], send = lane & o ? v[k] : v[k + o];
+        v[k] = keep + __shfl_xor_sync(full, send, o);
+      }
+    return v[0];
+  }
+  Sum3 v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float send = lane & 16 ? C[k] : C[k + 16];
+    v[k].s = lane & 16 ? C[k + 16] : C[k];
+    v[k].t = two_sum(v[k].s, __shfl_xor_sync(full, send, 16));
+    v[k].u = 0.f;
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const bool up = lane & o;
+      const Sum3 keep = up ? v[k + o] : v[k];
+      Sum3 send = up ? v[k] : v[k + o];
+      send.s = __shfl_xor_sync(full, send.s, o);
+      send.t = __shfl_xor_sync(full, send.t, o);
+      if (o < 8) send.u = __shfl_xor_sync(full, send.u, o);   // zero before
+      v[k] = keep + send;
+    }
+  return v[0].value();
+}
+
 // Gradient partials: part[block][d][32] = sum over the block's (pair, 32-site tile)s of
 // g(x)_s,c conj((T_d in)(x)_t,c) (16 complex = 32 values).  A block has one warp per offset d, so a
-// warp keeps one offset's 32 sums over all its sites and needs one lane reduction for every
-// GRAD_CHUNK sites of a thread.  (One warp walking all nine offsets took nine five-step FP64 trees
-// of 32 values for one or two sites a thread: the FP64 pipe, 1/58 of the FP32 rate, was 76 % busy
-// and the kernel took 289 us at 16^3 x 32; this form takes 45 us.)  The lane reduction
-// transposes as it sums: each step adds the half of the values that a lane keeps to the same half of
-// its partner's, 31 FP64 additions for the 32 values instead of 160, and leaves value k in lane k.
+// warp keeps one offset's 32 sums over all its sites and takes one lane reduction for every `run` sites of
+// a thread.  (One warp walking all nine offsets took nine five-step FP64 trees of 32 values for one or two sites a
+// thread: the FP64 pipe was 76 % busy and the kernel took 289 us at 16^3 x 32; this form takes 53 us, 48 us a
+// pair in a batch of four.)
 // The nine warps read the same tile's g and neighbours back to back, so L1 shares them.
 constexpr int GRAD_WARPS = NOFF;
 constexpr int GRAD_THREADS = 32 * GRAD_WARPS;
-constexpr int GRAD_CHUNK = 8;
+// Sites that a thread adds up in FP32 before a lane reduction, at most 8: as many as 77824 threads (608 blocks of 128) take
+// of the lattice, which is what one thread per site in a resident grid adds up.  Shorter runs err less, longer ones need
+// fewer reductions.  The gradient's error against 64 bits, mean of 12 fields, and the kernel's time in a batch of four at
+// 16^3 x 32: run 1 2.486e-8, 241 us; 2 (the rule) 2.490e-8, 191 us; 8 2.505e-8, 156 us.  12^3 x 24: run 1 (the rule)
+// 3.329e-8, 81 us; 8 3.354e-8, 55 us.
+int grad_run(int V) {
+  const int r = (V + 77823) / 77824;
+  return r > 8 ? 8 : r;
+}
 __global__ void __launch_bounds__(GRAD_THREADS, 2) net_grad_kernel(const cx<float>* __restrict__ L, const cx<float>* __restrict__ gr,
-                                                                   const cx<float>* __restrict__ in, Geom g, int pairs,
+                                                                   const cx<float>* __restrict__ in, Geom g, int pairs, int run,
                                                                    double* __restrict__ part, bool accumulate) {
   const int lane = threadIdx.x & 31, d = threadIdx.x >> 5;
-  const int ntiles = (g.V + 31) / 32;
-  const long long work = (long long)ntiles * pairs;
+  // (32-bit indices: a group of pairs holds at most 256 MiB of activations, or it is one pair)
+  const unsigned ntiles = (g.V + 31) / 32, work = ntiles * pairs;
   double tot = 0.0;
-  for (long long w0 = blockIdx.x; w0 < work; w0 += (long long)gridDim.x * GRAD_CHUNK) {
+  for (unsigned w0 = blockIdx.x; w0 < work; w0 += gridDim.x * run) {
     float C[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) C[k] = 0.f;
 #pragma unroll 1
-    for (int u = 0; u < GRAD_CHUNK; ++u) {
-      const long long w = w0 + (long long)u * gridDim.x;
+    for (int u = 0; u < run; ++u) {
+      const unsigned w = w0 + u * gridDim.x;
       if (w >= work) break;
-      const int q = (int)(w / ntiles), x = (int)(w % ntiles) * 32 + lane;
+      const int q = w / ntiles, x = w % ntiles * 32 + lane;
       if (x >= g.V) continue;
       const size_t off = (size_t)q * 12 * g.V;
       int c[4];
@@ -240,23 +294,7 @@ __global__ void __launch_bounds__(GRAD_THREADS, 2) net_grad_kernel(const cx<floa
           C[2 * (4 * s + t) + 1] = z.im;
         }
     }
-    // transposing lane reduction: after the step of width o, value index bits >= o are the lane's
-    double v[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const bool up = lane & 16;
-      const float keep = up ? C[k + 16] : C[k], send = up ? C[k] : C[k + 16];
-      v[k] = (double)keep + (double)__shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < o; ++k) {
-        const bool up = lane & o;
-        const double keep = up ? v[k + o] : v[k], send = up ? v[k] : v[k + o];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    tot += v[0];
+    tot += lane_sums(C, lane);
   }
   double* p = part + (size_t)blockIdx.x * NPAR + threadIdx.x;
   *p = accumulate ? *p + tot : tot;
@@ -472,7 +510,7 @@ int group_backprop(ok_net* N, const ok_W* W, int pairs, const cx<float>* b, cons
     const cx<float>* lin = l == 0 ? b : N->t.acts + (size_t)(l - 1) * gn;
     {
       TraceScope ts("net_grad", st);
-      net_grad_kernel<<<gb, GRAD_THREADS, 0, st>>>((const cx<float>*)W->L32, tg[cur], lin, g, pairs,
+      net_grad_kernel<<<gb, GRAD_THREADS, 0, st>>>((const cx<float>*)W->L32, tg[cur], lin, g, pairs, grad_run(g.V),
                                                    N->t.part + (size_t)l * gb * NPAR, !first);
     }
     OK_LAUNCH_CHECK();

@@ -1,4 +1,4 @@
-// Sums with more than FP64's accuracy on the FP32 pipes (the training loss).
+// Sums with more than FP64's accuracy on the FP32 pipes (the training step's loss and gradient).
 #pragma once
 #include <math.h>
 
@@ -28,6 +28,11 @@ __host__ __device__ __forceinline__ float two_sum(float& acc, float x) {
   const float e = (acc - (s - bb)) + (x - bb);
   acc = s;
   return e;
+}
+__host__ __device__ __forceinline__ Sum3 operator+(Sum3 a, Sum3 b) {
+  const float r = two_sum(a.s, b.s), q = two_sum(a.t, b.t);
+  a.u += b.u + (q + two_sum(a.t, r));
+  return a;
 }
 // a += (d + e)^2, d + e a difference and its rounding error (|e| <= 2^-24 |d|).
 __host__ __device__ __forceinline__ void add_square(Sum3& a, float d, float e) {
