@@ -192,56 +192,58 @@ struct WOut {
   cx<__half>* W16;
 };
 
-// The FP32 and FP16 copies of a matrix, in 16-byte words (w_elem).
-__device__ __forceinline__ void store_low(const WOut& o, size_t base, int lane, const M3<float>& f) {
+// The FP32 and FP16 copies of a matrix, in 16-byte words (w_elem); f(e): element e in FP32.
+template <typename F>
+__device__ __forceinline__ void store_low(const WOut& o, size_t base, int lane, F&& f) {
   if (o.W32) {
     cx<float>* p = o.W32 + base;
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      reinterpret_cast<float4*>(p)[q * LANES + lane] = make_float4(f.e[2 * q].re, f.e[2 * q].im, f.e[2 * q + 1].re, f.e[2 * q + 1].im);
-    reinterpret_cast<float2*>(p)[8 * LANES + lane] = make_float2(f.e[8].re, f.e[8].im);
+    for (int q = 0; q < 4; ++q) {
+      const cx<float> u = f(2 * q), v = f(2 * q + 1);
+      reinterpret_cast<float4*>(p)[q * LANES + lane] = make_float4(u.re, u.im, v.re, v.im);
+    }
+    const cx<float> u = f(8);
+    reinterpret_cast<float2*>(p)[8 * LANES + lane] = make_float2(u.re, u.im);
   }
   if (o.W16) {
     cx<__half>* p = o.W16 + base;
-    unsigned h[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      const __half2 v = __halves2half2(__float2half_rn(f.e[e].re), __float2half_rn(f.e[e].im));
-      h[e] = *reinterpret_cast<const unsigned*>(&v);
-    }
+    auto half2 = [&](int e) {
+      const cx<float> u = f(e);
+      const __half2 v = __halves2half2(__float2half_rn(u.re), __float2half_rn(u.im));
+      return *reinterpret_cast<const unsigned*>(&v);
+    };
 #pragma unroll
     for (int q = 0; q < 2; ++q)
-      reinterpret_cast<uint4*>(p)[q * LANES + lane] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-    reinterpret_cast<unsigned*>(p)[8 * LANES + lane] = h[8];
+      reinterpret_cast<uint4*>(p)[q * LANES + lane] = make_uint4(half2(4 * q), half2(4 * q + 1), half2(4 * q + 2), half2(4 * q + 3));
+    reinterpret_cast<unsigned*>(p)[8 * LANES + lane] = half2(8);
   }
 }
 
 __device__ __forceinline__ void store_mat(const WOut& o, int site, int m, const M3<double>& a) {
   const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
   const int lane = site & 31;
-  M3<float> f;
+  M3<float> f;   // converted once: the conversions take the FP64 pipe
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     if (o.W64) o.W64[base + w_elem<double>(e, lane)] = a.e[e];
     if (o.Wdf) o.Wdf[base + w_elem<dd>(e, lane)] = mk<dd>(split_df(a.e[e].re), split_df(a.e[e].im));
     f.e[e] = mk<float>((float)a.e[e].re, (float)a.e[e].im);
   }
-  store_low(o, base, lane, f);
+  store_low(o, base, lane, [&](int e) { return f.e[e]; });
 }
 
 // The same stores from a double-float result (the FP32-pipe precompute, used when no native FP64
 // copy is kept): the double-float copy takes the pairs as they are, the FP32 and FP16 copies the
-// rounded high parts.
+// rounded high parts, formed where their word is stored (kept for the whole matrix, the 18 floats spilled 1408
+// bytes of the kernel's 128 registers: 16^3 x 32, W and its release, 3306 us in FP32 instead of 3200).
 __device__ __forceinline__ void store_mat(const WOut& o, int site, int m, const M3<dd>& a) {
   const size_t base = ((size_t)(site >> 5) * NMAT + m) * (9 * LANES);
   const int lane = site & 31;
-  M3<float> f;
+  if (o.Wdf) {
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    if (o.Wdf) o.Wdf[base + w_elem<dd>(e, lane)] = a.e[e];
-    f.e[e] = mk<float>(a.e[e].re.hi + a.e[e].re.lo, a.e[e].im.hi + a.e[e].im.lo);
+    for (int e = 0; e < 9; ++e) o.Wdf[base + w_elem<dd>(e, lane)] = a.e[e];
   }
-  store_low(o, base, lane, f);
+  store_low(o, base, lane, [&](int e) { return mk<float>(a.e[e].re.hi + a.e[e].re.lo, a.e[e].im.hi + a.e[e].im.lo); });
 }
 
 constexpr int K2_THREADS = 64;
