@@ -10,7 +10,9 @@
 // fewer registers, or the reverse, take as long).  Left to itself the compiler keeps about one hop's loads in
 // flight once the hops form one basic block (122 us at 16^3 x 32); a __syncwarp between a step's requests and
 // its arithmetic keeps it from sinking the loads to their use.  16^3 x 32 / 28^3 x 96, FP32: 98 / 1735 us
-// with the split kernel before, 92 / 1491 us now; FP16: 86 / 1610 us before, 74 / 1373 us now.
+// with the split kernel before, 92 / 1450 us now; FP16: 86 / 1610 us before, 74 / 1375 us now.  14x18x11x27 and 14^3 x 28
+// in FP32 were 1 to 2 % faster with the split kernel: their 2339 and 2401 tiles fill its four rounds of 608 blocks, and 5.1
+// and 5.3 rounds of this kernel's 456.
 #include "ok_pair.cuh"
 
 namespace okgb {
@@ -129,7 +131,11 @@ __device__ __forceinline__ int mat_of(int p) {
   else return M_VIJ + (H - 8) / 2 + 3 * ((H - 8) % 2);
 }
 
-template <typename SH, bool FWD, bool AP, int H0, int H1>
+// Antiperiodic directions (BC): none, time alone (physics runs), any.  Hop h can cross such a boundary.
+enum : int { BC_NONE = 0, BC_TIME = 1, BC_ANY = 2 };
+constexpr bool signed_hop(int h, int bc) { return bc == BC_ANY ? h != 0 : bc == BC_TIME && h == 4; }
+
+template <typename SH, bool FWD, int BC, int H0, int H1>
 struct Ctx {
   using WT = typename SH::W;
 
@@ -141,13 +147,11 @@ struct Ctx {
 };
 
 // The shape of the pipeline for W elements of type T: resident blocks per SM, and how many steps ahead a
-// matrix and a half-spinor are requested.  An FP16 matrix waits in half the registers, so it is
-// requested earlier at four blocks per SM.  FAR: lattices whose time slice of W is large (see launch_pipe).
-template <typename T, bool FAR> struct PipeShape;
-template <> struct PipeShape<float, false> { using W = float; static constexpr int MINB = 3, LA = 3, PLA = 2; };
-template <> struct PipeShape<float, true> { using W = float; static constexpr int MINB = 3, LA = 2, PLA = 2; };
-template <> struct PipeShape<__half, false> { using W = __half; static constexpr int MINB = 4, LA = 5, PLA = 1; };
-template <> struct PipeShape<__half, true> { using W = __half; static constexpr int MINB = 4, LA = 4, PLA = 1; };
+// matrix (LA) and a half-spinor (PLA) are requested.  An FP16 matrix waits in half the registers, so it is
+// requested earlier at four blocks per SM.
+template <typename T, int N> struct PipeShape;
+template <int N> struct PipeShape<float, N> { using W = float; static constexpr int MINB = 3, LA = N, PLA = 2; };
+template <int N> struct PipeShape<__half, N> { using W = __half; static constexpr int MINB = 4, LA = N, PLA = 1; };
 
 template <typename SH>
 struct Bufs {
@@ -164,14 +168,14 @@ constexpr int psi_step(int h, int h0, int pla) {
   return k < 0 ? -1 : k;
 }
 
-template <int H, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ int site_of(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, bool& neg) {
+template <int H, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ int site_of(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, bool& neg) {
   constexpr Off o = hop_off(H, FWD);
-  return nbr_site<o.d[0], o.d[1], o.d[2], o.d[3], AP>(C.c, g, neg);
+  return nbr_site<o.d[0], o.d[1], o.d[2], o.d[3], signed_hop(H, BC)>(C.c, g, neg);
 }
 
-template <int K, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void request(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
+template <int K, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void request(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
   // matrix of step K
   if constexpr (K < first_step(H1, H0)) {
     constexpr int H = hop_of(K, H0), J = sub_of(K, H0);
@@ -187,8 +191,8 @@ __device__ __forceinline__ void request(const Ctx<SH, FWD, AP, H0, H1>& C, const
     B.v[K % (SH::LA + 1)].load(C.W, w, mat_of<H, J, FWD>(C.p));
   }
 }
-template <int H, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void request_psi(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
+template <int H, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void request_psi(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
   bool neg = false;
   int n = C.s;
   if constexpr (!FWD && psi_step(H, H0, SH::PLA) >= first_step(H, H0) - SH::LA) n = B.n[H & 7];  // its matrix request came first
@@ -213,9 +217,9 @@ struct Accs {
   H6<float> y;      // on-site: the sum of the thread's Y term
 };
 
-template <int H, bool AP>
+template <int H, int BC>
 __device__ __forceinline__ void take(H6<float>& m, bool neg) {
-  if constexpr (AP && H != 0) {
+  if constexpr (signed_hop(H, BC)) {
     const float sg = neg ? -1.f : 1.f;
 #pragma unroll
     for (int q = 0; q < 2; ++q)
@@ -224,11 +228,11 @@ __device__ __forceinline__ void take(H6<float>& m, bool neg) {
   }
 }
 
-template <int K, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void compute(const Ctx<SH, FWD, AP, H0, H1>& C, Bufs<SH>& B, Accs& A, float c0q, float a_ii, float b_ii) {
+template <int K, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void compute(const Ctx<SH, FWD, BC, H0, H1>& C, Bufs<SH>& B, Accs& A, float c0q, float a_ii, float b_ii) {
   constexpr int H = hop_of(K, H0), J = sub_of(K, H0);
   const M3<float> V = B.v[K % (SH::LA + 1)].get();
-  if constexpr (J == 0) take<H, AP>(B.m[H % (SH::PLA + 1)], B.neg[H & 7]);
+  if constexpr (J == 0) take<H, BC>(B.m[H % (SH::PLA + 1)], B.neg[H & 7]);
   const H6<float>& m = B.m[H % (SH::PLA + 1)];
   if constexpr (H == 0) {
     if constexpr (J == 0) {
@@ -292,16 +296,16 @@ __device__ __forceinline__ void compute(const Ctx<SH, FWD, AP, H0, H1>& C, Bufs<
   }
 }
 
-template <int H, int K, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void psi_due(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
+template <int H, int K, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void psi_due(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
   if constexpr (H < H1) {
     if constexpr (psi_step(H, H0, SH::PLA) == K) request_psi<H>(C, g, B);
     psi_due<H + 1, K>(C, g, B);
   }
 }
 
-template <int K, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void steps(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Bufs<SH>& B, Accs& A, float c0q, float a_ii,
+template <int K, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void steps(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Bufs<SH>& B, Accs& A, float c0q, float a_ii,
                                       float b_ii) {
   if constexpr (K < first_step(H1, H0)) {
     request<K + SH::LA>(C, g, B);
@@ -312,16 +316,16 @@ __device__ __forceinline__ void steps(const Ctx<SH, FWD, AP, H0, H1>& C, const G
   }
 }
 
-template <int K, typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void prologue(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
+template <int K, typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void prologue(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Bufs<SH>& B) {
   if constexpr (K < SH::LA) {
     request<K>(C, g, B);
     prologue<K + 1>(C, g, B);
   }
 }
 
-template <typename SH, bool FWD, bool AP, int H0, int H1>
-__device__ __forceinline__ void run_part(const Ctx<SH, FWD, AP, H0, H1>& C, const Geom& g, Accs& A, float c0q, float a_ii, float b_ii) {
+template <typename SH, bool FWD, int BC, int H0, int H1>
+__device__ __forceinline__ void run_part(const Ctx<SH, FWD, BC, H0, H1>& C, const Geom& g, Accs& A, float c0q, float a_ii, float b_ii) {
   Bufs<SH> B;
 #pragma unroll
   for (int k = 0; k < 8; ++k) B.neg[k] = false;
@@ -330,7 +334,7 @@ __device__ __forceinline__ void run_part(const Ctx<SH, FWD, AP, H0, H1>& C, cons
   steps<0>(C, g, B, A, c0q, a_ii, b_ii);
 }
 
-template <typename SH, bool AP>
+template <typename SH, int BC>
 __global__ void __launch_bounds__(PIPE_THREADS, SH::MINB)
     apply_pipe_kernel(const cx<typename SH::W>* __restrict__ W, const cx<float>* __restrict__ psi, cx<float>* __restrict__ out, Geom g,
                       float c0q, float a_ii, float b_ii, int spread, const int* halt) {
@@ -363,11 +367,11 @@ __global__ void __launch_bounds__(PIPE_THREADS, SH::MINB)
     c[1] = r % g.L[1]; r /= g.L[1];
     c[2] = r % g.L[2]; c[3] = r / g.L[2];
     if (half == 0) {
-      const Ctx<SH, true, AP, 0, NHOPS> C{W, psi, sc, pr.p, {c[0], c[1], c[2], c[3]}, pr};
+      const Ctx<SH, true, BC, 0, NHOPS> C{W, psi, sc, pr.p, {c[0], c[1], c[2], c[3]}, pr};
       run_part(C, g, A, c0q, a_ii, b_ii);
       to_h(A.d, pr, A.acc);
     } else {
-      const Ctx<SH, false, AP, 1, NHOPS> C{W, psi, sc, pr.p, {c[0], c[1], c[2], c[3]}, pr};
+      const Ctx<SH, false, BC, 1, NHOPS> C{W, psi, sc, pr.p, {c[0], c[1], c[2], c[3]}, pr};
       run_part(C, g, A, c0q, a_ii, b_ii);
       to_h(A.d, pr, A.acc);
 #pragma unroll
@@ -402,7 +406,7 @@ constexpr int SMALL_SITES = 16;
 template <typename WT, bool FWD, int H0, int H1>
 __device__ __forceinline__ void small_part(const cx<WT>* W, const cx<float>* psi, int s, const int (&c)[4], const Pair& pr,
                                            const Geom& g, Accs& A, float c0q, float a_ii, float b_ii) {
-  const Ctx<PipeShape<WT, false>, FWD, true, H0, H1> C{W, psi, s, pr.p, {c[0], c[1], c[2], c[3]}, pr};
+  const Ctx<PipeShape<WT, sizeof(WT) == 2 ? 5 : 3>, FWD, BC_ANY, H0, H1> C{W, psi, s, pr.p, {c[0], c[1], c[2], c[3]}, pr};
   run_part(C, g, A, c0q, a_ii, b_ii);
 }
 
@@ -469,11 +473,11 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2)
   if (s0 < g.V) store_half<float>(out, s, pr.p, o);
 }
 
-template <typename SH, bool AP>
+template <typename SH, int BC>
 void launch(const cx<typename SH::W>* W, const cx<float>* psi, cx<float>* out, const Geom& g, float c0q, float a, float b, const int* halt,
             cudaStream_t st) {
   static int resident = 0;
-  auto kern = apply_pipe_kernel<SH, AP>;
+  auto kern = apply_pipe_kernel<SH, BC>;
   if (resident == 0) {
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, PIPE_THREADS, 0) != cudaSuccess || nb < 1) nb = 1;
@@ -499,20 +503,42 @@ void launch_pipe(const cx<WT>* W, const cx<float>* psi, cx<float>* out, const Ge
     apply_small_kernel<WT><<<small, SMALL_THREADS, 0, st>>>(W, psi, out, g, c0q, a, b, halt);
     return;
   }
-  // FAR: the backward temporal hop reads W a time slice back.  Where a slice outgrows what L2 still holds
-  // from a slice ago, fewer blocks' requests ahead keep more of it.  Measured (us, near / far): FP32
-  // 24^3 x 64, slice 43 MB, 584 / 603; 28^3 x 48, 68 MB, 773 / 737; 28^3 x 96 1657 / 1491.  FP16 16^3 x 32,
-  // slice 6.3 MB, 77 / 74; 20^3 x 64, 12 MB, 296 / 280; 28^3 x 96, 34 MB, 1419 / 1373.
+  // The form of the boundaries and the lookahead.  The requests are the same in all forms, but the compiler schedules
+  // each in its own way, and which is the fastest was found by measurement: us, old form / new form, before the slash
+  // the sign of every hop as a multiplication, behind it only the temporal hop's (BC_TIME, for periodic lattices too).
+  //   FP32, time antiperiodic: 14x18x11x27 63.0 / 60.6; 20^3 x 64 350 / 337; 28^3 x 96 1532 / 1445.  Periodic, against the
+  //   form without signs: 61.6 / 60.6; 343 / 337; 1461 / 1445.
+  //   FP16, time antiperiodic: 14x18x11x27 47.0 / 45.1; 18^3 x 36 126 / 117; 20^3 x 64 296 / 282; 28^3 x 48 663 / 648 and 647 /
+  //   660 in two runs.  Periodic: 45.1 / 45.1; 117 / 117; 276 / 282; 24^3 x 64 480 / 506, so there the form without signs stays.
+  // LA against the bytes of a time slice of W (us, LA 2 / 3 and 4 / 5; the crossover lies between the two nearest):
+  //   FP32 BC_TIME: 9 MB (14^3 x 28) 61.5 / 63.0; 43 MB (24^3 x 64) 578 / 590; 68 MB (28^3 x 48) 797 / 729.
+  //   FP32 BC_ANY the other way round: 43 MB 627 / 593; 68 MB 770 / 755; 28^3 x 96 1533 / 1585.
+  //   FP16 BC_NONE: 4.2 MB (14^3 x 28) 46.6 / 45.2, 11x15x9x40 43.3 / 41.7; 6.3 MB (16^3 x 32) 74.1 / 79.4, 12 MB (20^3 x 64)
+  //   276 / 305, 34 MB (28^3 x 96) 1349 / 1417; against the rule 10^3 x 20 19.9 / 21.1 and 18^3 x 36 117.1 / 116.1.
+  //   FP16 BC_ANY: 4.2 MB 49.2 / 47.2; 6.3 MB 78.9 / 82.3; 12 MB 301 / 331; against the rule 18^3 x 36 125.8 / 121.6.
+  //   FP16 BC_TIME: LA 4 from 1 % slower (14x14x16x59 104.5 / 103.3) to 5 % faster (12^3 x 24 32.9 / 34.6) everywhere.
   const size_t slice = (size_t)g.L[0] * g.L[1] * g.L[2] * SITE_ELEMS * sizeof(cx<WT>);
-  const bool far = slice > (sizeof(WT) == 2 ? (size_t)6 << 20 : (size_t)56 << 20);
-  using Near = PipeShape<WT, false>;
-  using Far = PipeShape<WT, true>;
-  if (far) {
-    if (g.bcneg) launch<Far, true>(W, psi, out, g, c0q, a, b, halt, st);
-    else launch<Far, false>(W, psi, out, g, c0q, a, b, halt, st);
+  const bool time_only = (g.bcneg & ~8) == 0;
+  if constexpr (sizeof(WT) == 4) {
+    const bool wide = slice > (size_t)56 << 20;
+    if (time_only) {
+      if (wide) launch<PipeShape<WT, 3>, BC_TIME>(W, psi, out, g, c0q, a, b, halt, st);
+      else launch<PipeShape<WT, 2>, BC_TIME>(W, psi, out, g, c0q, a, b, halt, st);
+    } else {
+      if (wide) launch<PipeShape<WT, 2>, BC_ANY>(W, psi, out, g, c0q, a, b, halt, st);
+      else launch<PipeShape<WT, 3>, BC_ANY>(W, psi, out, g, c0q, a, b, halt, st);
+    }
   } else {
-    if (g.bcneg) launch<Near, true>(W, psi, out, g, c0q, a, b, halt, st);
-    else launch<Near, false>(W, psi, out, g, c0q, a, b, halt, st);
+    const bool wide = slice > (size_t)5 << 20;
+    if (g.bcneg == 8) {
+      launch<PipeShape<WT, 4>, BC_TIME>(W, psi, out, g, c0q, a, b, halt, st);
+    } else if (g.bcneg == 0) {
+      if (wide) launch<PipeShape<WT, 4>, BC_NONE>(W, psi, out, g, c0q, a, b, halt, st);
+      else launch<PipeShape<WT, 5>, BC_NONE>(W, psi, out, g, c0q, a, b, halt, st);
+    } else {
+      if (wide) launch<PipeShape<WT, 4>, BC_ANY>(W, psi, out, g, c0q, a, b, halt, st);
+      else launch<PipeShape<WT, 5>, BC_ANY>(W, psi, out, g, c0q, a, b, halt, st);
+    }
   }
 }
 template void launch_pipe<float>(const cx<float>*, const cx<float>*, cx<float>*, const Geom&, float, float, float, const int*, cudaStream_t);
