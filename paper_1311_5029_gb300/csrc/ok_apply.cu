@@ -563,44 +563,44 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 4)
     Halves<R> hs;
     zero_halves(hs);
     // Every forward thread takes part in the waits and barriers, active or not.
-    { auto w = chunk(M_UT); if (active) pair_time<R, true, true>(w, psi, c, g, s, pr, hs); release(); }
+    { auto w = chunk(M_UT); if (active) pair_time<R, true>(w, psi, c, g, s, pr, hs); release(); }
     {
       auto w = chunk(M_VII);
       if (active) {
-        pair_two<R, 0, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
-        pair_two<R, 1, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
-        pair_two<R, 2, true, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
+        pair_two<R, 0, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
+        pair_two<R, 1, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
+        pair_two<R, 2, true>(w, psi, c, g, s, pr, a_ii, b_ii, hs);
       }
       release();
     }
     {
       auto w = chunk(M_VIJ);
       if (active) {
-        pair_diag<R, 0, 1, 0, true, true>(w, psi, c, g, s, pr, hs);
-        pair_diag<R, 0, 2, 1, true, true>(w, psi, c, g, s, pr, hs);
-        pair_diag<R, 1, 2, 2, true, true>(w, psi, c, g, s, pr, hs);
+        pair_diag<R, 0, 1, 0, true>(w, psi, c, g, s, pr, hs);
+        pair_diag<R, 0, 2, 1, true>(w, psi, c, g, s, pr, hs);
+        pair_diag<R, 1, 2, 2, true>(w, psi, c, g, s, pr, hs);
         to_h(hs, pr, acc);
       }
       release();
     }
     { auto w = chunk(M_Y0P); if (active) pair_onsite<R>(w, psi, s, pr, c0q, acc); release(); }
-    { auto w = chunk(M_WP + 0); if (active) pair_spatial<R, 0, true, true>(w, psi, c, g, s, pr, acc); release(); }
-    { auto w = chunk(M_WP + 8); if (active) pair_spatial<R, 1, true, true>(w, psi, c, g, s, pr, acc); release(); }
-    { auto w = chunk(M_WP + 16); if (active) pair_spatial<R, 2, true, true>(w, psi, c, g, s, pr, acc); release(); }
+    { auto w = chunk(M_WP + 0); if (active) pair_spatial<R, 0, true>(w, psi, c, g, s, pr, acc); release(); }
+    { auto w = chunk(M_WP + 8); if (active) pair_spatial<R, 1, true>(w, psi, c, g, s, pr, acc); release(); }
+    { auto w = chunk(M_WP + 16); if (active) pair_spatial<R, 2, true>(w, psi, c, g, s, pr, acc); release(); }
   } else if (active) {
     Halves<R> hs;
     zero_halves(hs);
-    pair_time<R, false, true>(Wg, psi, c, g, s, pr, hs);
-    pair_two<R, 0, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
-    pair_two<R, 1, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
-    pair_two<R, 2, false, true>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
-    pair_diag<R, 0, 1, 0, false, true>(Wg, psi, c, g, s, pr, hs);
-    pair_diag<R, 0, 2, 1, false, true>(Wg, psi, c, g, s, pr, hs);
-    pair_diag<R, 1, 2, 2, false, true>(Wg, psi, c, g, s, pr, hs);
+    pair_time<R, false>(Wg, psi, c, g, s, pr, hs);
+    pair_two<R, 0, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_two<R, 1, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_two<R, 2, false>(Wg, psi, c, g, s, pr, a_ii, b_ii, hs);
+    pair_diag<R, 0, 1, 0, false>(Wg, psi, c, g, s, pr, hs);
+    pair_diag<R, 0, 2, 1, false>(Wg, psi, c, g, s, pr, hs);
+    pair_diag<R, 1, 2, 2, false>(Wg, psi, c, g, s, pr, hs);
     to_h(hs, pr, acc);
-    pair_spatial<R, 0, false, true>(Wg, psi, c, g, s, pr, acc);
-    pair_spatial<R, 1, false, true>(Wg, psi, c, g, s, pr, acc);
-    pair_spatial<R, 2, false, true>(Wg, psi, c, g, s, pr, acc);
+    pair_spatial<R, 0, false>(Wg, psi, c, g, s, pr, acc);
+    pair_spatial<R, 1, false>(Wg, psi, c, g, s, pr, acc);
+    pair_spatial<R, 2, false>(Wg, psi, c, g, s, pr, acc);
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq)
 #pragma unroll

@@ -41,32 +41,32 @@ __device__ __forceinline__ void mr_block2h(const WS& W, int site, int m, const H
   for (int r = 0; r < NR; ++r) { if (DAG) mdv_add(acc[r].v[1], b, h[r].v[1]); else mv_add(acc[r].v[1], b, h[r].v[1]); }
 }
 
-template <typename R, int NR, int I, bool FWD, bool AP, typename WS>
+template <typename R, int NR, int I, bool FWD, typename WS>
 __device__ __forceinline__ void mr_spatial(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
                                            const Geom& g, int s, const Pair& pr, H6<R> (&acc)[NR]) {
   const int base = M_WP + 8 * I;
   H6<R> h[NR];
   if constexpr (FWD) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) gather_pair<R, I == 0, I == 1, I == 2, 0, AP>(psi + r * rs, c, g, pr, h[r]);
+    for (int r = 0; r < NR; ++r) gather_pair<R, I == 0, I == 1, I == 2, 0>(psi + r * rs, c, g, pr, h[r]);
     mr_block2h<R, NR, false>(W, s, base + 4 * pr.p, h, acc);
   } else {
     int n = 0;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) n = gather_pair<R, -(I == 0), -(I == 1), -(I == 2), 0, AP>(psi + r * rs, c, g, pr, h[r]);
+    for (int r = 0; r < NR; ++r) n = gather_pair<R, -(I == 0), -(I == 1), -(I == 2), 0>(psi + r * rs, c, g, pr, h[r]);
     mr_block2h<R, NR, true>(W, n, base + 4 * (1 - pr.p), h, acc);
   }
 }
 
 // The hops without exchange between the threads (see pair_time, pair_two, pair_diag): each matrix is
 // applied to the thread's own halves of NR right-hand sides.
-template <typename R, int NR, bool FWD, bool AP, typename WS>
+template <typename R, int NR, bool FWD, typename WS>
 __device__ __forceinline__ void mr_time(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
                                         const Geom& g, int s, const Pair& pr, Halves<R> (&d)[NR]) {
   H6<R> m[NR];
   if constexpr (FWD) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) gather_mine<R, 0, 0, 0, 1, AP>(psi + r * rs, c, g, pr, m[r]);
+    for (int r = 0; r < NR; ++r) gather_mine<R, 0, 0, 0, 1>(psi + r * rs, c, g, pr, m[r]);
     M3<R> A = W(s, M_ST + 0);
 #pragma unroll
     for (int r = 0; r < NR; ++r) { mv_add(d[r].cross.v[0], A, m[r].v[0]); mv_sub(d[r].cross.v[1], A, m[r].v[1]); }
@@ -82,7 +82,7 @@ __device__ __forceinline__ void mr_time(const WS& W, const cx<R>* __restrict__ p
   } else {
     int n = 0;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) n = gather_mine<R, 0, 0, 0, -1, AP>(psi + r * rs, c, g, pr, m[r]);
+    for (int r = 0; r < NR; ++r) n = gather_mine<R, 0, 0, 0, -1>(psi + r * rs, c, g, pr, m[r]);
     M3<R> A = W(n, M_ST + 0);
 #pragma unroll
     for (int r = 0; r < NR; ++r) { mdv_sub(d[r].cross.v[0], A, m[r].v[0]); mdv_add(d[r].cross.v[1], A, m[r].v[1]); }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void mr_time(const WS& W, const cx<R>* __restrict__ p
   }
 }
 
-template <typename R, int NR, int I, bool FWD, bool AP, typename WS>
+template <typename R, int NR, int I, bool FWD, typename WS>
 __device__ __forceinline__ void mr_two(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
                                        const Geom& g, int s, const Pair& pr, R a, R b, Halves<R> (&d)[NR]) {
   constexpr int f = FWD ? 1 : -1;
@@ -106,7 +106,7 @@ __device__ __forceinline__ void mr_two(const WS& W, const cx<R>* __restrict__ ps
   int n = s;
 #pragma unroll
   for (int r = 0; r < NR; ++r)
-    n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0, AP>(psi + r * rs, c, g, pr, m[r]);
+    n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0>(psi + r * rs, c, g, pr, m[r]);
   const M3<R> V = W(FWD ? s : n, M_VII + I);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
@@ -117,7 +117,7 @@ __device__ __forceinline__ void mr_two(const WS& W, const cx<R>* __restrict__ ps
   }
 }
 
-template <typename R, int NR, int I, int J, int P, bool FWD, bool AP, typename WS>
+template <typename R, int NR, int I, int J, int P, bool FWD, typename WS>
 __device__ __forceinline__ void mr_diag(const WS& W, const cx<R>* __restrict__ psi, long long rs, const int (&c)[4],
                                         const Geom& g, int s, const Pair& pr, Halves<R> (&d)[NR]) {
   constexpr int f = FWD ? 1 : -1;
@@ -127,7 +127,7 @@ __device__ __forceinline__ void mr_diag(const WS& W, const cx<R>* __restrict__ p
   int n = s;
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    n = gather_mine<R, f * A0, f * A1, f * A2, 0, AP>(psi + r * rs, c, g, pr, m);
+    n = gather_mine<R, f * A0, f * A1, f * A2, 0>(psi + r * rs, c, g, pr, m);
     sigma_pair<R, I, J, 1>(m, y[r]);
   }
   M3<R> V = W(FWD ? s : n, M_VIJ + P);
@@ -135,7 +135,7 @@ __device__ __forceinline__ void mr_diag(const WS& W, const cx<R>* __restrict__ p
   for (int r = 0; r < NR; ++r) colour2h_acc<R, !FWD>(d[r].cross, V, y[r]);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
-    n = gather_mine<R, f * B0, f * B1, f * B2, 0, AP>(psi + r * rs, c, g, pr, m);
+    n = gather_mine<R, f * B0, f * B1, f * B2, 0>(psi + r * rs, c, g, pr, m);
     sigma_pair<R, I, J, -1>(m, y[r]);
   }
   V = W(FWD ? s : n, M_XIJ + P);
@@ -143,7 +143,7 @@ __device__ __forceinline__ void mr_diag(const WS& W, const cx<R>* __restrict__ p
   for (int r = 0; r < NR; ++r) colour2h_acc<R, !FWD>(d[r].cross, V, y[r]);
 }
 
-template <int NR, int EPI, typename WT, bool AP = true>
+template <int NR, int EPI, typename WT>
 __global__ void __launch_bounds__(MR_THREADS, mr_minb<NR>())
     apply_mrhs_kernel(const cx<WT>* __restrict__ W, const cx<float>* __restrict__ psi, cx<float>* __restrict__ out, long long rs,
                       Geom g, float c0q, float a_ii, float b_ii, MultiEpi ep) {
@@ -192,33 +192,33 @@ __global__ void __launch_bounds__(MR_THREADS, mr_minb<NR>())
 #pragma unroll
       for (int r = 0; r < NR; ++r) zero_halves(hs[r]);
       if (half == 0) {
-        mr_time<R, NR, true, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_two<R, NR, 0, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_two<R, NR, 1, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_two<R, NR, 2, true, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_diag<R, NR, 0, 1, 0, true, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_diag<R, NR, 0, 2, 1, true, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_diag<R, NR, 1, 2, 2, true, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_time<R, NR, true>(Wg, P, rs, c, g, s, pr, hs);
+        mr_two<R, NR, 0, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 1, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 2, true>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_diag<R, NR, 0, 1, 0, true>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 0, 2, 1, true>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 1, 2, 2, true>(Wg, P, rs, c, g, s, pr, hs);
 #pragma unroll
         for (int r = 0; r < NR; ++r) to_h(hs[r], pr, acc[r]);
 #pragma unroll
         for (int r = 0; r < NR; ++r) pair_onsite<R>(Wg, P + r * rs, s, pr, c0q, acc[r]);
-        mr_spatial<R, NR, 0, true, AP>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 1, true, AP>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 2, true, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 0, true>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 1, true>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 2, true>(Wg, P, rs, c, g, s, pr, acc);
       } else {
-        mr_time<R, NR, false, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_two<R, NR, 0, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_two<R, NR, 1, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_two<R, NR, 2, false, AP>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
-        mr_diag<R, NR, 0, 1, 0, false, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_diag<R, NR, 0, 2, 1, false, AP>(Wg, P, rs, c, g, s, pr, hs);
-        mr_diag<R, NR, 1, 2, 2, false, AP>(Wg, P, rs, c, g, s, pr, hs);
+        mr_time<R, NR, false>(Wg, P, rs, c, g, s, pr, hs);
+        mr_two<R, NR, 0, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 1, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_two<R, NR, 2, false>(Wg, P, rs, c, g, s, pr, a_ii, b_ii, hs);
+        mr_diag<R, NR, 0, 1, 0, false>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 0, 2, 1, false>(Wg, P, rs, c, g, s, pr, hs);
+        mr_diag<R, NR, 1, 2, 2, false>(Wg, P, rs, c, g, s, pr, hs);
 #pragma unroll
         for (int r = 0; r < NR; ++r) to_h(hs[r], pr, acc[r]);
-        mr_spatial<R, NR, 0, false, AP>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 1, false, AP>(Wg, P, rs, c, g, s, pr, acc);
-        mr_spatial<R, NR, 2, false, AP>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 0, false>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 1, false>(Wg, P, rs, c, g, s, pr, acc);
+        mr_spatial<R, NR, 2, false>(Wg, P, rs, c, g, s, pr, acc);
 #pragma unroll
         for (int r = 0; r < NR; ++r)
 #pragma unroll

@@ -210,19 +210,17 @@ struct Pair {
 
 // The thread's own half of the neighbour at offset D, with the boundary sign (a multiplication, not a
 // branch: the hops stay one basic block, so the loads of the next hop can be issued early).
-template <typename R, int D0, int D1, int D2, int D3, bool AP>
+template <typename R, int D0, int D1, int D2, int D3>
 __device__ __forceinline__ int gather_mine(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
                                            H6<R>& mine) {
   bool neg;
-  const int n = nbr_site<D0, D1, D2, D3, AP>(c, g, neg);
+  const int n = nbr_site<D0, D1, D2, D3>(c, g, neg);
   load_half<R>(psi, n, pr.p, mine);
-  if constexpr (AP) {
-    const R sg = neg ? R(-1) : R(1);
+  const R sg = neg ? R(-1) : R(1);
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+  for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) mine.v[s][a] = sg * mine.v[s][a];
-  }
+    for (int a = 0; a < 3; ++a) mine.v[s][a] = sg * mine.v[s][a];
   return n;
 }
 
@@ -241,11 +239,11 @@ __device__ __forceinline__ void halves_to_h(const H6<R>& mine, const Pair& pr, H
 }
 
 // h+ (p = 0) or h- (p = 1) of the neighbour at offset D.
-template <typename R, int D0, int D1, int D2, int D3, bool AP>
+template <typename R, int D0, int D1, int D2, int D3>
 __device__ __forceinline__ int gather_pair(const cx<R>* __restrict__ psi, const int (&c)[4], const Geom& g, const Pair& pr,
                                            H6<R>& h) {
   H6<R> mine;
-  const int n = gather_mine<R, D0, D1, D2, D3, AP>(psi, c, g, pr, mine);
+  const int n = gather_mine<R, D0, D1, D2, D3>(psi, c, g, pr, mine);
   halves_to_h(mine, pr, h);
   return n;
 }
@@ -317,12 +315,12 @@ __device__ __forceinline__ void colour2h(H6<R>& y, const M3<R>& V, const H6<R>& 
 
 // Each hop function does the forward (FWD) or the backward half of its part of the stencil; the two
 // run in different warps.
-template <typename R, int I, bool FWD, bool AP, typename WS>
+template <typename R, int I, bool FWD, typename WS>
 __device__ __forceinline__ void pair_spatial(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                              const Geom& g, int s, const Pair& pr, H6<R>& acc) {
   constexpr int base = M_WP + 8 * I, f = FWD ? 1 : -1;
   H6<R> h;
-  const int n = gather_pair<R, f * (I == 0), f * (I == 1), f * (I == 2), 0, AP>(psi, c, g, pr, h);
+  const int n = gather_pair<R, f * (I == 0), f * (I == 1), f * (I == 2), 0>(psi, c, g, pr, h);
   if constexpr (FWD) block2h<R, false>(W, s, base + 4 * pr.p, h, acc);
   else block2h<R, true>(W, n, base + 4 * (1 - pr.p), h, acc);
 }
@@ -338,12 +336,12 @@ __device__ __forceinline__ void only(H6<R>& m, bool mine) {
 
 // On (u, l): W^+_4 = [[0, S], [S, -U]] with the matrices at x, W^-_4 = [[-U^dag, -S^dag], [-S^dag, 0]]
 // with those at x - t (halves stored); S = [[s3, n1], [n2, -s3]].
-template <typename R, bool FWD, bool AP, typename WS>
+template <typename R, bool FWD, typename WS>
 __device__ __forceinline__ void pair_time(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                           const Geom& g, int s, const Pair& pr, Halves<R>& d) {
   H6<R> m;
   if constexpr (FWD) {
-    gather_mine<R, 0, 0, 0, 1, AP>(psi, c, g, pr, m);
+    gather_mine<R, 0, 0, 0, 1>(psi, c, g, pr, m);
     M3<R> A = W(s, M_ST + 0);
     mv_add(d.cross.v[0], A, m.v[0]);
     mv_sub(d.cross.v[1], A, m.v[1]);
@@ -357,7 +355,7 @@ __device__ __forceinline__ void pair_time(const WS& W, const cx<R>* __restrict__
     mv_sub(d.same.v[1], A, m.v[1]);
   } else {
     // S^dag = [[s3^dag, n2^dag], [n1^dag, -s3^dag]]
-    const int n = gather_mine<R, 0, 0, 0, -1, AP>(psi, c, g, pr, m);
+    const int n = gather_mine<R, 0, 0, 0, -1>(psi, c, g, pr, m);
     M3<R> A = W(n, M_ST + 0);
     mdv_sub(d.cross.v[0], A, m.v[0]);
     mdv_add(d.cross.v[1], A, m.v[1]);
@@ -384,12 +382,12 @@ __device__ __forceinline__ void add_scaled_h(H6<R>& acc, R a, const H6<R>& y) {
 }
 
 // W^{++}_ii = [[a, b sigma_i], [b sigma_i, a]] (x) V forward, [[a, -b sigma_i], [-b sigma_i, a]] (x) V^dag backward.
-template <typename R, int I, bool FWD, bool AP, typename WS>
+template <typename R, int I, bool FWD, typename WS>
 __device__ __forceinline__ void pair_two(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                          const Geom& g, int s, const Pair& pr, R a, R b, Halves<R>& d) {
   constexpr int f = FWD ? 1 : -1;
   H6<R> m, y;
-  const int n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0, AP>(psi, c, g, pr, m);
+  const int n = gather_mine<R, 2 * f * (I == 0), 2 * f * (I == 1), 2 * f * (I == 2), 0>(psi, c, g, pr, m);
   const M3<R> V = W(FWD ? s : n, M_VII + I);
   colour2h<R, !FWD>(y, V, m);
   add_scaled_h(d.same, a, y);
@@ -423,18 +421,18 @@ __device__ __forceinline__ void colour2h_acc(H6<R>& y, const M3<R>& V, const H6<
 
 // Diagonal pair (I, J): [[0, S], [S, 0]] with S = (s_I + s_J) (x) V from x+I+J and (s_I - s_J) (x) X from
 // x+I-J (forward), minus their adjoints from x-I-J and x-I+J (backward).
-template <typename R, int I, int J, int P, bool FWD, bool AP, typename WS>
+template <typename R, int I, int J, int P, bool FWD, typename WS>
 __device__ __forceinline__ void pair_diag(const WS& W, const cx<R>* __restrict__ psi, const int (&c)[4],
                                           const Geom& g, int s, const Pair& pr, Halves<R>& d) {
   constexpr int f = FWD ? 1 : -1;
   constexpr int A0 = (I == 0) + (J == 0), A1 = (I == 1) + (J == 1), A2 = (I == 2) + (J == 2);
   constexpr int B0 = (I == 0) - (J == 0), B1 = (I == 1) - (J == 1), B2 = (I == 2) - (J == 2);
   H6<R> m, y;
-  int n = gather_mine<R, f * A0, f * A1, f * A2, 0, AP>(psi, c, g, pr, m);
+  int n = gather_mine<R, f * A0, f * A1, f * A2, 0>(psi, c, g, pr, m);
   sigma_pair<R, I, J, 1>(m, y);
   M3<R> V = W(FWD ? s : n, M_VIJ + P);
   colour2h_acc<R, !FWD>(d.cross, V, y);
-  n = gather_mine<R, f * B0, f * B1, f * B2, 0, AP>(psi, c, g, pr, m);
+  n = gather_mine<R, f * B0, f * B1, f * B2, 0>(psi, c, g, pr, m);
   sigma_pair<R, I, J, -1>(m, y);
   V = W(FWD ? s : n, M_XIJ + P);
   colour2h_acc<R, !FWD>(d.cross, V, y);
