@@ -1,10 +1,34 @@
-// The table that the double-float apply (ok_apply_dd.cu) walks, built on the host: the 27 offsets
-// of Eq. minFlopForm and, for each, its colour matrix-vector products with their accumulators,
-// factors and units.  The entries follow the hop functions of ok_apply.cu term by term.
+// The colour matrix-vector products of one application of M (Eq. minFlopForm) as one list on the h+- halves: 27 offsets and,
+// for each, its products with their accumulators, factors and units.  No kernel walks it: it is the statement of the
+// products that the host tests hold the entries of ok_dd_entries.cuh against, which the double-float apply walks.
 #pragma once
-#include "ok_dd.cuh"
+#include "ok_internal.cuh"
 
 namespace okgb {
+
+struct DDHop {
+  signed char d[4];       // offset (x, y, z, t)
+  unsigned char kind;     // DD_ONSITE, DD_PLAIN, DD_THIRD_L, DD_THIRD_U
+  unsigned char first;    // first action
+  unsigned char count;    // number of actions
+  unsigned char pad;
+};
+struct DDAct {
+  unsigned char m;        // colour matrix of the site record (0 .. 42)
+  unsigned char flags;    // bit 0: matrix at the offset's site (else at x); bit 1: adjoint;
+                          // bits 2-4: source (slot * 2 + spin)
+  signed char dst[2];     // accumulator (half * 2 + spin: acc+ 0, 1; acc- 2, 3), or -1
+  unsigned char mul[2];   // bits 0-1: scalar (1, a_ii, b_ii); bits 2-4: unit (1, i, -1, -i, 1+i, 1-i, -1-i, -1+i)
+  unsigned char pad[2];
+};
+constexpr int DD_HOPS = 27;
+constexpr int DD_ACTS = 148;
+enum : int { DD_ONSITE = 0, DD_PLAIN = 1, DD_THIRD_L = 2, DD_THIRD_U = 3 };
+struct DDTable {
+  DDHop hop[DD_HOPS];
+  DDAct act[DD_ACTS];
+};
+
 namespace ddtab {
 
 // Table entries: sources (slot * 2 + spin), accumulators (half * 2 + spin), scalars and units.
