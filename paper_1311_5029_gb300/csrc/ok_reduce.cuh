@@ -15,19 +15,11 @@ struct dcx { double re, im; };
 
 __host__ __device__ __forceinline__ dcx dmk(double a, double b) { dcx z; z.re = a; z.im = b; return z; }
 __host__ __device__ __forceinline__ dcx dmul(dcx a, dcx b) { return dmk(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
-// x / d and y / d.  The finalisations run on one thread, where an FP64 division is a long chain, so both share one:
-// q = x (1 / d), put right by its exact remainder, q + (x - q d) (1 / d) (Markstein, IBM J. Res. Dev. 34 (1990)), where
-// nothing on the way can leave the normal range; the divisions themselves elsewhere.
-__host__ __device__ __forceinline__ bool quot_range(double x) { return fabs(x) >= 0x1p-400 && fabs(x) <= 0x1p400; }
-__host__ __device__ __forceinline__ dcx quot2(double x, double y, double d) {
-  if (quot_range(d) && (x == 0.0 || quot_range(x)) && (y == 0.0 || quot_range(y))) {
-    const double r = 1.0 / d, p = x * r, q = y * r;
-    return dmk(::fma(::fma(-p, d, x), r, p), ::fma(::fma(-q, d, y), r, q));
-  }
-  return dmk(x / d, y / d);
-}
+// Two divisions: with 1 / |b|^2 the quotients take one rounding more, and are infinite for |b|^2 below 5.6e-309 where they need
+// not be.  (A reciprocal saves 1 us of 315 an iteration at 16^3 x 32, and nothing when its rounding is put right.)
 __host__ __device__ __forceinline__ dcx ddiv(dcx a, dcx b) {
-  return quot2(a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im, b.re * b.re + b.im * b.im);
+  const double d = b.re * b.re + b.im * b.im;
+  return dmk((a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d);
 }
 __host__ __device__ __forceinline__ double dabs2(dcx a) { return a.re * a.re + a.im * a.im; }
 __host__ __device__ __forceinline__ bool dfinite(dcx a) { return isfinite(a.re) && isfinite(a.im); }
