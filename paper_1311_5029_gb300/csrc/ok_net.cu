@@ -12,8 +12,8 @@
 //             The adjoint layer L^dag = sum_d A_d^dag T_{-d} is the same kernel with the offsets
 //             reversed and the weights conjugate-transposed.
 //   gradient: dloss/dA_{l,d} = 2 sum_{x, colour} g_l(x) (T_d psi_{l-1})(x)^dag: one warp per offset,
-//             FP32 sums over a few sites, FP64 sums over lanes, blocks and pairs in a fixed order
-//             (deterministic).
+//             FP32 sums over a few sites, then sums over lanes, blocks and pairs with FP64's accuracy or
+//             better, in a fixed order (deterministic for a given group of pairs).
 //   loss:     |P b - x|^2 / |x|^2 per pair with the seed g_K = (P b - x) / |x|^2.
 //   Adam:     on the real and imaginary parts of every A entry, in the gradient's final sum.
 // A training step runs every kernel once for a group of its pairs, not once per pair.

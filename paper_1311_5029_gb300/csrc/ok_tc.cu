@@ -296,10 +296,10 @@ struct Lane {
 
 // FP16 input layout (the applied vectors, scaled): per (site, b) a 512-byte tile of 8 pairs x 4
 // colour slots x 16 bytes; the word of pair p and colour c < 3 holds right-hand side p in its
-// first 8 bytes and p + 8 in its last 8 (each: h_b spin 0, h_b spin 1).  Lane (g, t < 3) reads
-// word 4 g + t, both of its rows in one 16-byte load, so a quarter-warp reads 96 bytes of one
-// aligned 128-byte line (one L1 wavefront); the slots c = 3 (the zero K pairs) are never read,
-// and absent right-hand sides are zero.
+// first 8 bytes and p + 8 in its last 8 (each: h_b spin 0, h_b spin 1).  Lane (g, t) reads
+// word 4 g + t, both of its rows in one 16-byte load, so a quarter-warp reads one aligned 128-byte line
+// (one L1 wavefront).  Slot 3 holds the zero K pairs and must be zero: the products of lane t = 3 take it with
+// another lane's W words.  Absent right-hand sides are zero too.
 constexpr int IN16_TILE_U4 = 32;   // 16-byte words per (site, projection) tile
 __host__ __device__ __forceinline__ size_t in16_index(int site, int b, int r, int c) {  // 8-byte units
   return ((((size_t)site * 2 + b) * IN16_TILE_U4) + 4 * (r & 7) + c) * 2 + (r >> 3);
