@@ -6,14 +6,14 @@
 // the half-spinor of a hop PLA steps ahead are requested before step k is computed, so several loads of
 // every warp are always in flight.
 //
-// What bounds it: memory latency (16^3 x 32, FP32: 5.3 warps waiting for loads per issue, issue 36 %, L1 57 %, DRAM 55 %;
-// FP16: 3.8, issue 49 %, L1 45 %, DRAM 35 %).  The requests start anew with every tile and the halves meet at its end, which
-// a pipeline over the tile boundary would avoid (not tried).  More warps with fewer registers take as long or longer.  Left to itself the compiler keeps about one hop's loads in
-// flight once the hops form one basic block (122 us at 16^3 x 32); a __syncwarp between a step's requests and
-// its arithmetic keeps it from sinking the loads to their use.  16^3 x 32 / 28^3 x 96, FP32: 98 / 1735 us
-// with the split kernel before, 92 / 1450 us now; FP16: 86 / 1610 us before, 74 / 1375 us now.  14x18x11x27 and 14^3 x 28
-// in FP32 were 1 to 2 % faster with the split kernel: their 2339 and 2401 tiles fill its four rounds of 608 blocks, and 5.1
-// and 5.3 rounds of this kernel's 456.
+// What bounds it: memory latency (16^3 x 32, FP32: 5.4 warps waiting for loads per issue and 0.2 at the barrier where the
+// halves meet, issue 35 %, L1 57 %, DRAM 56 %; FP16: 3.8 and 0.4, issue 49 %, L1 45 %, DRAM 35 %).  Every tile starts with
+// nothing in flight; requests over the tile boundary have not been tried.  More warps with fewer registers take as long or
+// longer.  Left to itself the compiler keeps about one hop's loads in flight once the hops form one basic block (122 us at
+// 16^3 x 32); a __syncwarp between a step's requests and its arithmetic keeps it from sinking the loads to their use.
+// 16^3 x 32 / 28^3 x 96, FP32: 98 / 1735 us with the split kernel before, 92 / 1450 us now; FP16: 86 / 1610 us before, 74 /
+// 1375 us now.  14x18x11x27 and 14^3 x 28 in FP32 were 1 to 2 % faster with the split kernel: their 2339 and 2401 tiles fill
+// its four rounds of 608 blocks, and 5.1 and 5.3 rounds of this kernel's 456.
 #include "ok_pair.cuh"
 
 namespace okgb {

@@ -110,7 +110,7 @@ template <typename R> __device__ __forceinline__ void mdv(cx<R> (&y)[3], const M
 // ---------------------------------------------------------------------------- geometry
 // Neighbour x + d with fermion boundary sign; |d_mu| <= 2.  The coordinate is wrapped by at most
 // two conditional subtractions (two are needed only when L_mu < |d_mu|, on lattices of extent 1
-// or 2); the sign flips once per wrap across an antiperiodic boundary (AP false: there is none).
+// or 2); the sign flips once per wrap across an antiperiodic boundary (AP false: none that this hop can cross).
 template <int D0, int D1, int D2, int D3, bool AP = true>
 __device__ __forceinline__ int nbr_site(const int (&c)[4], const Geom& g, bool& neg) {
   const int d[4] = {D0, D1, D2, D3};
