@@ -505,15 +505,15 @@ void launch_pipe(const cx<WT>* W, const cx<float>* psi, cx<float>* out, const Ge
     return;
   }
   // The form of the boundaries and the lookahead.  The requests are the same in all forms, but the compiler schedules
-  // each in its own way, and which is the fastest was found by measurement: us, old form / new form, before the slash
-  // the sign of every hop as a multiplication, behind it only the temporal hop's (BC_TIME, for periodic lattices too).
+  // each in its own way, and which is the fastest was found by measurement.  The form, us: before the slash every hop's sign
+  // is a multiplication, behind it only the temporal hop's (BC_TIME, for periodic lattices too).
   //   FP32, time antiperiodic: 14x18x11x27 63.0 / 60.6; 20^3 x 64 350 / 337; 28^3 x 96 1532 / 1445.  Periodic, against the
   //   form without signs: 61.6 / 60.6; 343 / 337; 1461 / 1445.
   //   FP16, time antiperiodic: 14x18x11x27 47.0 / 45.1; 18^3 x 36 126 / 117; 20^3 x 64 296 / 282; 28^3 x 48 663 / 648 and 647 /
   //   660 in two runs.  Periodic: 45.1 / 45.1; 117 / 117; 276 / 282; 24^3 x 64 480 / 506, so there the form without signs stays.
   // LA against the bytes of a time slice of W (us, LA 2 / 3 and 4 / 5; the crossover lies between the two nearest):
   //   FP32 BC_TIME: 9 MB (14^3 x 28) 61.5 / 63.0; 43 MB (24^3 x 64) 578 / 590; 68 MB (28^3 x 48) 797 / 729.
-  //   FP32 BC_ANY the other way round: 43 MB 627 / 593; 68 MB 770 / 755; 28^3 x 96 1533 / 1585.
+  //   FP32 BC_ANY the other way round: 43 MB 627 / 593; 28^3 x 96 (68 MB) 1533 / 1585; against the rule 28^3 x 48 770 / 755.
   //   FP16 BC_NONE: 4.2 MB (14^3 x 28) 46.6 / 45.2, 11x15x9x40 43.3 / 41.7; 6.3 MB (16^3 x 32) 74.1 / 79.4, 12 MB (20^3 x 64)
   //   276 / 305, 34 MB (28^3 x 96) 1349 / 1417; against the rule 10^3 x 20 19.9 / 21.1 and 18^3 x 36 117.1 / 116.1.
   //   FP16 BC_ANY: 4.2 MB 49.2 / 47.2; 6.3 MB 78.9 / 82.3; 12 MB 301 / 331; against the rule 18^3 x 36 125.8 / 121.6.
