@@ -293,7 +293,7 @@ int ok_true_residual(const ok_W* W, const void* b, const void* x, double* relres
  * prec OK_F64 (complex128 fields, OK_W_F64; OK_REDUCE_TS then needs y == psi), OK_F32 (complex64,
  * OK_W_F32) or OK_F32_W16 (complex64, OK_W_F16).  psi, y, out: device [V][4][3]; out must not
  * overlap psi or y; sums: host, 3 doubles.  The partial sums are FP64
- * (FP32 fields: FP32 chunks of a few elements, then double-float) and summed in a fixed order.
+ * (FP32 fields: of FP32 sums over a few elements) and summed in a fixed order.
  * Allocates stream-ordered scratch and synchronises `stream`.
  * Errors: OK_EINVAL (null or misaligned pointers, overlap, a missing copy, an unknown kind),
  * OK_ENOMEM, OK_ECUDA. */

@@ -150,14 +150,14 @@ __global__ void __launch_bounds__(BLAS_THREADS) update_p_kernel(typename Unit<R>
 // The inner products a BiCGStab half-iteration takes from its application of M, in a pass of their
 // own (the FP32 applications run without a fused epilogue; the separate pass over two vectors
 // costs less than the epilogue did): ALPHA: <a, b> (a = rhat, b = v) -> FIN_ALPHA;
-// OMEGA: <a, b>, <a, a> (a = t, b = s) -> FIN_OMEGA.
-template <typename R, bool OMEGA>
+// OMEGA: <a, b>, <a, a> (a = t, b = s) -> FIN_OMEGA.  S: the type of the totals.
+template <typename R, bool OMEGA, typename S = typename RedT<R>::T>
 __global__ void __launch_bounds__(BLAS_THREADS) dots_kernel(const typename Unit<R>::T* __restrict__ a,
                                                             const typename Unit<R>::T* __restrict__ b, long long nu,
                                                             SolverState* __restrict__ st, RedArgs ra, unsigned* ticket) {
   if (st->halt) return;
   using U = Unit<R>;
-  typename RedT<R>::T red[3] = {0, 0, 0};
+  S red[3] = {0, 0, 0};
   OK_CHUNK_STRIDE(i0, nu) {
     cx<R> d = mk<R>(0, 0);
     R n2 = 0;
@@ -175,12 +175,12 @@ __global__ void __launch_bounds__(BLAS_THREADS) dots_kernel(const typename Unit<
     red_add(red[1], d.im);
     red_add(red[2], n2);
   }
-  if (OMEGA) {
-    grid_reduce_r<R, 3>(red, ra, ticket);
-  } else {
-    typename RedT<R>::T v2[2] = {red[0], red[1]};
-    grid_reduce_r<R, 2>(v2, ra, ticket);
-  }
+  constexpr int NP = OMEGA ? 3 : 2;
+  S v[NP];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) v[k] = red[k];
+  if constexpr (std::is_same<S, double>::value) grid_reduce<NP, BLAS_THREADS>(v, ra, ticket);
+  else grid_reduce_dd<NP, BLAS_THREADS>(v, ra, ticket);
 }
 
 // ---------------------------------------------------------------------------- small systems
@@ -604,10 +604,10 @@ int launch_update_xr(cx<R>* x, const cx<R>* p, const cx<R>* s, const cx<R>* t, c
 }
 
 template <typename R>
-int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm, int fin) {
+int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm) {
   using T = typename Unit<R>::T;
   long long nu = units_of<R>(n);
-  RedArgs ra{st, part, nullptr, fin >= 0 ? fin : omega ? FIN_OMEGA : FIN_ALPHA};
+  RedArgs ra{st, part, nullptr, omega ? FIN_OMEGA : FIN_ALPHA};
   {
     TraceScope ts(omega ? (sizeof(R) == 8 ? "dots_ts_f64" : "dots_ts_f32") : (sizeof(R) == 8 ? "dot_rv_f64" : "dot_rv_f32"), strm);
     if (omega)
@@ -616,6 +616,18 @@ int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverS
     else
       dots_kernel<R, false><<<wave_blocks(dots_kernel<R, false>, nu, true), BLAS_THREADS, 0, strm>>>((const T*)a, (const T*)b, nu, st, ra,
                                                                                             &st->ticket[0]);
+  }
+  OK_LAUNCH_CHECK();
+  return OK_SUCCESS;
+}
+
+int launch_sums(const cx<float>* a, const cx<float>* b, long long n, bool norm, SolverState* st, double* part, cudaStream_t strm) {
+  const long long nu = units_of<float>(n);
+  const RedArgs ra{st, part, nullptr, FIN_NONE};
+  auto kern = norm ? dots_kernel<float, true, double> : dots_kernel<float, false, double>;
+  {
+    TraceScope ts("sums_f32", strm);
+    kern<<<wave_blocks(kern, nu, true), BLAS_THREADS, 0, strm>>>((const float4*)a, (const float4*)b, nu, st, ra, &st->ticket[0]);
   }
   OK_LAUNCH_CHECK();
   return OK_SUCCESS;
@@ -730,8 +742,8 @@ int launch_norms(const cx<double>* x, const cx<double>* b, long long n, SolverSt
 
 template int launch_update_s<double>(const cx<double>*, const cx<double>*, cx<double>*, long long, const SolverState*, cudaStream_t);
 template int launch_update_s<float>(const cx<float>*, const cx<float>*, cx<float>*, long long, const SolverState*, cudaStream_t);
-template int launch_dots<float>(const cx<float>*, const cx<float>*, long long, bool, SolverState*, double*, cudaStream_t, int);
-template int launch_dots<double>(const cx<double>*, const cx<double>*, long long, bool, SolverState*, double*, cudaStream_t, int);
+template int launch_dots<float>(const cx<float>*, const cx<float>*, long long, bool, SolverState*, double*, cudaStream_t);
+template int launch_dots<double>(const cx<double>*, const cx<double>*, long long, bool, SolverState*, double*, cudaStream_t);
 template int launch_update_xr<double>(cx<double>*, const cx<double>*, const cx<double>*, const cx<double>*, cx<double>*, const cx<double>*, long long, SolverState*, double*, cudaStream_t, const cx<double>*);
 template int launch_update_xr<float>(cx<float>*, const cx<float>*, const cx<float>*, const cx<float>*, cx<float>*, const cx<float>*, long long, SolverState*, double*, cudaStream_t, const cx<float>*);
 template int launch_update_p<double>(cx<double>*, const cx<double>*, const cx<double>*, long long, const SolverState*, cudaStream_t);

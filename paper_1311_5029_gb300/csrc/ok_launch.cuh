@@ -97,11 +97,12 @@ int launch_update_xr(cx<R>* x, const cx<R>* p, const cx<R>* s, const cx<R>* t, c
                      SolverState* st, double* part, cudaStream_t strm, const cx<R>* sx = nullptr);
 template <typename R>
 int launch_update_p(cx<R>* p, const cx<R>* r, const cx<R>* v, long long n, const SolverState* st, cudaStream_t strm);
-// <a, b> -> FIN_ALPHA (a = rhat, b = v), or with omega <a, b>, <a, a> -> FIN_OMEGA (a = t, b = s); fin >= 0:
-// that finalisation instead.
+// <a, b> -> FIN_ALPHA (a = rhat, b = v), or with omega <a, b>, <a, a> -> FIN_OMEGA (a = t, b = s).
 template <typename R>
-int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm,
-                int fin = -1);
+int launch_dots(const cx<R>* a, const cx<R>* b, long long n, bool omega, SolverState* st, double* part, cudaStream_t strm);
+// <a, b>, and with norm <a, a>, into the state's aux: FP32 sums over chunks as launch_dots takes them, the totals in FP64, whose
+// range the totals of a field of large values need (in pairs of floats they end at 3.4e38).
+int launch_sums(const cx<float>* a, const cx<float>* b, long long n, bool norm, SolverState* st, double* part, cudaStream_t strm);
 // The work between two applications in one cluster launch each, for systems of few elements: the inner
 // product, alpha and s = r - alpha v; omega, x, r, beta and p.
 bool small_system(long long n);

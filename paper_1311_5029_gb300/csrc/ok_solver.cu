@@ -396,13 +396,12 @@ int apply_reduce(const ok_W* W, ok_prec prec, int kind, const void* psi, const v
     EpiArgs<double> e{(const cx<double>*)y, nullptr, ra, &dst->ticket[0], nullptr};
     OK_TRY(launch_apply<double>(W, (const cx<double>*)psi, (cx<double>*)out, epi, e, st));
   } else {
-    // as the FP32 iteration runs it: the plain application, then its inner products
+    // as the FP32 iteration runs it, the plain application and then its inner products, but for the totals' type
     const EpiArgs<float> e{};
     if (prec == OK_F32) OK_TRY(launch_apply<float>(W, (const cx<float>*)psi, (cx<float>*)out, EPI_NONE, e, st));
     else OK_TRY(launch_apply_w16(W, (const cx<float>*)psi, (cx<float>*)out, EPI_NONE, e, st));
     const bool ts = kind == 2;  // <out, y>, <out, out>, else <y, out>
-    OK_TRY(launch_dots<float>((const cx<float>*)(ts ? out : y), (const cx<float>*)(ts ? y : out), 12LL * W->g.V, ts, dst, part, st,
-                              FIN_NONE));
+    OK_TRY(launch_sums((const cx<float>*)(ts ? out : y), (const cx<float>*)(ts ? y : out), 12LL * W->g.V, ts, dst, part, st));
   }
   OK_TRY(read_state(dst, hs.h, st));
   for (int k = 0; k < 3; ++k) sums[k] = kind == 1 && k == 2 ? 0.0 : hs.h->aux[k];
